@@ -479,7 +479,8 @@ int eogp_score_workspace_size(int N, const int* k_per_module, int U, int mode, i
  * scores [Q x ld_scores] fp32 device, ld_scores >= N.
  * ws: 256-byte aligned device workspace of at least eogp_score_workspace_size
  * bytes (0 bytes for the CUDA-core kernels); CODES and PAPER use the tensor
- * cores when it is given, the shape allows (CODES: Q >= 64, k_u % 128 == 0;
+ * cores when it is given, the shape allows (CODES: k_u % 128 == 0 and Q >= 17,
+ * or Q >= 9 with every k_u % 256 == 0, or Q >= 5 when those sum to 4096 or more;
  * PAPER: k_u % 64 == 0) and the code rows are aligned (CODES: ld_train % 4 == 0
  * and a 16-byte aligned base; PAPER: ld_train % 2 == 0, 8-byte base). CODES on
  * the tensor cores multiplies exact +-1 operands: e2m1 through the block-scaled

@@ -1372,8 +1372,10 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
   const bool tc_ok = (mode == EOGP_SCORE_CODES || mode == EOGP_SCORE_PAPER) &&
                      score_tc_supported(mode, ks, U, Q);
   const int force = topk_fused_override();
+  // Fewer than 64 one-bit queries keep the dense path, whose scores any row
+  // alignment can have (the fused kernel's rows need the tensor cores').
   p.fused = tc_ok && score_tc_topk_fits(mode, ks, U, Q, K) && force != 0 &&
-            (force == 1 || N > topk_select_max_n());
+            (mode != EOGP_SCORE_CODES || Q >= 64) && (force == 1 || N > topk_select_max_n());
   p.select = !p.fused && N <= topk_select_max_n();
   p.q_bytes = tc_ok ? score_tc_ws_bytes(mode, ks, U, Q) : 0;
   if (p.fused) {

@@ -10,11 +10,16 @@
 // PAPER mode (query unquantised): sum_u s_iu <y_u, b_iu> with b in {+-1}.
 //
 // Kernels:
-//  k_score_codes_smallq<QT>: Q <= 8 queries; one thread per stored row, query
-//    words broadcast from shared memory; stored codes staged through shared
-//    memory with coalesced 128-byte row loads. This is the HBM-bound scan.
-//  k_score_codes_tiled: 64 stored rows x 64 queries per block, 4 x 4 per thread.
+//  k_score_codes_smallq<QT>: QT <= 8 queries a pass; one thread per stored row,
+//    query words broadcast from shared memory; stored codes staged through shared
+//    memory with coalesced 128-byte row loads. Up to two queries this is the
+//    HBM-bound scan, at eight it is bound by the popcounts (0.86 of their measured
+//    rate).
+//  k_score_codes_tiled: 64 stored rows x 64 queries per block, 4 x 4 per thread,
+//    for many queries against short modules or unaligned rows.
 //  k_score_paper_tiled: same tiling, one 32-coordinate word per step.
+#include <algorithm>
+
 #include "eogp_dev.cuh"
 #include "eogp_internal.h"
 
@@ -323,21 +328,33 @@ cudaError_t launch_score_codes(const uint32_t* train, int ldt, const float* ts, 
   ModInfo local;  // passed by value: kernel parameters are copied at launch
   if (!fill_modinfo(local, ks, U)) return cudaErrorInvalidValue;
   if (N <= 0 || Q <= 0) return cudaSuccess;
-  if (Q <= 8) {
-    const int qt = Q <= 1 ? 1 : Q <= 2 ? 2 : Q <= 4 ? 4 : 8;
-    dim3 grid((N + 255) / 256, (Q + qt - 1) / qt);
-    int vec = ((ldt & 3) == 0) && ((reinterpret_cast<uintptr_t>(train) & 15) == 0);
-    for (int u = 0; u < U; ++u) vec &= (((ks[u] + 31) / 32) % 4) == 0;
+  int vec = ((ldt & 3) == 0) && ((reinterpret_cast<uintptr_t>(train) & 15) == 0);
+  for (int u = 0; u < U; ++u) vec &= (((ks[u] + 31) / 32) % 4) == 0;
+  // Passes of 8 queries that cost no more than one 64-query tile (measured, one
+  // pass against one tile: 200K rows of 4096 bits 51 / 438 us, of 7 x 640 bits
+  // 67 / 560; with rows the vector loads cannot take 77 / 455; modules of a few
+  // words fill a fraction of a staged chunk: 200K rows of 3 x 96 bits 23 / 83).
+  const long long passes = (Q + 7) / 8, tiles = (Q + 63) / 64;
+  const int per_tile = local.off[U] < 16 * U ? 3 : vec ? 8 : 5;
+  if (passes > 1 && passes > per_tile * tiles) {
+    const dim3 grid((N + 63) / 64, static_cast<unsigned>(tiles));
+    k_score_codes_tiled<<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, query, ldq, qs, ldqs, Q, out, ldo);
+    return cudaGetLastError();
+  }
+  const int qt = Q <= 1 ? 1 : Q <= 2 ? 2 : Q <= 4 ? 4 : 8;
+  constexpr int kMaxPasses = 65535;  // grid.y
+  for (int q0 = 0; q0 < Q; q0 += kMaxPasses * 8) {
+    const int nq = std::min(Q - q0, kMaxPasses * 8);
+    const dim3 grid((N + 255) / 256, (nq + qt - 1) / qt);
+    const uint32_t* qc = query + static_cast<size_t>(q0) * ldq;
+    const float* qsc = qs + static_cast<size_t>(q0) * ldqs;
+    float* o = out + static_cast<size_t>(q0) * ldo;
     switch (qt) {
-      case 1: k_score_codes_smallq<1><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, query, ldq, qs, ldqs, Q, out, ldo, vec); break;
-      case 2: k_score_codes_smallq<2><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, query, ldq, qs, ldqs, Q, out, ldo, vec); break;
-      case 4: k_score_codes_smallq<4><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, query, ldq, qs, ldqs, Q, out, ldo, vec); break;
-      default: k_score_codes_smallq<8><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, query, ldq, qs, ldqs, Q, out, ldo, vec); break;
+      case 1: k_score_codes_smallq<1><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, qc, ldq, qsc, ldqs, nq, o, ldo, vec); break;
+      case 2: k_score_codes_smallq<2><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, qc, ldq, qsc, ldqs, nq, o, ldo, vec); break;
+      case 4: k_score_codes_smallq<4><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, qc, ldq, qsc, ldqs, nq, o, ldo, vec); break;
+      default: k_score_codes_smallq<8><<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, qc, ldq, qsc, ldqs, nq, o, ldo, vec); break;
     }
-  } else {
-    dim3 grid((N + 63) / 64, (Q + 63) / 64);
-    k_score_codes_tiled<<<grid, 256, 0, st>>>(train, ldt, ts, ldts, N, local, query, ldq, qs, ldqs,
-                                              Q, out, ldo);
   }
   return cudaGetLastError();
 }

@@ -573,15 +573,29 @@ cudaError_t dispatch_tc(int mode, const TcCfg& c, const CUtensorMap& t0, const C
   return launch_tc_kernel<EOGP_SCORE_CODES, TOPK, 128, true>(t0, t1, g, grid, st);
 }
 
+// Fewest one-bit queries the tensor cores take. Their time does not depend on
+// the queries up to 64 (the expansion of the stored rows sets it), the popcount
+// kernel's is one pass of 8 queries after another, so the line lies where the
+// two cross. Measured, popcount then tensor cores: 1M rows of 16,384 bits
+// 575 / 614 us at 4 queries, 955 / 615 at 6 (7,890 / 615 at 20 against the 64 x
+// 64 popcount tiles); 300K rows of 48 x 1024 bits 564 / 787 at 4, 990 / 788 at 6. Rows of less than 4096 bits
+// pay for a tile's drain: 1M rows of 1024 bits 69 / 123 at 8, two passes 138 /
+// 124 at 9. The e4m3 operands (modules not a multiple of 256 bits) are
+// expanded twice as wide: 1M rows of 7 x 640 bits 668 / 720 at 16, 1,002 / 721
+// at 17.
+int codes_min_queries(bool f4, long long bits) { return !f4 ? 17 : bits >= 4096 ? 5 : 9; }
+
 }  // namespace
 
 bool score_tc_supported(int mode, const int* ks, int U, int Q) {
   if (U < 1 || U > kMaxMods || Q < 1 || Q > 65535) return false;
   if (mode == EOGP_SCORE_CODES) {
-    if (Q < 64) return false;  // the popcount kernels are faster for a handful of queries
-    for (int u = 0; u < U; ++u)
+    long long D = 0;
+    for (int u = 0; u < U; ++u) {
       if (ks[u] <= 0 || ks[u] % 128) return false;
-    return true;
+      D += ks[u];
+    }
+    return Q >= codes_min_queries(tc_f4(mode, ks, U), D);
   }
   if (mode == EOGP_SCORE_PAPER) {
     for (int u = 0; u < U; ++u)
