@@ -106,9 +106,11 @@ int eogp_profile_read(int kind, int* launches, double* total_ms, int reset);
  *     kernel. 0 (default): e2m1 (kind::mxf4, unit scales) when every module is
  *     a multiple of 256 bits and the stored rows are 16-byte aligned, else
  *     e4m3; 1: always e4m3 (kind::f8f6f4). Scores are bit-identical.
- *   EOGP_OPT_TOPK_PATH: ranking path of eogp_score_topk. 0 (default): chosen
- *     by size; 1: ranking fused into the tensor-core scoring kernel where it
- *     applies; 2: dense scores then a ranking kernel.
+ *   EOGP_OPT_TOPK_PATH: ranking path of eogp_score_topk. 0 (default) and 2: dense
+ *     scores, up to 1 GiB of them at a time, then a ranking kernel; 1: ranking
+ *     fused into the tensor-core scoring kernel where it applies (slower, but a
+ *     workspace of tens of MB). With 0, requests the fused kernel could take are
+ *     refused beyond 49,152 rows that are not aligned for it.
  * eogp_set_option returns EOGP_EINVAL for an unknown option or value. */
 #define EOGP_OPT_SCORE_OPERAND 0
 #define EOGP_OPT_TOPK_PATH     1
@@ -523,10 +525,10 @@ int eogp_score_topk_workspace_size(int N, const int* k_per_module, int U, int mo
                                    int topk, size_t* bytes);
 
 /* Per query, the `topk` best stored rows under the eogp_score definition of
- * `mode`, without materialising the Q x N scores when the tensor-core kernels
- * apply and topk <= 64 (the ranking then runs in their epilogue; the Q x N
- * matrix is never written). Otherwise the scores go to the workspace and a
- * ranking kernel follows. Arguments as eogp_score, plus:
+ * `mode`. The scores of as many stored rows as fit 1 GiB of workspace are formed
+ * and ranked at a time; with EOGP_OPT_TOPK_PATH = 1, where the tensor-core
+ * kernels apply and topk <= 32, the ranking runs in their epilogue instead, with
+ * no scores written and a workspace of tens of MB. Arguments as eogp_score, plus:
  *   top_scores [Q x ld_top_scores] fp32 device and top_index [Q x ld_top_index]
  *   int32 device (stored row numbers), ld >= topk: row q lists its best rows by
  *   score descending, equal scores by lower row number; NaN scores never rank;

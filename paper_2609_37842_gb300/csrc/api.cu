@@ -1350,18 +1350,29 @@ extern "C" int eogp_score(const void* train, int ld_train, const float* train_sc
 // Workspace plan of eogp_score_topk: fused (tensor-core scoring with the ranking in
 // its epilogue) or dense (scores into the workspace, then a ranking kernel).
 struct TopkPlan {
-  bool fused, select;
-  int slots;
+  bool fused;
+  bool tc_rows;  // refused unless the code rows are aligned for the tensor cores
+  int slots;     // fused: per-CTA lists
+  int slice, rows;       // dense: stored rows ranked per block, and scored at a time (a multiple of slice)
+  long long n1, n2;      // dense: list entries per query of the first level, and of the second (0: none)
   size_t q_bytes, dense_bytes, list_bytes, buf_bytes, scr_bytes, total;
 };
 
-// Paths: up to topk_select_max_n() stored rows, dense scores (tensor cores
-// where they apply) and a radix select per query row (k_topk_select); beyond,
-// the ranking is fused into the tensor-core scoring kernel when it supports the
-// request (the Q x N matrix then never reaches HBM), else dense scores, per-slot
-// lists and a merge. Measured on the GPT-2 query workload (N = 16384, Q = 1024,
-// top 20): fused 2.4 ms, dense + per-slot lists 2.9 ms. EOGP_OPT_TOPK_PATH = 1 / 2
-// forces the fused / a dense path.
+// Paths. Dense: scores (tensor cores where they apply) of as many stored rows as
+// 1 GiB of workspace holds, ranked slice by slice by k_topk_select, and so on
+// over the rows; then the slices' lists are ranked. Fused: the ranking in the
+// tensor-core kernel's epilogue, no scores in memory; there it holds up the MMAs
+// while the lists fill. Measured, top 20, fused / dense in us: 64 queries over
+// 300K rows of 16,384 bits 657 / 258, 1024 queries 3,756 / 1,853, 1024 over
+// 2M rows 12,236 / 11,984; 64 over 20,000 rows of 48 x 1024 bits 378 / 148. So the
+// dense path is the default; EOGP_OPT_TOPK_PATH = 1 selects the fused one where it
+// applies.
+constexpr size_t kTopkDenseMax = size_t(1) << 30;
+// Stored rows up to which any row alignment is ranked; more of them in a request
+// the fused path supports need the alignment of the tensor cores on every path.
+constexpr int kTopkAnyRowsMaxN = 49152;
+constexpr int kTopkListSlice = 16384;  // list entries ranked per block
+
 static int topk_fused_override() {
   const int v = option(EOGP_OPT_TOPK_PATH);
   return v == 1 ? 1 : v == 2 ? 0 : -1;
@@ -1372,22 +1383,29 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
   const bool tc_ok = (mode == EOGP_SCORE_CODES || mode == EOGP_SCORE_PAPER) &&
                      score_tc_supported(mode, ks, U, Q);
   const int force = topk_fused_override();
-  // Fewer than 64 one-bit queries keep the dense path, whose scores any row
-  // alignment can have (the fused kernel's rows need the tensor cores').
-  p.fused = tc_ok && score_tc_topk_fits(mode, ks, U, Q, K) && force != 0 &&
-            (mode != EOGP_SCORE_CODES || Q >= 64) && (force == 1 || N > topk_select_max_n());
-  p.select = !p.fused && N <= topk_select_max_n();
+  // Fewer than 64 one-bit queries are always scored dense, which any row
+  // alignment allows.
+  const bool can = tc_ok && score_tc_topk_fits(mode, ks, U, Q, K) && force != 0 &&
+                   (mode != EOGP_SCORE_CODES || Q >= 64);
+  p.fused = can && force == 1;
+  p.tc_rows = can && (force == 1 || N > kTopkAnyRowsMaxN);
   p.q_bytes = tc_ok ? score_tc_ws_bytes(mode, ks, U, Q) : 0;
   if (p.fused) {
     p.slots = score_tc_grid(mode, ks, U, N, Q, K, sm_count());
-    p.dense_bytes = 0;
+    p.list_bytes = al256(static_cast<size_t>(p.slots) * Q * K * 4);
+    p.buf_bytes = al256(score_tc_list_buf_bytes(mode, ks, U, Q, K, p.slots));
+    p.scr_bytes = al256(score_tc_scratch_bytes(mode, ks, U, Q, K, p.slots));
   } else {
-    p.slots = p.select ? 0 : topk_dense_slots(N);
-    p.dense_bytes = al256(static_cast<size_t>(Q) * ((static_cast<size_t>(N) + 3) & ~size_t(3)) * 4);
+    p.slice = topk_slice(N, Q);
+    const long long fit = static_cast<long long>(kTopkDenseMax / (4 * static_cast<size_t>(std::max(Q, 1))));
+    p.rows = N <= fit ? std::max(N, 1) : static_cast<int>(std::max<long long>(1, fit / p.slice) * p.slice);
+    p.dense_bytes = al256(static_cast<size_t>(Q) * ((static_cast<size_t>(std::min(p.rows, N)) + 3) & ~size_t(3)) * 4);
+    const long long slots = (static_cast<long long>(N) + p.slice - 1) / p.slice;
+    p.n1 = slots > 1 ? slots * K : 0;
+    p.n2 = p.n1 > kTopkListSlice ? (p.n1 + kTopkListSlice - 1) / kTopkListSlice * K : 0;
+    p.list_bytes = al256(static_cast<size_t>(Q) * ((p.n1 + 3) & ~3ll) * 4) +
+                   al256(static_cast<size_t>(Q) * ((p.n2 + 3) & ~3ll) * 4);
   }
-  p.list_bytes = al256(static_cast<size_t>(p.slots) * Q * K * 4);
-  p.buf_bytes = p.fused ? al256(score_tc_list_buf_bytes(mode, ks, U, Q, K, p.slots)) : 0;
-  p.scr_bytes = p.fused ? al256(score_tc_scratch_bytes(mode, ks, U, Q, K, p.slots)) : 0;
   p.total = al256(p.q_bytes) + p.dense_bytes + 2 * p.list_bytes + 2 * p.buf_bytes +
             (p.fused ? al256(static_cast<size_t>(Q) * 4) : 0) + p.scr_bytes;
   return p;
@@ -1439,7 +1457,7 @@ extern "C" int eogp_score_topk(const void* train, int ld_train, const float* tra
                                         2 * p.buf_bytes + al256(static_cast<size_t>(Q) * 4));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   ProfScope ps(EOGP_K_SCORE, st);
-  if (p.fused && N > 0) {
+  if (p.tc_rows && N > 0) {
     if (!train_scales || (mode == EOGP_SCORE_CODES && !query_scales))
       return set_error(EOGP_EINVAL, "scales are NULL");
     if (ld_train < W || ld_tscale < U ||
@@ -1449,6 +1467,8 @@ extern "C" int eogp_score_topk(const void* train, int ld_train, const float* tra
       return set_error(EOGP_EUNSUPPORTED, mode == EOGP_SCORE_CODES
                                               ? "fused top-K needs 16-byte aligned code rows (ld_train % 4 == 0)"
                                               : "fused top-K needs 8-byte aligned code rows (ld_train % 2 == 0)");
+  }
+  if (p.fused && N > 0) {
     unsigned* status = status_word();
     if (!status) return set_error(EOGP_ECUDA, "device status word unavailable");
     TcTopK tk{topk, lst, lsi, bufs, bufi, gtau, scr, top_scores, ld_top_scores, top_index, ld_top_index};
@@ -1457,18 +1477,43 @@ extern "C" int eogp_score_topk(const void* train, int ld_train, const float* tra
                              0, &tk, qws, sm_count(), status, st));
     return EOGP_OK;
   }
-  const int ldd = (N + 3) & ~3;
-  if (N > 0) {
-    const int rc = score_dense(train, ld_train, train_scales, ld_tscale, N, k_per_module, U, mode, query,
-                               ld_query, query_scales, ld_qscale, Q, dense, ldd, qws, p.q_bytes, W, D, st);
-    if (rc != EOGP_OK) return rc;
+  // Dense: chunks of p.rows stored rows scored and ranked slice by slice.
+  const int ldd = (std::min(p.rows, N) + 3) & ~3;
+  const size_t ld1 = static_cast<size_t>((p.n1 + 3) & ~3ll), ld2 = static_cast<size_t>((p.n2 + 3) & ~3ll);
+  const size_t l1 = al256(static_cast<size_t>(Q) * ld1 * 4);  // bytes of a first-level list array
+  float* s1 = lst;
+  int* i1 = lsi;
+  float* s2 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(lst) + l1);
+  int* i2 = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(lsi) + l1);
+  const size_t esz = 4;  // code words and fp32 coordinates alike
+  for (long long r0 = 0; r0 < std::max(N, 1); r0 += p.rows) {
+    const int r = static_cast<int>(r0), nr = std::min(p.rows, N - r);
+    if (nr > 0) {
+      const int rc = score_dense(static_cast<const uint8_t*>(train) + static_cast<size_t>(r) * ld_train * esz, ld_train,
+                                 train_scales ? train_scales + static_cast<size_t>(r) * ld_tscale : nullptr, ld_tscale,
+                                 nr, k_per_module, U, mode, query, ld_query, query_scales, ld_qscale, Q, dense, ldd,
+                                 qws, p.q_bytes, W, D, st);
+      if (rc != EOGP_OK) return rc;
+    }
+    const size_t at = static_cast<size_t>(r / p.slice) * topk;  // the chunk's first list entry
+    if (p.n1 == 0)
+      CUDA_TRY(launch_topk_select(dense, nullptr, ldd, Q, nr, r, topk, p.slice, false, top_scores, ld_top_scores,
+                                  top_index, ld_top_index, st));
+    else
+      CUDA_TRY(launch_topk_select(dense, nullptr, ldd, Q, nr, r, topk, p.slice, true, s1 + at, ld1, i1 + at, ld1, st));
   }
-  if (p.select) {
-    CUDA_TRY(launch_topk_select(dense, ldd, Q, N, topk, top_scores, ld_top_scores, top_index, ld_top_index, st));
-    return EOGP_OK;
+  // The lists, as rows of scores, until one slice holds what is left of a query.
+  long long n = p.n1;
+  size_t ld = ld1, ldo = ld2;
+  while (n > kTopkListSlice) {
+    CUDA_TRY(launch_topk_select(s1, i1, ld, Q, static_cast<int>(n), 0, topk, kTopkListSlice, true, s2, ldo, i2, ldo, st));
+    n = (n + kTopkListSlice - 1) / kTopkListSlice * topk;
+    std::swap(s1, s2);
+    std::swap(i1, i2);
+    std::swap(ld, ldo);
   }
-  CUDA_TRY(launch_topk_dense(dense, ldd, Q, N, topk, lst, lsi, st));
-  CUDA_TRY(launch_topk_merge(lst, lsi, topk_dense_slots(N), Q, topk, top_scores, ld_top_scores, top_index,
-                             ld_top_index, st));
+  if (n > 0)
+    CUDA_TRY(launch_topk_select(s1, i1, ld, Q, static_cast<int>(n), 0, topk, kTopkListSlice, false, top_scores,
+                                ld_top_scores, top_index, ld_top_index, st));
   return EOGP_OK;
 }

@@ -3,22 +3,26 @@
 // Order: score descending, equal scores by lower stored index; NaN scores
 // never rank; missing places are (-inf, -1).
 //
-// Three kernels:
-// * k_topk_select ranks one row of a dense [Q, N] score matrix per block when
-//   the row fits in shared memory (N <= kSelectMaxN): the K-th largest score
-//   is found exactly as the largest order-preserving 32-bit key t with at
-//   least K keys >= t, built bit by bit from the top (block-wide counting
-//   passes over the row held in shared memory, no atomics); the K winners are
-//   gathered (the equal-to-threshold ones in index order, so the lowest indices
-//   win ties) and sorted.
-// * k_topk_dense ranks a dense [Q, N] score matrix: block (slot s, query tile)
-//   owns stored rows [s R, (s+1) R) of 32 queries; 128-row chunks are staged
-//   transposed in shared memory and the warp offers each query's column to
-//   that query's list.
-// * k_topk_merge merges per-slot lists [S][Q][K] (written by k_topk_dense or by
-//   the fused tensor-core scoring epilogue) into the final [Q, K]. Every slot
-//   list is sorted, so the largest K-th entry over the slots is a lower bound
-//   on the final K-th entry; only candidates at or above it are sorted.
+// Two kernels:
+// * k_topk_select ranks one slice (at most 16,384 values) of one row of scores per
+//   block. The block holds the slice as order keys in registers (32 a thread,
+//   16-byte loads) and reads it once: the K-th largest of the 512 threads' own
+//   maxima is a lower bound on the slice's K-th score, so the keys at or above it
+//   hold the answer and are few (about K of them for scores in no particular
+//   order); they are collected in shared memory and each finds its own rank among
+//   them by comparison. Should they not fit (scores sorted so that few threads
+//   hold all the best, or many equal ones), the exact K-th largest (score, place)
+//   is built bit by bit from the top by counting. Rows of several slices are
+//   ranked by the same kernel over the slices' lists, laid out as shorter rows.
+//   Bound by reading the scores and the block's 22 barriers. Ranking the GPT-2
+//   queries' 1024 x 16,384 scores (67 MB), top 20, takes the whole call from 583 to
+//   467 us (counting 33 times over keys in shared memory alone took 147); 200
+//   queries over 400,000 rows rank in 144 us, where one list per warp and a merge
+//   took over 300 for 8 queries.
+// * k_topk_merge merges the per-CTA lists [S][Q][K] of the fused tensor-core
+//   scoring epilogue into the final [Q, K]. Every list is sorted, so the largest
+//   K-th entry over the lists is a lower bound on the final K-th entry; only
+//   candidates at or above it are sorted.
 #include <algorithm>
 #include <cmath>
 
@@ -27,11 +31,7 @@
 
 namespace {
 
-constexpr int kChunk = 128;
-constexpr int kTs = kChunk + 1;  // staged row stride (floats)
-constexpr int kMaxSlots = 512;
 constexpr int kMergeCap = 4096;  // keys sorted at once by the merge
-constexpr int kSelectMaxN = 49152;  // rows k_topk_select holds in shared memory (192 KB)
 
 // Order-preserving 64-bit key: larger key = larger score, then lower index
 // (-0 and +0 are the same score).
@@ -50,54 +50,12 @@ __device__ __forceinline__ int key_index(unsigned long long key) {
   return static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(key));
 }
 
-template <int E>
-__global__ void __launch_bounds__(32) k_topk_dense(const float* __restrict__ sc, int ld, int Q, int N,
-                                                   int K, int rows_per_slot, float* __restrict__ lst,
-                                                   int* __restrict__ lsi) {
-  constexpr int kCap = 32 * E;
-  extern __shared__ float sm[];
-  float* tb = sm;                                     // [32 queries][kTs]
-  float* ls = sm + 32 * kTs;                          // [32][kCap]
-  int* li = reinterpret_cast<int*>(ls + 32 * kCap);   // [32][kCap]
-  int* cnt = li + 32 * kCap;                          // [32]
-  float* tau = reinterpret_cast<float*>(cnt + 32);    // [32]
-  const int lane = threadIdx.x;
-  const int slot = blockIdx.x, q0 = blockIdx.y * 32;
-  const int nq = min(32, Q - q0);
-  const int r_beg = slot * rows_per_slot, r_end = min(N, r_beg + rows_per_slot);
-  const bool vec = (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(sc) & 15) == 0;
-  auto list_of = [&](int j) {
-    return eogp::WarpTopk{ls + static_cast<size_t>(j) * kCap, li + static_cast<size_t>(j) * kCap, cnt + j, tau + j,
-                          K, nullptr};
-  };
-  for (int j = 0; j < nq; ++j) eogp::topk_warp_reset(list_of(j), lane);
-  for (int r0 = r_beg; r0 < r_end; r0 += kChunk) {
-    const int nr = min(kChunk, r_end - r0);
-    for (int j = 0; j < nq; ++j) {
-      const float* src = sc + static_cast<size_t>(q0 + j) * ld + r0;
-      if (vec && nr == kChunk) {
-        const float4 v = __ldcs(reinterpret_cast<const float4*>(src) + lane);
-        float* d = tb + j * kTs + 4 * lane;
-        d[0] = v.x;
-        d[1] = v.y;
-        d[2] = v.z;
-        d[3] = v.w;
-      } else {
-        for (int c = lane; c < nr; c += 32) tb[j * kTs + c] = src[c];
-      }
-    }
-    __syncwarp();
-    for (int j = 0; j < nq; ++j) eogp::topk_warp_offer<E>(tb + j * kTs, nr, r0, list_of(j), lane);
-    __syncwarp();
-  }
-  for (int j = 0; j < nq; ++j) {
-    const size_t o = (static_cast<size_t>(slot) * Q + q0 + j) * K;
-    eogp::topk_warp_write<E>(list_of(j), lane, lst + o, lsi + o);
-  }
-}
-
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelVecs = 8;  // 16-byte loads a thread
+constexpr int kSelSlice = 4 * kSelVecs * kSelThreads;  // stored rows a block ranks
+constexpr int kSelCand = 1024;  // candidates collected in shared memory
+static_assert(EOGP_TOPK_MAX <= kSelThreads, "the bound is the K-th of one maximum a thread");
 
 // 32-bit order key of a score: larger score, larger key; -0 and +0 equal; NaN
 // maps to 0, below every score (no non-NaN float maps to 0).
@@ -107,12 +65,9 @@ __device__ __forceinline__ uint32_t sel_key(float s) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-// Number of keys of this block's row that are >= t (block-uniform result).
-// red is double-buffered by `parity` so consecutive calls need one barrier.
-__device__ __forceinline__ uint32_t count_ge(const uint32_t* skey, int N, uint32_t t, uint32_t* red,
-                                             int parity) {
-  uint32_t c = 0;
-  for (int i = threadIdx.x; i < N; i += kSelThreads) c += skey[i] >= t ? 1u : 0u;
+// Sum over the block (block-uniform). red is double-buffered by `parity` so that
+// consecutive calls need one barrier each.
+__device__ __forceinline__ uint32_t block_sum(uint32_t c, uint32_t* red, int parity) {
   c = __reduce_add_sync(0xffffffffu, c);
   if ((threadIdx.x & 31) == 0) red[parity * kSelWarps + (threadIdx.x >> 5)] = c;
   __syncthreads();
@@ -122,93 +77,112 @@ __device__ __forceinline__ uint32_t count_ge(const uint32_t* skey, int N, uint32
   return tot;
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_topk_select(const float* __restrict__ sc, int ld, int N,
-                                                             int K, float* __restrict__ out_s, int ld_os,
-                                                             int* __restrict__ out_i, int ld_oi) {
-  extern __shared__ uint32_t skey[];  // [N] keys of this query's row
+// Block b ranks slice b % S (values [slice s, slice (s + 1)) ) of row b / S into K
+// places at K s + ld q of the outputs. A value's stored row is map[its place in
+// the row] (a list of an earlier level), or without a map its place + row0.
+// Missing places are (-inf, -1), in lists for a further level (`mid`) (NaN, -1).
+__global__ void __launch_bounds__(kSelThreads, 2)
+    k_topk_select(const float* __restrict__ sc, const int* __restrict__ map, size_t ld, int N, int row0, int K, int S,
+                  int slice, int mid, float* __restrict__ out_s, size_t ld_os, int* __restrict__ out_i, size_t ld_oi) {
   __shared__ uint32_t red[2 * kSelWarps];
-  __shared__ uint32_t weq[kSelWarps];
-  __shared__ unsigned long long cand[EOGP_TOPK_MAX];
-  __shared__ uint32_t s_ngt;
-  const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* row = sc + static_cast<size_t>(q) * ld;
-  for (int i = tid; i < N; i += kSelThreads) skey[i] = sel_key(row[i]);
-  if (tid == 0) s_ngt = 0;
-  __syncthreads();
-  // Valid (non-NaN) scores are the keys >= 1.
-  int parity = 0;
-  const uint32_t nv = count_ge(skey, N, 1u, red, parity);
-  parity ^= 1;
-  const int Kv = static_cast<int>(min(static_cast<uint32_t>(K), nv));
-  if (Kv > 0) {
-    // T = the Kv-th largest key: the largest t with at least Kv keys >= t, built
-    // bit by bit from the top.
-    uint32_t T = 0;
-    for (int bit = 31; bit >= 0; --bit) {
-      const uint32_t c = T | (1u << bit);
-      if (count_ge(skey, N, c, red, parity) >= static_cast<uint32_t>(Kv)) T = c;
-      parity ^= 1;
+  __shared__ unsigned long long cand[kSelCand];
+  __shared__ uint32_t s_n;
+  const int q = blockIdx.x / S, s = blockIdx.x % S, tid = threadIdx.x;
+  const int r0 = s * slice, len = min(slice, N - r0);
+  const float* row = sc + static_cast<size_t>(q) * ld + r0;
+  // Key e = 4 j + c of the thread is row 4 (512 j + tid) + c of the slice; 0 past its end.
+  uint32_t key[4 * kSelVecs];
+  uint32_t top = 0;
+#pragma unroll
+  for (int j = 0; j < kSelVecs; ++j) {
+    const int i = 4 * (j * kSelThreads + tid);
+    float v[4];
+    if (i + 3 < len) {
+      const float4 f = *reinterpret_cast<const float4*>(row + i);
+      v[0] = f.x;
+      v[1] = f.y;
+      v[2] = f.z;
+      v[3] = f.w;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = i + c < len ? row[i + c] : NAN;
     }
-    const uint32_t ngt = T == 0xFFFFFFFFu ? 0u : count_ge(skey, N, T + 1u, red, parity);
-    parity ^= 1;
-    const uint32_t rem = static_cast<uint32_t>(Kv) - ngt;  // keys equal to T that rank, >= 1
-    // Gather. Keys above T (ngt of them) in any order; keys equal to T in index
-    // order, so that the rem lowest indices win: warp w scans the contiguous
-    // segment [w seg, (w+1) seg) twice (count, then place).
-    const int seg = ((N + kSelWarps - 1) / kSelWarps + 31) & ~31;
-    const int b0 = warp * seg, b1 = min(N, b0 + seg);
-    uint32_t mine = 0;
-    for (int base = b0; base < b1; base += 32) {
-      const int i = base + lane;
-      mine += __popc(__ballot_sync(0xffffffffu, i < b1 && skey[i] == T));
-    }
-    if (lane == 0) weq[warp] = mine;
-    __syncthreads();
-    uint32_t before = 0;
-    for (int w = 0; w < warp; ++w) before += weq[w];
-    for (int base = b0; base < b1; base += 32) {
-      const int i = base + lane;
-      const uint32_t k = i < b1 ? skey[i] : 0u;
-      const unsigned long long ck =
-          (static_cast<unsigned long long>(k) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(i));
-      if (k > T) cand[atomicAdd(&s_ngt, 1u)] = ck;
-      const unsigned b = __ballot_sync(0xffffffffu, i < b1 && k == T);
-      const uint32_t pos = before + static_cast<uint32_t>(__popc(b & ((1u << lane) - 1u)));
-      if (((b >> lane) & 1u) && pos < rem) cand[ngt + pos] = ck;
-      before += static_cast<uint32_t>(__popc(b));
-    }
-    __syncthreads();
-    // Sort the Kv winners: descending key = score descending, then lower index.
-    int P = 1;
-    while (P < Kv) P <<= 1;
-    for (int i = Kv + tid; i < P; i += kSelThreads) cand[i] = 0ull;
-    __syncthreads();
-    for (int k2 = 2; k2 <= P; k2 <<= 1) {
-      for (int j = k2 >> 1; j > 0; j >>= 1) {
-        for (int i = tid; i < P; i += kSelThreads) {
-          const int ixj = i ^ j;
-          if (ixj > i) {
-            const unsigned long long a = cand[i], b2 = cand[ixj];
-            const bool desc = (i & k2) == 0;
-            if (desc ? (a < b2) : (a > b2)) {
-              cand[i] = b2;
-              cand[ixj] = a;
-            }
-          }
-        }
-        __syncthreads();
-      }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      key[4 * j + c] = sel_key(v[c]);
+      top = max(top, key[4 * j + c]);
     }
   }
-  for (int p = tid; p < K; p += kSelThreads) {
-    float v = -INFINITY;
-    int ix = -1;
-    if (p < Kv) {
-      ix = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(cand[p]));
-      v = row[ix];  // the stored score itself (keys merge -0 into +0)
+  // (score, lower place first), 0 for no score. Lists come in the order of their
+  // slices and equal scores within them by place, so the lower place is the lower
+  // stored row at every level.
+  auto composite = [&](int e) -> unsigned long long {
+    const int i = 4 * ((e >> 2) * kSelThreads + tid) + (e & 3);
+    return key[e] ? (static_cast<unsigned long long>(key[e]) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(i)) : 0ull;
+  };
+  if (tid == 0) s_n = 0;
+  // Lower bound: the K-th largest thread maximum, its upper 20 bits (a few more
+  // candidates for twelve barriers less). At least K keys are at or above it,
+  // unless fewer than K threads hold a score: then every score is a candidate.
+  uint32_t t0 = 0;
+  for (int bit = 31; bit >= 12; --bit) {
+    const uint32_t c = t0 | (1u << bit);
+    if (__syncthreads_count(top >= c) >= K) t0 = c;
+  }
+  t0 = max(t0, 1u);
+  if (top >= t0) {
+#pragma unroll
+    for (int e = 0; e < 4 * kSelVecs; ++e)
+      if (key[e] >= t0) {
+        const uint32_t p = atomicAdd(&s_n, 1u);
+        if (p < kSelCand) cand[p] = composite(e);
+      }
+  }
+  __syncthreads();
+  int n = static_cast<int>(s_n);
+  if (n > kSelCand) {
+    // T = the Kv-th largest composite (all are distinct), Kv = min(K, scores): the
+    // largest value with at least Kv composites at or above it.
+    uint32_t c = 0;
+#pragma unroll
+    for (int e = 0; e < 4 * kSelVecs; ++e) c += key[e] ? 1u : 0u;
+    int parity = 0;
+    const uint32_t nv = block_sum(c, red, parity);
+    const uint32_t Kv = min(static_cast<uint32_t>(K), nv);
+    unsigned long long T = 0;
+    for (int bit = 63; bit >= 0; --bit) {
+      const unsigned long long t = T | (1ull << bit);
+      c = 0;
+#pragma unroll
+      for (int e = 0; e < 4 * kSelVecs; ++e) c += composite(e) >= t ? 1u : 0u;
+      parity ^= 1;
+      if (block_sum(c, red, parity) >= Kv) T = t;
     }
-    out_s[static_cast<size_t>(q) * ld_os + p] = v;
-    out_i[static_cast<size_t>(q) * ld_oi + p] = ix;
+    if (tid == 0) s_n = 0;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4 * kSelVecs; ++e)
+      if (composite(e) >= T) cand[atomicAdd(&s_n, 1u)] = composite(e);
+    __syncthreads();
+    n = static_cast<int>(s_n);
+  }
+  // Each candidate's rank among them is its place in the list.
+  float* os = out_s + static_cast<size_t>(q) * ld_os + static_cast<size_t>(s) * K;
+  int* oi = out_i + static_cast<size_t>(q) * ld_oi + static_cast<size_t>(s) * K;
+  const int* mp = map ? map + static_cast<size_t>(q) * ld + r0 : nullptr;
+  for (int i = tid; i < n; i += kSelThreads) {
+    const unsigned long long mine = cand[i];
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += cand[j] > mine ? 1 : 0;
+    if (rank < K) {
+      const int at = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(mine));
+      os[rank] = row[at];  // the score itself (keys merge -0 into +0)
+      oi[rank] = mp ? mp[at] : row0 + r0 + at;
+    }
+  }
+  for (int p = n + tid; p < K; p += kSelThreads) {
+    os[p] = mid ? NAN : -INFINITY;
+    oi[p] = -1;
   }
 }
 
@@ -282,58 +256,28 @@ __global__ void __launch_bounds__(256) k_topk_merge(const float* __restrict__ ls
   }
 }
 
-int rows_per_slot(int N) {
-  const int nch = (N + kChunk - 1) / kChunk;
-  const int per = (nch + kMaxSlots - 1) / kMaxSlots;
-  return std::max(1, per) * kChunk;
-}
-
 }  // namespace
 
-int topk_dense_slots(int N) {
-  const int R = rows_per_slot(N);
-  return std::max(1, (N + R - 1) / R);
+// One block ranks up to 16,384 stored rows of a query by itself; more rows take
+// the fewest slices of that size, or for few queries enough of at least 4096 rows
+// to give every SM two blocks.
+int topk_slice(int N, int Q) {
+  if (N <= kSelSlice) return kSelSlice;
+  const int least = (N + kSelSlice - 1) / kSelSlice;
+  const int S = std::max(least, std::min((N + 4095) / 4096, (2 * 152 + Q - 1) / std::max(Q, 1)));
+  return ((N + S - 1) / S + 3) & ~3;
 }
 
-template <int E>
-cudaError_t launch_topk_dense_e(const float* scores, int ld, int Q, int N, int K, float* lst, int* lsi,
-                                cudaStream_t st) {
-  const int S = topk_dense_slots(N);
-  const size_t smem = (32 * kTs + 32 * static_cast<size_t>(32 * E) * 2 + 64) * 4;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_topk_dense<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
-  dim3 grid(S, (Q + 31) / 32);
-  k_topk_dense<E><<<grid, 32, smem, st>>>(scores, ld, Q, N, K, rows_per_slot(N), lst, lsi);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_topk_dense(const float* scores, int ld, int Q, int N, int K, float* lst, int* lsi,
-                              cudaStream_t st) {
+cudaError_t launch_topk_select(const float* scores, const int* map, size_t ld, int Q, int N, int row0, int K, int slice,
+                               bool mid, float* out_s, size_t ld_os, int* out_i, size_t ld_oi, cudaStream_t st) {
   if (Q <= 0) return cudaSuccess;
-  switch (eogp::topk_entries_per_lane(K)) {
-    case 2: return launch_topk_dense_e<2>(scores, ld, Q, N, K, lst, lsi, st);
-    case 4: return launch_topk_dense_e<4>(scores, ld, Q, N, K, lst, lsi, st);
-    case 8: return launch_topk_dense_e<8>(scores, ld, Q, N, K, lst, lsi, st);
-    default: return launch_topk_dense_e<16>(scores, ld, Q, N, K, lst, lsi, st);
-  }
-}
-
-int topk_select_max_n() { return kSelectMaxN; }
-
-cudaError_t launch_topk_select(const float* scores, int ld, int Q, int N, int K, float* out_s, int ld_os,
-                               int* out_i, int ld_oi, cudaStream_t st) {
-  if (Q <= 0) return cudaSuccess;
-  if (N > kSelectMaxN || K > EOGP_TOPK_MAX) return cudaErrorInvalidValue;
-  const size_t smem = static_cast<size_t>(std::max(N, 1)) * 4;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_topk_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
-  k_topk_select<<<Q, kSelThreads, smem, st>>>(scores, ld, N, K, out_s, ld_os, out_i, ld_oi);
+  const int S = std::max(1, (N + slice - 1) / slice);
+  const long long blocks = static_cast<long long>(S) * Q;
+  if (K > EOGP_TOPK_MAX || slice > kSelSlice || (slice & 3) || (ld & 3) || (reinterpret_cast<uintptr_t>(scores) & 15) ||
+      blocks > 0x7FFFFFFF)
+    return cudaErrorInvalidValue;
+  k_topk_select<<<static_cast<unsigned>(blocks), kSelThreads, 0, st>>>(scores, map, ld, N, row0, K, S, slice, mid ? 1 : 0,
+                                                                       out_s, ld_os, out_i, ld_oi);
   return cudaGetLastError();
 }
 

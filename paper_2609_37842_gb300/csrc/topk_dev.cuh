@@ -1,5 +1,5 @@
 // Running per-query top-K lists, kept by one warp per query column (device
-// helpers shared by the fused scoring epilogue and the dense ranking kernel).
+// helpers of the fused scoring epilogue).
 //
 // A column's list is a buffer of 32 E (score, stored index) entries in shared
 // memory, its fill count and a threshold tau. Candidates (scores above tau) are
@@ -15,11 +15,6 @@
 #include <cmath>
 
 namespace eogp {
-
-// Entries per lane of a list that must hold K: the buffer takes K plus one ballot.
-__host__ __device__ constexpr int topk_entries_per_lane(int K) {
-  return K <= 32 ? 2 : K <= 96 ? 4 : K <= 224 ? 8 : 16;
-}
 
 struct WarpTopk {
   float* ls;   // [32 E] scores
@@ -125,14 +120,6 @@ __device__ __forceinline__ void topk_prune(const WarpTopk& w, int lane) {
     // Another list of the same query may skip scores below this one: this list
     // alone holds K stored rows scoring at least kth.
     if (keep == w.K && w.shared_tau) atomicMax(w.shared_tau, topk_key32(kth));
-  }
-  __syncwarp();
-}
-
-__device__ __forceinline__ void topk_warp_reset(const WarpTopk& w, int lane) {
-  if (lane == 0) {
-    *w.cnt = 0;
-    *w.tau = NAN;
   }
   __syncwarp();
 }
