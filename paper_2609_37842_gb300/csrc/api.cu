@@ -660,16 +660,22 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
   float* at = reinterpret_cast<float*>(w + lo.at);
   float* stt = reinterpret_cast<float*>(w + lo.st);
   const int nC = P->nC(), nR = P->nR();
-  CUDA_TRY(launch_simt_gemm(M, nC, L->d_in, 1.f, af, L->d_in, 1, static_cast<const float*>(VA),
-                            L->d_in, 1, at, nC, st));
-  CUDA_TRY(launch_simt_gemm(M, nR, L->d_out, 1.f, sf, L->d_out, 1, static_cast<const float*>(VS),
-                            L->d_out, 1, stt, nR, st));
-  CUDA_TRY(launch_rows_fixup(at, M, nC, nC, L->T, L->bias_A, nullptr, st));
-  CUDA_TRY(launch_rows_fixup(stt, M, nR, nR, L->T, nullptr, L->lengths, st));
   float* z = out_mode == EOGP_OUT_FIRST_STAGE ? out : reinterpret_cast<float*>(w + lo.z);
   const int ldz = out_mode == EOGP_OUT_FIRST_STAGE ? ld_out : L->m;
-  CUDA_TRY(launch_contract_f32(at, nC, stt, nR, B, L->T, L->m, P->d_posR, P->d_posC, P->d_scale, z,
-                               ldz, st));
+  if (f32_first_supported(B, L->T, nC, nR)) {
+    CUDA_TRY(launch_f32_first(af, sf, static_cast<const float*>(VA), static_cast<const float*>(VS), L->d_in, L->d_out,
+                              L->bias_A, L->lengths, B, L->T, L->m, nC, nR, P->d_posR, P->d_posC, P->d_scale, z, ldz,
+                              st));
+  } else {
+    CUDA_TRY(launch_simt_gemm(M, nC, L->d_in, 1.f, af, L->d_in, 1, static_cast<const float*>(VA),
+                              L->d_in, 1, at, nC, st));
+    CUDA_TRY(launch_simt_gemm(M, nR, L->d_out, 1.f, sf, L->d_out, 1, static_cast<const float*>(VS),
+                              L->d_out, 1, stt, nR, st));
+    CUDA_TRY(launch_rows_fixup(at, M, nC, nC, L->T, L->bias_A, nullptr, st));
+    CUDA_TRY(launch_rows_fixup(stt, M, nR, nR, L->T, nullptr, L->lengths, st));
+    CUDA_TRY(launch_contract_f32(at, nC, stt, nR, B, L->T, L->m, P->d_posR, P->d_posC, P->d_scale, z,
+                                 ldz, st));
+  }
   if (out_mode == EOGP_OUT_FIRST_STAGE) return EOGP_OK;
   if (uses_srht(L)) {
     const bool cd = out_mode == EOGP_OUT_CODES;
