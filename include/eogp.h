@@ -477,7 +477,11 @@ int eogp_score_workspace_size(int N, const int* k_per_module, int U, int mode, i
  *          the tensor cores with y split into bf16 hi + lo (about 2^-17 relative)
  *          and fp32 sums: |error| <= 1e-5 sum_u s_iu ||y_qu||_1 for k_u <= 16384.
  *   FP:    train = fp32 coordinates [N x ld_train], query = fp32 [Q x ld_query];
- *          scores[q][i] = <y_q, x_i>; scales ignored.
+ *          scores[q][i] = <y_q, x_i>; scales ignored. With 512 coordinates or
+ *          more, ld_train % 4 == 0, a 16-byte aligned base and the workspace
+ *          eogp_score_workspace_size reports, on the tensor cores with both sides
+ *          as exact sums of three bf16 parts (error against 64-bit sums no larger
+ *          than an fp32 chain's), else one fp32 chain per score.
  * scores [Q x ld_scores] fp32 device, ld_scores >= N.
  * ws: 256-byte aligned device workspace of at least eogp_score_workspace_size
  * bytes (0 bytes for the CUDA-core kernels); CODES and PAPER use the tensor

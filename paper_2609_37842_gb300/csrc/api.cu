@@ -1278,11 +1278,13 @@ extern "C" int eogp_score_workspace_size(int N, const int* k_per_module, int U, 
                                          size_t* bytes) {
   clear_error();
   if (!bytes) return set_error(EOGP_EINVAL, "bytes is NULL");
-  (void)N;
   *bytes = 0;
   if ((mode == EOGP_SCORE_CODES || mode == EOGP_SCORE_PAPER) && k_per_module && U >= 1 &&
       U <= 1024 && score_tc_supported(mode, k_per_module, U, Q))
     *bytes = score_tc_ws_bytes(mode, k_per_module, U, Q);
+  long long W, D;
+  if (mode == EOGP_SCORE_FP && score_args_ok(N, k_per_module, U, &W, &D) && score_fp_supported(N, D, Q))
+    *bytes = score_fp_ws_bytes(N, D, Q, sm_count());
   return EOGP_OK;
 }
 
@@ -1323,6 +1325,16 @@ static int score_dense(const void* train, int ld_train, const float* train_scale
     }
   } else if (mode == EOGP_SCORE_FP) {
     if (ld_train < D || ld_query < D) return set_error(EOGP_EINVAL, "leading dimension too small");
+    // Tensor cores under the same conditions as above.
+    if (score_fp_supported(N, D, Q) && ws && ws_bytes >= score_fp_ws_bytes(N, D, Q, sm_count()) &&
+        (ld_train % 4) == 0 && aligned16(train) && (reinterpret_cast<uintptr_t>(ws) & 255) == 0) {
+      unsigned* status = status_word();
+      if (!status) return set_error(EOGP_ECUDA, "device status word unavailable");
+      CUDA_TRY(launch_score_fp(static_cast<const float*>(train), ld_train, N, static_cast<int>(D),
+                               static_cast<const float*>(query), ld_query, Q, scores, ld_scores, ws, sm_count(),
+                               status, st));
+      return EOGP_OK;
+    }
     CUDA_TRY(launch_simt_gemm(Q, N, static_cast<int>(D), 1.f, static_cast<const float*>(query), ld_query,
                               1, static_cast<const float*>(train), ld_train, 1, scores, ld_scores, st));
   } else {
@@ -1406,6 +1418,13 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
     const long long fit = static_cast<long long>(kTopkDenseMax / (4 * static_cast<size_t>(std::max(Q, 1))));
     p.rows = N <= fit ? std::max(N, 1) : static_cast<int>(std::max<long long>(1, fit / p.slice) * p.slice);
     p.dense_bytes = al256(static_cast<size_t>(Q) * ((static_cast<size_t>(std::min(p.rows, N)) + 3) & ~size_t(3)) * 4);
+    long long W, D;
+    const int nr = std::min(p.rows, N);
+    // a last chunk of fewer rows may take more K ranges: room for either
+    if (mode == EOGP_SCORE_FP && score_args_ok(N, ks, U, &W, &D) && score_fp_supported(nr, D, Q)) {
+      p.q_bytes = score_fp_ws_bytes(nr, D, Q, sm_count());
+      if (N > nr && N % nr) p.q_bytes = std::max(p.q_bytes, score_fp_ws_bytes(N % nr, D, Q, sm_count()));
+    }
     const long long slots = (static_cast<long long>(N) + p.slice - 1) / p.slice;
     p.n1 = slots > 1 ? slots * K : 0;
     p.n2 = p.n1 > kTopkListSlice ? (p.n1 + kTopkListSlice - 1) / kTopkListSlice * K : 0;

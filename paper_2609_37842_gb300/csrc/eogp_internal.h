@@ -112,6 +112,13 @@ cudaError_t launch_score_tc(int mode, const uint32_t* train, int ldt, const floa
                             int ldqs, int Q, float* out, int ldo, const TcTopK* topk, void* ws,
                             int num_sms, unsigned* status, cudaStream_t st);
 
+// k_score_fp.cu: unquantised scores on the tensor cores (rows of `train` 16-byte
+// aligned), with a workspace of score_fp_ws_bytes.
+bool score_fp_supported(int N, long long D, int Q);
+size_t score_fp_ws_bytes(int N, long long D, int Q, int num_sms);
+cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const float* query, int ldq, int Q,
+                            float* out, int ldo, void* ws, int num_sms, unsigned* status, cudaStream_t st);
+
 // k_topk.cu: the K best (K <= EOGP_TOPK_MAX) of every slice of a row of scores
 // [Q x ld] (ld a multiple of 4, 16-byte aligned): slice s of row q to K places at
 // K s + ld_o q. `map`: the values' stored rows (lists of an earlier level), else
