@@ -1282,6 +1282,8 @@ extern "C" int eogp_score_workspace_size(int N, const int* k_per_module, int U, 
   if ((mode == EOGP_SCORE_CODES || mode == EOGP_SCORE_PAPER) && k_per_module && U >= 1 &&
       U <= 1024 && score_tc_supported(mode, k_per_module, U, Q))
     *bytes = score_tc_ws_bytes(mode, k_per_module, U, Q);
+  if (mode == EOGP_SCORE_PAPER && *bytes && N > 0)
+    *bytes = std::max(*bytes, score_paper_ws_bytes(N, k_per_module, U, Q, sm_count()));
   long long W, D;
   if (mode == EOGP_SCORE_FP && score_args_ok(N, k_per_module, U, &W, &D) && score_fp_supported(N, D, Q))
     *bytes = score_fp_ws_bytes(N, D, Q, sm_count());
@@ -1311,9 +1313,14 @@ static int score_dense(const void* train, int ld_train, const float* train_scale
     if (tc) {
       unsigned* status = status_word();
       if (!status) return set_error(EOGP_ECUDA, "device status word unavailable");
-      CUDA_TRY(launch_score_tc(mode, static_cast<const uint32_t*>(train), ld_train, train_scales,
-                               ld_tscale, N, k_per_module, U, query, ld_query, query_scales,
-                               ld_qscale, Q, scores, ld_scores, nullptr, ws, sm_count(), status, st));
+      if (mode == EOGP_SCORE_PAPER && score_paper_supported(N, k_per_module, U, Q, train, ld_train))
+        CUDA_TRY(launch_score_paper_tc(static_cast<const uint32_t*>(train), ld_train, train_scales, ld_tscale, N,
+                                       k_per_module, U, static_cast<const float*>(query), ld_query, Q, scores,
+                                       ld_scores, ws, ws_bytes, sm_count(), status, st));
+      else
+        CUDA_TRY(launch_score_tc(mode, static_cast<const uint32_t*>(train), ld_train, train_scales,
+                                 ld_tscale, N, k_per_module, U, query, ld_query, query_scales,
+                                 ld_qscale, Q, scores, ld_scores, nullptr, ws, sm_count(), status, st));
     } else if (mode == EOGP_SCORE_CODES) {
       CUDA_TRY(launch_score_codes(static_cast<const uint32_t*>(train), ld_train, train_scales,
                                   ld_tscale, N, k_per_module, U, static_cast<const uint32_t*>(query),
@@ -1424,6 +1431,10 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
     if (mode == EOGP_SCORE_FP && score_args_ok(N, ks, U, &W, &D) && score_fp_supported(nr, D, Q)) {
       p.q_bytes = score_fp_ws_bytes(nr, D, Q, sm_count());
       if (N > nr && N % nr) p.q_bytes = std::max(p.q_bytes, score_fp_ws_bytes(N % nr, D, Q, sm_count()));
+    }
+    if (mode == EOGP_SCORE_PAPER && tc_ok && nr > 0) {
+      p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(nr, ks, U, Q, sm_count()));
+      if (N % nr) p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(N % nr, ks, U, Q, sm_count()));
     }
     const long long slots = (static_cast<long long>(N) + p.slice - 1) / p.slice;
     p.n1 = slots > 1 ? slots * K : 0;

@@ -119,6 +119,19 @@ size_t score_fp_ws_bytes(int N, long long D, int Q, int num_sms);
 cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const float* query, int ldq, int Q,
                             float* out, int ldo, void* ws, int num_sms, unsigned* status, cudaStream_t st);
 
+// out[q][i] = the S slabs' values [S][Q x ldp], added in order.
+cudaError_t launch_sum_slabs(const float* part, int S, size_t slab, int ldp, int N, int Q, float* out, int ldo,
+                             cudaStream_t st);
+
+// k_score_paper.cu: unquantised queries against stored codes (rows of `train`
+// 16-byte aligned, modules multiples of 64 bits). With the 4 Q sum k bytes the
+// queries take alone as workspace, one K range per row tile.
+bool score_paper_supported(int N, const int* ks, int U, int Q, const void* train, int ldt);
+size_t score_paper_ws_bytes(int N, const int* ks, int U, int Q, int num_sms);
+cudaError_t launch_score_paper_tc(const uint32_t* train, int ldt, const float* ts, int ldts, int N, const int* ks,
+                                  int U, const float* y, int ldy, int Q, float* out, int ldo, void* ws,
+                                  size_t ws_bytes, int num_sms, unsigned* status, cudaStream_t st);
+
 // k_topk.cu: the K best (K <= EOGP_TOPK_MAX) of every slice of a row of scores
 // [Q x ld] (ld a multiple of 4, 16-byte aligned): slice s of row q to K places at
 // K s + ld_o q. `map`: the values' stored rows (lists of an earlier level), else

@@ -379,17 +379,31 @@ __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict_
   for (int i = (q * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < nrt; i += gridDim.y * nthr) rbad[i] = 0;
 }
 
-// scores[q][i] = the slabs' values in order.
-__global__ void k_sum_slabs(const float* __restrict__ part, int S, size_t slab, int ldp, int N, int Q,
-                            float* __restrict__ out, int ldo) {
-  const long long tot = static_cast<long long>(Q) * N;
-  for (long long e = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; e < tot;
-       e += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int q = static_cast<int>(e / N), i = static_cast<int>(e % N);
+// scores[q][i] = the slabs' values in order; four scores a thread (ldp is a
+// multiple of four), query blockIdx.y and on.
+__global__ void __launch_bounds__(256) k_sum_slabs(const float* __restrict__ part, int S, size_t slab, int ldp, int N,
+                                                   int Q, float* __restrict__ out, int ldo, int vec) {
+  const int i = 4 * (blockIdx.x * 256 + threadIdx.x);
+  if (i >= N) return;
+  for (int q = blockIdx.y; q < Q; q += gridDim.y) {
     const float* p = part + static_cast<size_t>(q) * ldp + i;
-    float t = p[0];
-    for (int s = 1; s < S; ++s) t += p[static_cast<size_t>(s) * slab];
-    out[static_cast<size_t>(q) * ldo + i] = t;
+    float4 t = *reinterpret_cast<const float4*>(p);
+    for (int s = 1; s < S; ++s) {
+      const float4 v = *reinterpret_cast<const float4*>(p + static_cast<size_t>(s) * slab);
+      t.x += v.x;
+      t.y += v.y;
+      t.z += v.z;
+      t.w += v.w;
+    }
+    float* o = out + static_cast<size_t>(q) * ldo + i;
+    if (vec && i + 3 < N) {
+      *reinterpret_cast<float4*>(o) = t;
+    } else {
+      o[0] = t.x;
+      if (i + 1 < N) o[1] = t.y;
+      if (i + 2 < N) o[2] = t.z;
+      if (i + 3 < N) o[3] = t.w;
+    }
   }
 }
 
@@ -443,6 +457,13 @@ cudaError_t launch_qb(const CUtensorMap& tx, const CUtensorMap& ty, const FpArgs
 
 }  // namespace
 
+cudaError_t launch_sum_slabs(const float* part, int S, size_t slab, int ldp, int N, int Q, float* out, int ldo,
+                             cudaStream_t st) {
+  const int vec = (ldo & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  k_sum_slabs<<<dim3((N + 1023) / 1024, std::min(Q, 65535)), 256, 0, st>>>(part, S, slab, ldp, N, Q, out, ldo, vec);
+  return cudaGetLastError();
+}
+
 bool score_fp_supported(int N, long long D, int Q) {
   return D >= kMinD && N >= 1 && Q >= 1 && Q <= 65535 && D <= (1 << 28) &&
          static_cast<long long>((N + 127) / 128) * ((Q + 63) / 64) * 32 < (1ll << 30);
@@ -494,10 +515,7 @@ cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const flo
                    : launch_qb<16>(tx, ty, g, num_sms, st);
   if (e != cudaSuccess) return e;
   if (p.S > 1) {
-    const long long tot = static_cast<long long>(Q) * N;
-    k_sum_slabs<<<static_cast<unsigned>(std::min<long long>((tot + 255) / 256, 152 * 16)), 256, 0, st>>>(
-        part, p.S, g.slab, p.ldp, N, Q, out, ldo);
-    e = cudaGetLastError();
+    e = launch_sum_slabs(part, p.S, g.slab, p.ldp, N, Q, out, ldo, st);
     if (e != cudaSuccess) return e;
   }
   // scores of rows and queries with an infinity or a NaN, in fp32
