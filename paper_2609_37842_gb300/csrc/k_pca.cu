@@ -8,12 +8,10 @@
 //  1. A = Z^T Z / n (or Z Z^T): CUDA-core GEMM on the fp32 Z with fp64
 //     accumulation.
 //  2. Cyclic two-sided Jacobi (Golub & Van Loan, Sec. 8.5) in round-robin
-//     ("circle") order: each step rotates nn'/2 disjoint (p, q) pairs. One
-//     kernel forms the rotations (in double) from the current A; a second
-//     applies J^T A J to rows p, q of A (row rotation, then the column
-//     rotations of every pair inside the two rows held in shared memory) and
-//     J^T to rows p, q of V^T. Sweeps repeat until the off-diagonal mass stops
-//     shrinking or falls below 1e-11 of ||A||_F; A and V^T are kept in fp64.
+//     ("circle") order: each step rotates nn'/2 disjoint (p, q) pairs, J^T A J and
+//     J^T V^T, in double; a sweep of steps is one kernel (k_jacobi_sweep). Sweeps
+//     repeat until the off-diagonal mass stops shrinking or falls below 1e-11 of
+//     ||A||_F; A and V^T are kept in fp64.
 //  3. Rank the eigenvalues (descending, ties to the lower index), keep the top
 //     k, map Gram-route vectors through Z^T u / ||Z^T u||, normalise, and fix
 //     each vector's sign so its largest-magnitude entry is positive.
@@ -135,83 +133,221 @@ __global__ void k_eye(double* V, int n) {
   V[idx] = (idx / n == idx % n) ? 1.0 : 0.0;
 }
 
-__global__ void k_jacobi_params(const double* __restrict__ A, int n, int np, int s,
-                                double* __restrict__ cs) {
-  const int kidx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (kidx >= np / 2) return;
-  int p, q;
-  jac_pair(s, kidx, np, p, q);
-  double c = 1.0, sn = 0.0;
-  if (q < n) {
-    const double app = A[static_cast<size_t>(p) * n + p];
-    const double aqq = A[static_cast<size_t>(q) * n + q];
-    const double apq = A[static_cast<size_t>(p) * n + q];
-    if (apq != 0.0) {
-      const double tau = (aqq - app) / (2.0 * apq);
-      double t;
-      if (fabs(tau) > 1e150) {
-        t = 0.5 / tau;
-      } else {
-        t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-      }
-      c = 1.0 / sqrt(1.0 + t * t);
-      sn = t * c;
-    }
-  }
-  cs[2 * kidx] = c;
-  cs[2 * kidx + 1] = sn;
+// The pair of element x at step s (inverse of jac_pair).
+__device__ __forceinline__ int jac_index(int s, int x, int np) {
+  const int L = np - 1;
+  if (x == L || x == s) return 0;
+  const int d = x > s ? x - s : x - s + L;
+  return d < np / 2 ? d : L - d;
 }
 
-__global__ void __launch_bounds__(256) k_jacobi_apply(double* __restrict__ A, double* __restrict__ Vt,
-                                                      int n, int np, int s,
-                                                      const double* __restrict__ cs) {
-  extern __shared__ double rows[];
-  double* rp = rows;
-  double* rq = rows + n;
-  const int kidx = blockIdx.x;
-  int p, q;
-  jac_pair(s, kidx, np, p, q);
-  if (q >= n) return;
-  const double c = cs[2 * kidx];
-  const double sn = cs[2 * kidx + 1];
-  double* Ap = A + static_cast<size_t>(p) * n;
-  double* Aq = A + static_cast<size_t>(q) * n;
-  for (int x = threadIdx.x; x < n; x += blockDim.x) {
-    const double ap = Ap[x], aq = Aq[x];
-    rp[x] = c * ap - sn * aq;
-    rq[x] = sn * ap + c * aq;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < np / 2; j += blockDim.x) {
-    int pj, qj;
+// (x, y) <- (c x - s y, s x + c y)
+__device__ __forceinline__ void jac_rotate(double c, double s, double& x, double& y) {
+  const double a = x, b = y;
+  x = c * a - s * b;
+  y = s * a + c * b;
+}
+
+// Entry (x, y) after step s, formed from A before it and the step's rotations:
+// rows x and its partner rotated, then columns y and its partner. A row without a
+// partner (odd n) stays as it is. Loads and arithmetic apart, so that the loads of
+// several entries are in flight together.
+struct JacEntry {
+  double a, b, c, d;  // rows (x's pair) by columns (y's pair)
+  double2 ck, cj;
+  bool low_row, low_col, row_alone, col_alone, zero;
+  __device__ __forceinline__ void load(const double* __restrict__ A, int n, int np, int s,
+                                       const double2* __restrict__ cs, int x, int y) {
+    const int k = jac_index(s, x, np), j = jac_index(s, y, np);
+    int p, q, pj, qj;
+    jac_pair(s, k, np, p, q);
     jac_pair(s, j, np, pj, qj);
-    if (qj >= n) continue;
-    const double cj = cs[2 * j];
-    const double sj = cs[2 * j + 1];
-    double xp = rp[pj], xq = rp[qj];
-    rp[pj] = cj * xp - sj * xq;
-    rp[qj] = sj * xp + cj * xq;
-    xp = rq[pj];
-    xq = rq[qj];
-    rq[pj] = cj * xp - sj * xq;
-    rq[qj] = sj * xp + cj * xq;
+    row_alone = q >= n;
+    col_alone = qj >= n;
+    low_row = x == p;
+    low_col = y == pj;
+    zero = k == j && x != y;
+    const double* Ap = A + static_cast<size_t>(p) * n;
+    const double* Aq = A + static_cast<size_t>(row_alone ? p : q) * n;
+    const int qc = col_alone ? pj : qj;
+    ck = __ldcg(cs + k);
+    cj = __ldcg(cs + j);
+    a = __ldcg(Ap + pj);
+    b = __ldcg(Ap + qc);
+    c = __ldcg(Aq + pj);
+    d = __ldcg(Aq + qc);
+  }
+  __device__ __forceinline__ double value() {
+    if (row_alone) return low_col ? a : b;
+    jac_rotate(ck.x, ck.y, a, c);
+    if (col_alone) return low_row ? a : c;
+    jac_rotate(ck.x, ck.y, b, d);
+    jac_rotate(cj.x, cj.y, a, b);
+    jac_rotate(cj.x, cj.y, c, d);
+    if (zero && ck.y != 0.0) return 0.0;  // the annihilated pair
+    return low_row ? (low_col ? a : b) : (low_col ? c : d);
+  }
+};
+
+// The rotation that annihilates apq.
+__device__ double2 jac_params(double app, double aqq, double apq) {
+  double c = 1.0, sn = 0.0;
+  if (apq != 0.0) {
+    const double tau = (aqq - app) / (2.0 * apq);
+    double t;
+    if (fabs(tau) > 1e150) {
+      t = 0.5 / tau;
+    } else {
+      t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+    }
+    c = 1.0 / sqrt(1.0 + t * t);
+    sn = t * c;
+  }
+  return make_double2(c, sn);
+}
+
+// All blocks of the grid (a cooperative launch) wait until every one has arrived;
+// `count` rises by gridDim.x per barrier. Bounded: false after ~2 s, and the
+// status word says so.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, unsigned* status) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(count, 1u);
+    const long long t0 = clock64();
+    unsigned v;
+    ok = 1;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+      if (static_cast<int>(v - target) < 0 && clock64() - t0 > EOGP_WAIT_CYCLES) {
+        eogp::flag_status(status, EOGP_ST_TIMEOUT);
+        ok = 0;
+        break;
+      }
+    } while (static_cast<int>(v - target) < 0);
+    __threadfence();
   }
   __syncthreads();
-  if (threadIdx.x == 0 && sn != 0.0) {
-    rp[q] = 0.0;  // the annihilated pair
-    rq[p] = 0.0;
+  return ok != 0;
+}
+
+// One sweep: np - 1 steps, one grid-wide barrier each. A step reads A from one
+// buffer and writes the other, so everything in it is independent given its
+// rotations: the 2 x 2 blocks of A (pair k's rows by pair j's columns, a thread
+// each: J^T A J takes 16 fp64 operations on the four entries), the rows of V^T, and
+// the rotations of the next step, whose three entries of the new A are formed again
+// from the old one rather than waited for. Bound by the fp64 rate (6 operations per
+// entry and step) and the barrier. Measured at n = 640: 8.5 us a step, against 16.4
+// for two kernels a step (rotations, then whole rows in shared memory).
+constexpr int kJacThreads = 512;
+
+__global__ void __launch_bounds__(kJacThreads, 1)
+    k_jacobi_sweep(double* __restrict__ A0, double* __restrict__ A1, double* __restrict__ Vt, int n, int np,
+                   double2* __restrict__ cs0, double2* __restrict__ cs1, unsigned* count, unsigned* status) {
+  __shared__ int s_task;
+  const int h = np / 2, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kWarps = kJacThreads / 32;
+  unsigned target = gridDim.x;
+  for (int k = blockIdx.x + gridDim.x * threadIdx.x; k < h; k += gridDim.x * kJacThreads) {
+    int p, q;
+    jac_pair(0, k, np, p, q);
+    double2 r = make_double2(1.0, 0.0);
+    if (q < n)
+      r = jac_params(__ldcg(A0 + static_cast<size_t>(p) * n + p), __ldcg(A0 + static_cast<size_t>(q) * n + q),
+                     __ldcg(A0 + static_cast<size_t>(p) * n + q));
+    __stcg(cs0 + k, r);
   }
-  __syncthreads();
-  for (int x = threadIdx.x; x < n; x += blockDim.x) {
-    Ap[x] = rp[x];
-    Aq[x] = rq[x];
-  }
-  double* Vp = Vt + static_cast<size_t>(p) * n;
-  double* Vq = Vt + static_cast<size_t>(q) * n;
-  for (int x = threadIdx.x; x < n; x += blockDim.x) {
-    const double vp = Vp[x], vq = Vq[x];
-    Vp[x] = c * vp - sn * vq;
-    Vq[x] = sn * vp + c * vq;
+  if (threadIdx.x == 0) s_task = 0;
+  if (!grid_barrier(count, target, status)) return;
+  const int jc = (h + 31) / 32;           // warp tasks of a pair's rows of A
+  const int xc = (n + 63) / 64;           // and of V^T, two columns a lane
+  const int nA = h * jc, nAll = nA + h * xc;
+  const int pb = max(1, min((h + 31) / 32, static_cast<int>(gridDim.x) / 8));  // blocks for the rotations
+  for (int s = 0; s < np - 1; ++s) {
+    const double* A = s & 1 ? A1 : A0;
+    double* B = s & 1 ? A0 : A1;
+    const double2* cs = s & 1 ? cs1 : cs0;
+    double2* csn = s & 1 ? cs0 : cs1;
+    // The next step's rotations, a lane each: a long chain of divisions and roots
+    // that would wait for its turn at the fp64 unit behind every other warp of its
+    // SM, so the first blocks do nothing else.
+    if (blockIdx.x < pb) {
+      if (s + 1 < np - 1)
+        for (int k = 32 * (blockIdx.x + pb * warp) + lane; k < h; k += 32 * pb * kWarps) {
+          int p, q;
+          jac_pair(s + 1, k, np, p, q);
+          double2 r = make_double2(1.0, 0.0);
+          if (q < n) {
+            JacEntry pp, qq, pq;
+            pp.load(A, n, np, s, cs, p, p);
+            qq.load(A, n, np, s, cs, q, q);
+            pq.load(A, n, np, s, cs, p, q);
+            const double app = pp.value(), aqq = qq.value();
+            r = jac_params(app, aqq, pq.value());
+          }
+          __stcg(csn + k, r);
+        }
+    }
+    // The other blocks' tasks, taken by their warps as they come free.
+    while (blockIdx.x >= pb) {
+      int t = 0;
+      if (lane == 0) t = atomicAdd(&s_task, 1);
+      t = blockIdx.x - pb + (static_cast<int>(gridDim.x) - pb) * __shfl_sync(0xffffffffu, t, 0);
+      if (t >= nAll) break;
+      if (t < nA) {
+        const int k = t / jc, j = (t - k * jc) * 32 + lane;
+        if (j >= h) continue;
+        int p, q, pj, qj;
+        jac_pair(s, k, np, p, q);
+        jac_pair(s, j, np, pj, qj);
+        const size_t rp = static_cast<size_t>(p) * n, rq = static_cast<size_t>(q) * n;
+        if (q >= n) {  // a row without a partner
+          __stcg(B + rp + pj, __ldcg(A + rp + pj));
+          if (qj < n) __stcg(B + rp + qj, __ldcg(A + rp + qj));
+          continue;
+        }
+        const double2 ck = __ldcg(cs + k);
+        double a = __ldcg(A + rp + pj), c = __ldcg(A + rq + pj);
+        if (qj < n) {
+          const double2 cj = __ldcg(cs + j);
+          double b = __ldcg(A + rp + qj), d = __ldcg(A + rq + qj);
+          jac_rotate(ck.x, ck.y, a, c);
+          jac_rotate(ck.x, ck.y, b, d);
+          jac_rotate(cj.x, cj.y, a, b);
+          jac_rotate(cj.x, cj.y, c, d);
+          if (k == j && ck.y != 0.0) b = c = 0.0;  // the annihilated pair
+          __stcg(B + rp + qj, b);
+          __stcg(B + rq + qj, d);
+        } else {
+          jac_rotate(ck.x, ck.y, a, c);
+        }
+        __stcg(B + rp + pj, a);
+        __stcg(B + rq + pj, c);
+      } else {
+        const int k = (t - nA) / xc, x0 = ((t - nA) - k * xc) * 64 + lane;
+        int p, q;
+        jac_pair(s, k, np, p, q);
+        if (q >= n) continue;
+        const double2 ck = __ldcg(cs + k);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int x = x0 + 32 * e;
+          if (x < n) {
+            double* vp = Vt + static_cast<size_t>(p) * n + x;
+            double* vq = Vt + static_cast<size_t>(q) * n + x;
+            double a = __ldcg(vp), b = __ldcg(vq);
+            jac_rotate(ck.x, ck.y, a, b);
+            __stcg(vp, a);
+            __stcg(vq, b);
+          }
+        }
+      }
+    }
+    target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) s_task = 0;
+    if (!grid_barrier(count, target, status)) return;
   }
 }
 
@@ -475,76 +611,112 @@ __global__ void __launch_bounds__(256) k_diag_shift(const float* __restrict__ A,
   if (threadIdx.x == 0) shift[0] = static_cast<float>(rel * red[0] / n);
 }
 
-// ---- blocked Cholesky (lower, in place, fp32), panels of 32 columns
-// Diagonal block at j0: 32 x 32 threads, one entry each.
-__global__ void __launch_bounds__(1024) k_chol_diag(float* __restrict__ A, int lda, int n, int j0,
-                                                    unsigned* status) {
-  __shared__ float a[32][33];
-  const int i = threadIdx.y, j = threadIdx.x;
-  const int nb = min(32, n - j0);
-  a[i][j] = (i < nb && j < nb) ? A[static_cast<long long>(j0 + i) * lda + j0 + j] : 0.f;
-  __syncthreads();
-  for (int c = 0; c < nb; ++c) {
-    if (i == c && j == c) {
-      float d = a[c][c];
-      if (!(d > 0.f) || !isfinite(d)) {  // not positive definite: flag it, keep going
-        eogp::flag_status(status, EOGP_ST_DEVICE);
-        d = 1e-30f;
+// ---- blocked Cholesky (lower, in place, fp32), panels of 32 columns: the first
+// diagonal block, then per panel one kernel for the rows below it and one for the
+// trailing matrix, whose first block also factors the next diagonal block.
+
+// Factors a 32 x 32 block in one warp: lane i holds row i in registers, the column
+// being eliminated is passed by shuffles. Entries above the diagonal come out as 0.
+__device__ __forceinline__ void chol_block(float (&a)[32], int lane, int nb, unsigned* status) {
+#pragma unroll
+  for (int c = 0; c < 32; ++c) {
+    if (c < nb) {
+      if (lane == c) {
+        float d = a[c];
+        if (!(d > 0.f) || !isfinite(d)) {  // not positive definite: flag it, keep going
+          eogp::flag_status(status, EOGP_ST_DEVICE);
+          d = 1e-30f;
+        }
+        a[c] = sqrtf(d);
       }
-      a[c][c] = sqrtf(d);
+      const float dc = __shfl_sync(0xffffffffu, a[c], c);
+      if (lane > c) a[c] /= dc;
+#pragma unroll
+      for (int j = c + 1; j < 32; ++j) {
+        const float ajc = __shfl_sync(0xffffffffu, a[c], j);
+        if (j <= lane) a[j] -= a[c] * ajc;
+      }
     }
-    __syncthreads();
-    if (j == c && i > c && i < nb) a[i][c] /= a[c][c];
-    __syncthreads();
-    if (i > c && j > c && j <= i && i < nb) a[i][j] -= a[i][c] * a[j][c];
-    __syncthreads();
   }
-  if (i < nb && j < nb) A[static_cast<long long>(j0 + i) * lda + j0 + j] = (j <= i) ? a[i][j] : 0.f;
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (j > lane) a[j] = 0.f;
+}
+
+__global__ void __launch_bounds__(32) k_chol_diag(float* __restrict__ A, int lda, int n, int j0, unsigned* status) {
+  const int lane = threadIdx.x, nb = min(32, n - j0);
+  float a[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    a[j] = (lane < nb && j < nb) ? A[static_cast<long long>(j0 + lane) * lda + j0 + j] : 0.f;
+  chol_block(a, lane, nb, status);
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (lane < nb && j < nb) A[static_cast<long long>(j0 + lane) * lda + j0 + j] = a[j];
 }
 
 // Rows i >= j0 + 32: A[i][j0..j0+32) <- A[i][j0..j0+32) L_d^-T (forward
-// substitution, one thread per row).
-__global__ void __launch_bounds__(128) k_chol_panel(float* __restrict__ A, int lda, int n, int j0) {
+// substitution, one thread per row; rows are 16-byte aligned).
+__global__ void __launch_bounds__(64) k_chol_panel(float* __restrict__ A, int lda, int n, int j0) {
   __shared__ float L[32][33];
-  for (int e = threadIdx.x; e < 1024; e += 128) {
+  for (int e = threadIdx.x; e < 1024; e += 64) {
     const int r = e >> 5, c = e & 31;
     L[r][c] = A[static_cast<long long>(j0 + r) * lda + j0 + c];
   }
-  __syncthreads();
-  const int i = j0 + 32 + blockIdx.x * 128 + threadIdx.x;
-  if (i >= n) return;
-  float* row = A + static_cast<long long>(i) * lda + j0;
+  const int i = j0 + 32 + blockIdx.x * 64 + threadIdx.x;
+  float4* row = reinterpret_cast<float4*>(A + static_cast<long long>(i) * lda + j0);
   float x[32];
+  if (i < n) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float4 v = row[c];
+      x[4 * c] = v.x, x[4 * c + 1] = v.y, x[4 * c + 2] = v.z, x[4 * c + 3] = v.w;
+    }
+  }
+  __syncthreads();
+  if (i >= n) return;
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
-    float v = row[c];
+    float v = x[c];
 #pragma unroll
     for (int t = 0; t < c; ++t) v -= x[t] * L[c][t];
     x[c] = v / L[c][c];
   }
 #pragma unroll
-  for (int c = 0; c < 32; ++c) row[c] = x[c];
+  for (int c = 0; c < 8; ++c) row[c] = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
 }
 
 // Trailing update of the lower triangle: A[i][j] -= sum_t A[i][j0 + t] A[j][j0 + t]
 // for j0 + 32 <= j <= i < n; one block per 64 x 64 tile on or below the diagonal.
-__global__ void __launch_bounds__(256) k_chol_update(float* __restrict__ A, int lda, int n, int j0) {
+// Block 0 holds the next diagonal block and factors it.
+__global__ void __launch_bounds__(256) k_chol_update(float* __restrict__ A, int lda, int n, int j0, unsigned* status) {
   __shared__ float Pi[64][33];
   __shared__ float Pj[64][33];
   const int j1 = j0 + 32;
   const int b = blockIdx.x;
-  int ti = static_cast<int>((sqrt(8.0 * b + 1.0) - 1.0) * 0.5);
+  int ti = static_cast<int>((sqrtf(8.0f * b + 1.0f) - 1.0f) * 0.5f);
   while ((ti + 1) * (ti + 2) / 2 <= b) ++ti;
   while (ti * (ti + 1) / 2 > b) --ti;
   const int tj = b - ti * (ti + 1) / 2;
   const int r0 = j1 + ti * 64, c0 = j1 + tj * 64;
-  for (int e = threadIdx.x; e < 64 * 32; e += 256) {
-    const int r = e >> 5, t = e & 31;
-    Pi[r][t] = (r0 + r < n) ? A[static_cast<long long>(r0 + r) * lda + j0 + t] : 0.f;
-    Pj[r][t] = (c0 + r < n) ? A[static_cast<long long>(c0 + r) * lda + j0 + t] : 0.f;
+  for (int e = threadIdx.x; e < 64 * 8; e += 256) {
+    const int r = e >> 3, t = 4 * (e & 7);
+    float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+    if (r0 + r < n) u = *reinterpret_cast<const float4*>(A + static_cast<long long>(r0 + r) * lda + j0 + t);
+    if (c0 + r < n) v = *reinterpret_cast<const float4*>(A + static_cast<long long>(c0 + r) * lda + j0 + t);
+    Pi[r][t] = u.x, Pi[r][t + 1] = u.y, Pi[r][t + 2] = u.z, Pi[r][t + 3] = u.w;
+    Pj[r][t] = v.x, Pj[r][t + 1] = v.y, Pj[r][t + 2] = v.z, Pj[r][t + 3] = v.w;
   }
-  __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float old[4][4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int i = r0 + ty + 16 * u, j = c0 + tx + 16 * v;
+      old[u][v] = (i < n && j <= i) ? A[static_cast<long long>(i) * lda + j] : 0.f;
+    }
+  __syncthreads();
   float acc[4][4] = {};
 #pragma unroll 8
   for (int t = 0; t < 32; ++t) {
@@ -559,16 +731,29 @@ __global__ void __launch_bounds__(256) k_chol_update(float* __restrict__ A, int 
 #pragma unroll
       for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], bb[v], acc[u][v]);
   }
+  if (b == 0) __syncthreads();  // every thread is done with Pi
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int i = r0 + ty + 16 * u;
-    if (i >= n) continue;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const int j = c0 + tx + 16 * v;
-      if (j <= i) A[static_cast<long long>(i) * lda + j] -= acc[u][v];
+      const float x = old[u][v] - acc[u][v];
+      if (b == 0 && u < 2 && v < 2) Pi[ty + 16 * u][tx + 16 * v] = x;
+      if (i < n && j <= i && !(b == 0 && u < 2 && v < 2)) A[static_cast<long long>(i) * lda + j] = x;
     }
   }
+  if (b != 0) return;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x, nb = min(32, n - j1);
+  float a[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) a[j] = (lane < nb && j <= lane) ? Pi[lane][j] : 0.f;
+  chol_block(a, lane, nb, status);
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (lane < nb && j < nb) A[static_cast<long long>(j1 + lane) * lda + j1 + j] = a[j];
 }
 
 // ---- inverse of a lower-triangular matrix (fp32), 32 x 32 blocks; Li zeroed first
@@ -594,47 +779,63 @@ __global__ void k_trinv_diag(const float* __restrict__ L, int lda, float* __rest
   for (int i = c; i < nb; ++i) Li[static_cast<long long>(j0 + i) * ldi + j0 + c] = x[i];
 }
 
-// Blocks at distance d below the diagonal: Li[I][J] = -Li[I][I] sum_{K=J}^{I-1} L[I][K] Li[K][J],
-// I = J + d (grid = number of such blocks); 256 threads, 4 entries each.
-__global__ void __launch_bounds__(256) k_trinv_off(const float* __restrict__ L, int lda, float* __restrict__ Li,
-                                                   int ldi, int n, int d) {
-  __shared__ float As[32][33];
-  __shared__ float Bs[32][33];
-  const int J = blockIdx.x, I = J + d;
-  const int i0 = I * 32, j0 = J * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // ty 0..7: rows ty + 8u
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int K = J; K < I; ++K) {
-    const int k0 = K * 32;
-    for (int e = threadIdx.x; e < 1024; e += 256) {
-      const int r = e >> 5, c = e & 31;
-      As[r][c] = (i0 + r < n) ? L[static_cast<long long>(i0 + r) * lda + k0 + c] : 0.f;
-      Bs[r][c] = Li[static_cast<long long>(k0 + r) * ldi + j0 + c];
+// Blocks below the diagonal: Li[I][J] = -Li[I][I] sum_{K=J}^{I-1} L[I][K] Li[K][J].
+// The columns of an inverse are independent: a block of 256 threads takes w = 8
+// columns of block column J (4 where n x 8 floats exceed the shared memory) and goes
+// down its rows, the columns so far in shared memory. n is a multiple of 32; two
+// blocks of L are fetched ahead.
+__global__ void __launch_bounds__(256) k_trinv_cols(const float* __restrict__ L, int lda, float* __restrict__ Li,
+                                                    int ldi, int n, int w) {
+  extern __shared__ float col[];  // [row - 32 J][w]
+  __shared__ float As[2][32][33];
+  __shared__ float Ts[32][8];
+  const int J = blockIdx.x, c0 = J * 32 + blockIdx.y * w;
+  const int r = threadIdx.x >> 3, c = threadIdx.x & 7;      // this thread's row and column of a block
+  const int lr = threadIdx.x >> 3, lc = 4 * (threadIdx.x & 7);  // its 16 bytes of a 32 x 32 block
+  const bool mine = c < w;
+  if (mine) col[r * w + c] = Li[static_cast<long long>(J * 32 + r) * ldi + c0 + c];
+  const int nblk = n / 32;
+  // the blocks in the order they are used: L[I][J .. I-1], then Li[I][I]
+  auto fetch = [&](int I, int K) {
+    return K < I ? *reinterpret_cast<const float4*>(L + static_cast<long long>(I * 32 + lr) * lda + K * 32 + lc)
+                 : *reinterpret_cast<const float4*>(Li + static_cast<long long>(I * 32 + lr) * ldi + I * 32 + lc);
+  };
+  auto after = [&](int& I, int& K) {
+    if (++K > I) {
+      ++I;
+      K = J;
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int t = 0; t < 32; ++t) {
-      const float bv = Bs[t][tx];
+  };
+  int fI = J + 1, fK = J;
+  float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f), f1 = f0;
+  if (fI < nblk) f0 = fetch(fI, fK);
+  after(fI, fK);
+  if (fI < nblk) f1 = fetch(fI, fK);
+  after(fI, fK);
+  int buf = 0;
+  for (int I = J + 1; I < nblk; ++I) {
+    float acc = 0.f;
+    for (int K = J; K <= I; ++K, buf ^= 1) {
+      float(*A)[33] = As[buf];
+      A[lr][lc] = f0.x, A[lr][lc + 1] = f0.y, A[lr][lc + 2] = f0.z, A[lr][lc + 3] = f0.w;
+      if (K == I) Ts[r][c] = acc;
+      f0 = f1;
+      if (fI < nblk) f1 = fetch(fI, fK);
+      after(fI, fK);
+      __syncthreads();
+      if (!mine) continue;
+      if (K < I) {
+        const float* b = col + (K - J) * 32 * w + c;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] = fmaf(As[ty + 8 * u][t], bv, acc[u]);
+        for (int t = 0; t < 32; ++t) acc = fmaf(A[r][t], b[w * t], acc);
+      } else {
+        float v = 0.f;
+#pragma unroll
+        for (int t = 0; t < 32; ++t) v = fmaf(A[r][t], Ts[t][c], v);
+        col[(I - J) * 32 * w + r * w + c] = -v;
+        Li[static_cast<long long>(I * 32 + r) * ldi + c0 + c] = -v;
+      }
     }
-    __syncthreads();
-  }
-  // T = acc (rows ty + 8u, column tx) -> Bs; Li[I][I] -> As
-#pragma unroll
-  for (int u = 0; u < 4; ++u) Bs[ty + 8 * u][tx] = acc[u];
-  for (int e = threadIdx.x; e < 1024; e += 256) {
-    const int r = e >> 5, c = e & 31;
-    As[r][c] = (i0 + r < n && i0 + c < n) ? Li[static_cast<long long>(i0 + r) * ldi + i0 + c] : 0.f;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = ty + 8 * u;
-    float v = 0.f;
-#pragma unroll 8
-    for (int t = 0; t < 32; ++t) v = fmaf(As[r][t], Bs[t][tx], v);
-    if (i0 + r < n) Li[static_cast<long long>(i0 + r) * ldi + j0 + tx] = -v;
   }
 }
 
@@ -695,7 +896,7 @@ int pca_block(int k) { return rup(k + std::max(64, k / 4), 32); }
 bool use_subspace(int nn, int k) { return nn > 1024 && pca_block(k) < nn; }
 
 struct DenseLayout {
-  size_t A, Vt, cs, mu, sel, red, Pr, total;
+  size_t A, A2, Vt, cs, mu, sel, red, Pr, total;
 };
 
 DenseLayout dense_layout(int n, int m, int k) {
@@ -704,8 +905,9 @@ DenseLayout dense_layout(int n, int m, int k) {
   size_t o = 0;
   auto take = [&](size_t b) { const size_t at = o; o += al256(b); return at; };
   L.A = take(nn * nn * 8);
+  L.A2 = take(nn * nn * 8);
   L.Vt = take(nn * nn * 8);
-  L.cs = take((nn / 2 + 1) * 2 * 8);
+  L.cs = take((nn / 2 + 1) * 4 * 8);
   L.mu = take(nn * 8);
   L.sel = take(nn * 4);
   L.red = take(4 * 8);
@@ -723,7 +925,7 @@ struct SubLayout {
   size_t YTh, YTl, CTh, CTl;     // transposed splits [nn][p8]
   size_t G32, Li32, Sh, Sl;      // [p][p4] fp32, splits [p][p8]
   size_t rs, shift, theta, resid;
-  size_t H64, V64, cs, mu, sel, red;
+  size_t H64, H64b, V64, cs, mu, sel, red;
   size_t Pr;                     // Gram route: raw directions [k][m4] fp32
   size_t total;
 };
@@ -772,8 +974,9 @@ SubLayout sub_layout(int n, int m, int k, bool with_z) {
   L.theta = take(p * 4);
   L.resid = take(16);
   L.H64 = take(p * p * 8);
+  L.H64b = take(p * p * 8);
   L.V64 = take(p * p * 8);
-  L.cs = take((p / 2 + 1) * 2 * 8);
+  L.cs = take((p / 2 + 1) * 4 * 8);
   L.mu = take(p * 8);
   L.sel = take(p * 4);
   L.red = take(4 * 8);
@@ -809,26 +1012,33 @@ unsigned grid_for(long long tot) {
   return static_cast<unsigned>(std::max<long long>(1, std::min<long long>((tot + 255) / 256, 152LL * 16)));
 }
 
-// Cyclic Jacobi on A (fp64, n x n, overwritten by its diagonal form); Vt = eigenvectors as rows.
-int jacobi_eigen(double* A, double* Vt, int nn, double* cs, double* red, cudaStream_t st, int max_sweeps) {
+// Cyclic Jacobi on A (fp64, n x n, overwritten by its diagonal form; A2 of the same
+// size); Vt = eigenvectors as rows. cs: 2 (n + 1) doubles; red: 4 doubles.
+int jacobi_eigen(double* A, double* A2, double* Vt, int nn, double* cs, double* red, unsigned* status, cudaStream_t st,
+                 int max_sweeps) {
   const int np = nn + (nn & 1);
   {
     const long long tot = static_cast<long long>(nn) * nn;
     k_eye<<<static_cast<unsigned>((tot + 255) / 256), 256, 0, st>>>(Vt, nn);
     PCA_TRY(cudaGetLastError());
   }
-  const size_t apply_smem = 2 * static_cast<size_t>(nn) * sizeof(double);
-  PCA_TRY(cudaFuncSetAttribute(k_jacobi_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(apply_smem)));
+  int dev = 0, sms = 0;
+  PCA_TRY(cudaGetDevice(&dev));
+  PCA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  double* cur = A;
+  double* oth = A2;
+  double2* cs0 = reinterpret_cast<double2*>(cs);
+  double2* cs1 = cs0 + np / 2;
+  unsigned* count = reinterpret_cast<unsigned*>(red + 2);
   double prev_off = -1.0;
   for (int sweep = 0; sweep < max_sweeps && nn > 1; ++sweep) {
-    for (int s = 0; s < np - 1; ++s) {
-      k_jacobi_params<<<(np / 2 + 127) / 128, 128, 0, st>>>(A, nn, np, s, cs);
-      k_jacobi_apply<<<np / 2, 256, apply_smem, st>>>(A, Vt, nn, np, s, cs);
-    }
-    PCA_TRY(cudaGetLastError());
-    PCA_TRY(cudaMemsetAsync(red, 0, 2 * sizeof(double), st));
-    k_offnorm<<<304, 256, 0, st>>>(A, nn, red);
+    PCA_TRY(cudaMemsetAsync(red, 0, 4 * sizeof(double), st));
+    int n = nn, npv = np;
+    void* args[] = {&cur, &oth, &Vt, &n, &npv, &cs0, &cs1, &count, &status};
+    PCA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_jacobi_sweep), dim3(sms), dim3(kJacThreads), args,
+                                        0, st));
+    std::swap(cur, oth);  // np - 1 steps, an odd number
+    k_offnorm<<<304, 256, 0, st>>>(cur, nn, red);
     PCA_TRY(cudaGetLastError());
     double h[2];
     PCA_TRY(cudaMemcpyAsync(h, red, sizeof(h), cudaMemcpyDeviceToHost, st));
@@ -838,11 +1048,13 @@ int jacobi_eigen(double* A, double* Vt, int nn, double* cs, double* red, cudaStr
     if (prev_off >= 0.0 && sweep >= 4 && off > 0.5 * prev_off) break;  // rounding floor
     prev_off = off;
   }
+  if (cur != A)
+    PCA_TRY(cudaMemcpyAsync(A, cur, static_cast<size_t>(nn) * nn * sizeof(double), cudaMemcpyDeviceToDevice, st));
   return EOGP_OK;
 }
 
 int fit_dense(const float* Z, int n, int m, int ldz, int k, void* Pt, int ld_pt, int pt_dtype, float* eig,
-              char* ws, cudaStream_t st, const double* C_in, int ldc) {
+              char* ws, unsigned* status, cudaStream_t st, const double* C_in, int ldc) {
   const DenseLayout L = dense_layout(C_in ? m : n, m, k);
   double* A = reinterpret_cast<double*>(ws + L.A);
   double* Vt = reinterpret_cast<double*>(ws + L.Vt);
@@ -864,7 +1076,7 @@ int fit_dense(const float* Z, int n, int m, int ldz, int k, void* Pt, int ld_pt,
     // A = Z^T Z / n (m x m): A(i,j) = sum_r Z[r][i] Z[r][j]
     PCA_TRY(gemm_f64acc<float>(m, m, n, 1.0 / n, Z, 1, ldz, Z, 1, ldz, A, m, st));
   }
-  if (int rc = jacobi_eigen(A, Vt, nn, cs, red, st, 40)) return rc;
+  if (int rc = jacobi_eigen(A, reinterpret_cast<double*>(ws + L.A2), Vt, nn, cs, red, status, st, 40)) return rc;
   k_rank<<<(nn + 255) / 256, 256, 0, st>>>(A, nn, k, mu, sel);
   PCA_TRY(cudaGetLastError());
   const int bf = pt_dtype == EOGP_BF16 ? 1 : 0;
@@ -911,20 +1123,20 @@ int chol_qr_pass(const SubLayout& L, char* w, const float* Y32, float* X32, floa
   k_diag_shift<<<1, 256, 0, st>>>(G, L.p4, p, rel, shift);
   k_add_diag<<<(p + 255) / 256, 256, 0, st>>>(G, L.p4, p, shift);
   PCA_TRY(cudaGetLastError());
-  for (int j0 = 0; j0 < p; j0 += 32) {
-    k_chol_diag<<<1, dim3(32, 32), 0, st>>>(G, L.p4, p, j0, status);
-    const int below = p - (j0 + 32);
-    if (below > 0) {
-      k_chol_panel<<<(below + 127) / 128, 128, 0, st>>>(G, L.p4, p, j0);
-      const int nt = (below + 63) / 64;
-      k_chol_update<<<nt * (nt + 1) / 2, 256, 0, st>>>(G, L.p4, p, j0);
-    }
+  k_chol_diag<<<1, 32, 0, st>>>(G, L.p4, p, 0, status);
+  for (int j0 = 0; j0 + 32 < p; j0 += 32) {
+    const int below = p - (j0 + 32), nt = (below + 63) / 64;
+    k_chol_panel<<<(below + 63) / 64, 64, 0, st>>>(G, L.p4, p, j0);
+    k_chol_update<<<nt * (nt + 1) / 2, 256, 0, st>>>(G, L.p4, p, j0, status);
   }
   PCA_TRY(cudaGetLastError());
   PCA_TRY(cudaMemsetAsync(Li, 0, static_cast<size_t>(p) * L.p4 * 4, st));
   const int nblk = (p + 31) / 32;
   k_trinv_diag<<<nblk, 32, 0, st>>>(G, L.p4, Li, L.p4, p);
-  for (int d = 1; d < nblk; ++d) k_trinv_off<<<nblk - d, 256, 0, st>>>(G, L.p4, Li, L.p4, p, d);
+  const int cw = static_cast<size_t>(p) * 8 * sizeof(float) <= 200 * 1024 ? 8 : 4;
+  const size_t cols = static_cast<size_t>(p) * cw * sizeof(float);
+  PCA_TRY(cudaFuncSetAttribute(k_trinv_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(cols)));
+  k_trinv_cols<<<dim3(nblk, 32 / cw), 256, cols, st>>>(G, L.p4, Li, L.p4, p, cw);
   PCA_TRY(cudaGetLastError());
   k_split_rows<<<grid_for(static_cast<long long>(p) * L.p8), 256, 0, st>>>(Li, L.p4, p, p, nullptr, Sh, Sl, L.p8);
   PCA_TRY(cudaGetLastError());
@@ -982,8 +1194,8 @@ int rayleigh_ritz(const SubLayout& L, char* w, int k, unsigned* status, cudaStre
   PCA_TRY(launch_tc_gemm_hl(p, p, nn, Yh, Yl, L.nn8, YTh, YTl, L.nn8, H, L.p4, 1.0f, status, st));
   k_sym_f64<<<grid_for(static_cast<long long>(p) * p), 256, 0, st>>>(H, L.p4, p, H64);
   PCA_TRY(cudaGetLastError());
-  if (int rc = jacobi_eigen(H64, V64, p, reinterpret_cast<double*>(w + L.cs), reinterpret_cast<double*>(w + L.red),
-                            st, 40))
+  if (int rc = jacobi_eigen(H64, reinterpret_cast<double*>(w + L.H64b), V64, p, reinterpret_cast<double*>(w + L.cs),
+                            reinterpret_cast<double*>(w + L.red), status, st, 40))
     return rc;
   k_rank<<<(p + 255) / 256, 256, 0, st>>>(H64, p, p, mu, sel);
   k_ritz_rows<<<p, 256, 0, st>>>(V64, p, sel, mu, S32, L.p4, theta);
@@ -1092,7 +1304,7 @@ int fit_pca_device(const float* Z, int n, int m, int ldz, int k, void* Pt, int l
   const int nn = C_in ? m : std::min(n, m);
   char* w = static_cast<char*>(ws);
   if (use_subspace(nn, k)) return fit_subspace(Z, n, m, ldz, k, Pt, ld_pt, pt_dtype, eig, w, status, st, C_in, ldc);
-  return fit_dense(Z, n, m, ldz, k, Pt, ld_pt, pt_dtype, eig, w, st, C_in, ldc);
+  return fit_dense(Z, n, m, ldz, k, Pt, ld_pt, pt_dtype, eig, w, status, st, C_in, ldc);
 }
 
 cudaError_t second_moment_device(const float* Z, int n, int m, int ldz, double* C, int ldc, int accumulate,
