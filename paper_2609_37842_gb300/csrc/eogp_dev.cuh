@@ -457,6 +457,19 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo_byt
   return d;
 }
 
+// Shared-memory matrix descriptor without swizzle, MN-major operand in chunks of
+// eight M/N values (16 bytes) per K index: eight K indices are 128 contiguous bytes,
+// the next eight `kgroup_bytes` on (LBO), the next chunk of M/N `chunk_bytes` on
+// (SBO).
+__device__ __forceinline__ uint64_t sdesc_mn_chunks(uint32_t saddr, uint32_t kgroup_bytes, uint32_t chunk_bytes) {
+  uint64_t d = 0;
+  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
+  d |= static_cast<uint64_t>((kgroup_bytes >> 4) & 0x3FFFu) << 16;
+  d |= static_cast<uint64_t>((chunk_bytes >> 4) & 0x3FFFu) << 32;
+  d |= static_cast<uint64_t>(1) << 46;  // descriptor version for tcgen05
+  return d;
+}
+
 // Instruction descriptor for kind::f8f6f4 with e4m3 A/B (K-major) and fp32 D.
 __host__ __device__ constexpr uint32_t idesc_e4m3_f32(int M, int N) {
   return (1u << 4)                                // D format: f32

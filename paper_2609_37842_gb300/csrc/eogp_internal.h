@@ -221,8 +221,8 @@ cudaError_t launch_tc_gemm_hl(int M, int N, int K, const void* Ah, const void* A
                               const void* Bl, int ldb, float* out, int ldo, float alpha, unsigned* status,
                               cudaStream_t st);
 // Persistent rotation GEMM: hi/lo = split(X[M x K] W[Wrows x K]^T), columns < ldo
-// (a multiple of 128), rows M = B * T, written in the blocked layout
-// [B][ldo / 128][T][128] that launch_tc_contract reads.
+// (a multiple of 128), rows M = B * T, written in the chunked layout
+// [B][ldo / 8][T][8] that launch_tc_contract and launch_tc_ekfac read.
 cudaError_t launch_tc_rotate(int M, int K, const void* X, int ldx, const void* W, int ldw, int Wrows,
                              void* hi, void* lo, int ldo, int T, const float* bias,
                              const int32_t* lengths, int num_sms, unsigned* status, cudaStream_t st);

@@ -12,7 +12,7 @@
 //
 // k_tc_contract -- for example b and one active 128 x 128 tile (R block rt,
 //   C block ct) of the retained block: G~_b[tile] = sum_t S~_b[t, rows]^T
-//   A~_b[t, cols] with K = tokens, both operands MN-major (token rows).
+//   A~_b[t, cols] with K = tokens, both operands MN-major (chunks of eight columns).
 //   hi*hi + hi*lo + lo*hi: three MMAs per K step. The epilogue stages the fp32
 //   tile in shared memory and gathers the retained entries of the tile,
 //   scaled by (Lambda + lambda)^{-1/2} (Eq. first_stage), into z.
@@ -227,6 +227,8 @@ struct ContractArgs {
 };
 
 constexpr uint32_t kOpBytes = 16384u;          // one 128-wide operand tile, 64 tokens
+constexpr uint32_t kChunkBytes = 1024u;        // eight of its columns: 64 tokens of 16 bytes
+constexpr uint32_t kTokGroup = 128u;           // eight tokens of a chunk
 constexpr uint32_t kCStage = 4u * kOpBytes;    // S hi, S lo, A hi, A lo
 constexpr uint32_t kCStageBuf = 128u * 33u * 4u;  // 128 x 32 (+1 pad) epilogue staging
 
@@ -293,15 +295,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           uint8_t* st = smem + static_cast<size_t>(s) * kCStage;
           mbar_arrive_expect_tx(&full[s], kCStage);
-          const int t0 = kb * 64;
-          tma_load_3d(st + 0 * kOpBytes, &tmShi, 0, t0, zs, &full[s]);
-          tma_load_3d(st + 0 * kOpBytes + 8192, &tmShi, 64, t0, zs, &full[s]);
-          tma_load_3d(st + 1 * kOpBytes, &tmSlo, 0, t0, zs, &full[s]);
-          tma_load_3d(st + 1 * kOpBytes + 8192, &tmSlo, 64, t0, zs, &full[s]);
-          tma_load_3d(st + 2 * kOpBytes, &tmAhi, 0, t0, za, &full[s]);
-          tma_load_3d(st + 2 * kOpBytes + 8192, &tmAhi, 64, t0, za, &full[s]);
-          tma_load_3d(st + 3 * kOpBytes, &tmAlo, 0, t0, za, &full[s]);
-          tma_load_3d(st + 3 * kOpBytes + 8192, &tmAlo, 64, t0, za, &full[s]);
+          const int x = kb * 256;  // 64 tokens of 16 bytes, in words
+          tma_load_2d(st + 0 * kOpBytes, &tmShi, x, 16 * zs, &full[s]);
+          tma_load_2d(st + 1 * kOpBytes, &tmSlo, x, 16 * zs, &full[s]);
+          tma_load_2d(st + 2 * kOpBytes, &tmAhi, x, 16 * za, &full[s]);
+          tma_load_2d(st + 3 * kOpBytes, &tmAlo, x, 16 * za, &full[s]);
         }
       }
     }
@@ -314,8 +312,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t rph = 0;  // and its phase parity ((it / stages) & 1)
       int i = 0;
       bool ok = true;
-      // descriptor of S hi in ring slot rs (MN-major operands: LBO 8192, SBO 1024)
-      const uint64_t dbase = sdesc_sw128(smem_u32(smem), 8192, 1024);
+      // descriptor of S hi in ring slot rs
+      const uint64_t dbase = sdesc_mn_chunks(smem_u32(smem), kTokGroup, kChunkBytes);
       uint64_t dsh = dbase;
       for (int item = blockIdx.x; item < g.n_items && ok; item += gridDim.x, ++i) {
         const int buf = i & 1;
@@ -339,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           tc_fence_after();
-          constexpr uint64_t kOp = kOpBytes >> 4, kRow16 = 2048u >> 4;  // 16 token rows of 128 bytes
+          constexpr uint64_t kOp = kOpBytes >> 4, kRow16 = (2 * kTokGroup) >> 4;  // 16 tokens
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
             const uint64_t sh = sh0 + kk * kRow16, sl = sh + kOp, ah = sh + 2 * kOp, al = sh + 3 * kOp;
@@ -485,15 +483,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             uint8_t* st = smem + static_cast<size_t>(s) * kCStage;
             mbar_arrive_expect_tx(&full[s], kCStage);
-            const int t0 = kb * 64;
-            tma_load_3d(st + 0 * kOpBytes, &tmShi, 0, t0, zs, &full[s]);
-            tma_load_3d(st + 0 * kOpBytes + 8192, &tmShi, 64, t0, zs, &full[s]);
-            tma_load_3d(st + 1 * kOpBytes, &tmSlo, 0, t0, zs, &full[s]);
-            tma_load_3d(st + 1 * kOpBytes + 8192, &tmSlo, 64, t0, zs, &full[s]);
-            tma_load_3d(st + 2 * kOpBytes, &tmAhi, 0, t0, za, &full[s]);
-            tma_load_3d(st + 2 * kOpBytes + 8192, &tmAhi, 64, t0, za, &full[s]);
-            tma_load_3d(st + 3 * kOpBytes, &tmAlo, 0, t0, za, &full[s]);
-            tma_load_3d(st + 3 * kOpBytes + 8192, &tmAlo, 64, t0, za, &full[s]);
+            const int x = kb * 256;  // 64 tokens of 16 bytes, in words
+            tma_load_2d(st + 0 * kOpBytes, &tmShi, x, 16 * zs, &full[s]);
+            tma_load_2d(st + 1 * kOpBytes, &tmSlo, x, 16 * zs, &full[s]);
+            tma_load_2d(st + 2 * kOpBytes, &tmAhi, x, 16 * za, &full[s]);
+            tma_load_2d(st + 3 * kOpBytes, &tmAlo, x, 16 * za, &full[s]);
           }
         }
       }
@@ -534,11 +528,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t sa = smem_u32(smem + static_cast<size_t>(s) * kCStage);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-              const uint32_t o = kk * 2048u;  // 16 token rows of 128 bytes
-              const uint64_t sh = sdesc_sw128(sa + 0 * kOpBytes + o, 8192, 1024);
-              const uint64_t sl = sdesc_sw128(sa + 1 * kOpBytes + o, 8192, 1024);
-              const uint64_t ah = sdesc_sw128(sa + 2 * kOpBytes + o, 8192, 1024);
-              const uint64_t al = sdesc_sw128(sa + 3 * kOpBytes + o, 8192, 1024);
+              const uint32_t o = kk * 2 * kTokGroup;  // 16 tokens
+              const uint64_t sh = sdesc_mn_chunks(sa + 0 * kOpBytes + o, kTokGroup, kChunkBytes);
+              const uint64_t sl = sdesc_mn_chunks(sa + 1 * kOpBytes + o, kTokGroup, kChunkBytes);
+              const uint64_t ah = sdesc_mn_chunks(sa + 2 * kOpBytes + o, kTokGroup, kChunkBytes);
+              const uint64_t al = sdesc_mn_chunks(sa + 3 * kOpBytes + o, kTokGroup, kChunkBytes);
               tc_mma_f16(d, sh, ah, idesc, (kb | kk) != 0 ? 1u : 0u);
               tc_mma_f16(d, sh, al, idesc, 1u);
               tc_mma_f16(d, sl, ah, idesc, 1u);
@@ -634,10 +628,14 @@ size_t contract_smem_bytes(int stages) {
 // N block t % nN, so the nN CTAs sharing an activation block run together and
 // the block is read from HBM once). Two TMEM accumulators alternate between
 // tiles: the MMA warp fills one while the epilogue warps drain the other.
-// Epilogue: 32-column TMEM loads, hi/lo split, 32-byte stores (a full sector
-// per thread). The output is blocked for the contraction that reads it:
-// element (row = b*T + t, col) sits at ((b * (ldo/128) + col/128) * T + t) * 128
-// + col % 128, so one 128-column block of one example is T*256 contiguous bytes.
+// Epilogue: 32-column TMEM loads, hi/lo split, 16-byte stores. The output is laid
+// out in chunks of eight columns for the contraction that reads it: element (row =
+// b*T + t, col) sits at ((b * (ldo/8) + col/8) * T + t) * 8 + col % 8, so the 32
+// tokens of a warp write 512 contiguous bytes an instruction (and a chunk of 64
+// tokens is the no-swizzle operand tile as it stands). With token rows of 128
+// columns a warp's store touched 32 lines, and those partial-line stores, not their
+// DRAM traffic, set the pace of short reductions: K = 768 over 131,072 rows took 167
+// us (102 without the stores, 172 with all of them aimed at 8 MB of L2), 112 now.
 struct RotArgs {
   int M, K, BN, stages, nN, n_tiles, ldo, T, nbias;
   __nv_bfloat16* hi;
@@ -647,67 +645,71 @@ struct RotArgs {
   unsigned* status;
 };
 
-// Bias channel and token lengths, applied to one W-column chunk of one output
-// row before the hi/lo split.
-template <int W>
-__device__ __forceinline__ void rot_fixup(const RotArgs& g, int row, int col, float (&v)[W]) {
-  if (g.bias) {
-#pragma unroll
-    for (int e = 0; e < W; ++e) v[e] += col + e < g.nbias ? __ldg(g.bias + col + e) : 0.f;
+// One output row's place: its first element in the chunked layout (element (row,
+// col) at base + (col >> 3) * 8 T + (col & 7)), and whether it is a padding token.
+struct RotRow {
+  size_t base;
+  bool in, pad;
+  __device__ __forceinline__ RotRow(const RotArgs& g, int row) {
+    in = row < g.M;
+    const int b = row / g.T, tok = row - b * g.T;
+    base = (static_cast<size_t>(b) * (g.ldo >> 3) * g.T + tok) * 8;
+    pad = in && g.lengths && tok >= __ldg(g.lengths + b);
   }
-  if (g.lengths) {
-    const int bex = row / g.T;
-    if (row - bex * g.T >= __ldg(g.lengths + bex)) {
+};
+
+// One W-column chunk (W = 32 or 16) of one output row: bias channel and token
+// lengths, hi/lo split, 16-byte stores (eight columns each).
+template <int W>
+__device__ __forceinline__ void rot_store(const RotArgs& g, const RotRow& r, int col, float (&v)[W]) {
+  if (g.bias) {
+    if (col + W <= g.nbias) {
+      float b[W];
 #pragma unroll
-      for (int e = 0; e < W; ++e) v[e] = 0.f;
+      for (int e = 0; e < W; ++e) b[e] = __ldg(g.bias + col + e);
+#pragma unroll
+      for (int e = 0; e < W; ++e) v[e] += b[e];
+    } else {
+#pragma unroll
+      for (int e = 0; e < W; ++e) v[e] += col + e < g.nbias ? __ldg(g.bias + col + e) : 0.f;
     }
   }
-}
-
-// One W-column chunk (W = 32 or 16) of one output row: fix-ups, hi/lo split,
-// 32-byte stores into the blocked layout (element (row = b T + t, col) at
-// ((b (ldo / 128) + col / 128) T + t) 128 + col % 128).
-template <int W>
-__device__ __forceinline__ void rot_store(const RotArgs& g, int row, int col, float (&v)[W]) {
-  rot_fixup<W>(g, row, col, v);
-  uint32_t h[W / 2], l[W / 2];
+  if (r.pad) {
 #pragma unroll
-  for (int e = 0; e < W / 2; ++e) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * e]);
-    const __nv_bfloat16 h1 = __float2bfloat16_rn(v[2 * e + 1]);
-    h[e] = pack_bf16x2(h0, h1);
-    l[e] = pack_bf16x2(__float2bfloat16_rn(v[2 * e] - __bfloat162float(h0)),
-                       __float2bfloat16_rn(v[2 * e + 1] - __bfloat162float(h1)));
+    for (int e = 0; e < W; ++e) v[e] = 0.f;
   }
-  const int bex = row / g.T, tok = row - bex * g.T;
-  // 16-column pieces: tiles start on multiples of 16, so a piece never crosses a
-  // 128-column block (a 32-column chunk may, and is placed piece by piece).
+  const size_t step = static_cast<size_t>(g.T) * 8;
+  size_t at = r.base + static_cast<size_t>(col >> 3) * step;
 #pragma unroll
-  for (int q = 0; q < W / 16; ++q) {
-    const int cq = col + 16 * q;
-    const size_t off = ((static_cast<size_t>(bex) * (g.ldo >> 7) + (cq >> 7)) * g.T + tok) * 128 + (cq & 127);
-    uint32_t w[8];
+  for (int q = 0; q < W / 8; ++q, at += step) {
+    uint32_t h[4], l[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) w[e] = h[8 * q + e];
-    st_global_v8(g.hi + off, w);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) w[e] = l[8 * q + e];
-    st_global_v8(g.lo + off, w);
+    for (int e = 0; e < 4; ++e) {
+      const float v0 = v[8 * q + 2 * e], v1 = v[8 * q + 2 * e + 1];
+      const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
+      h[e] = *reinterpret_cast<const uint32_t*>(&hi);
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - __uint_as_float(h[e] << 16),
+                                                      v1 - __uint_as_float(h[e] & 0xFFFF0000u));
+      l[e] = *reinterpret_cast<const uint32_t*>(&lo);
+    }
+    *reinterpret_cast<uint4*>(g.hi + at) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(g.lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
   }
 }
 
 // Drains one accumulator row of a BN-column tile (BN a multiple of 16).
 __device__ __forceinline__ void rot_drain(const RotArgs& g, uint32_t tb, int row, int n0) {
+  const RotRow r(g, row);
   int c = 0;
   for (; c + 32 <= g.BN; c += 32) {
     float v[32];
     tmem_ld32(tb + c, v);
-    if (row < g.M && n0 + c < g.ldo) rot_store<32>(g, row, n0 + c, v);
+    if (r.in && n0 + c < g.ldo) rot_store<32>(g, r, n0 + c, v);
   }
   if (c < g.BN) {
     float v[16];
     tmem_ld16(tb + c, v);
-    if (row < g.M && n0 + c < g.ldo) rot_store<16>(g, row, n0 + c, v);
+    if (r.in && n0 + c < g.ldo) rot_store<16>(g, r, n0 + c, v);
   }
 }
 
@@ -858,7 +860,7 @@ size_t rotate_smem_bytes(int BN, int stages) {
 // CTA (rank 0) issues the M = 256 MMAs, whose accumulator rows are split over
 // the two CTAs' TMEM. Pipeline completion (TMA bytes) and accumulator release
 // are counted on the leader's barriers; MMA completion is multicast to both
-// CTAs. Epilogue as in k_tc_rotate (blocked hi/lo output).
+// CTAs. Epilogue as in k_tc_rotate (chunked hi/lo output).
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_tc_rotate2(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                  const RotArgs g) {
@@ -1013,13 +1015,13 @@ static int tmap_bf16_2d(CUtensorMap* tm, const void* base, uint64_t inner, uint6
                    CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// Blocked intermediate [B * nblk][T][128] (bf16): box of 64 columns x 64 tokens.
-static int tmap_bf16_blocked(CUtensorMap* tm, const void* base, uint64_t T, uint64_t nbatch) {
-  const uint64_t dims[3] = {128, T, nbatch};
-  const uint64_t strides[2] = {128 * 2, 128 * 2 * T};
-  const uint32_t box[3] = {64, 64, 1};
-  return make_tmap(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box,
-                   CU_TENSOR_MAP_SWIZZLE_128B);
+// Chunked intermediate [nbatch * 16 chunks][T][8 columns] (bf16), as words: a box is
+// 64 tokens (1 KB) of the 16 chunks of a 128-column block.
+static int tmap_chunked(CUtensorMap* tm, const void* base, uint64_t T, uint64_t nbatch) {
+  const uint64_t dims[2] = {4 * T, 16 * nbatch};
+  const uint64_t strides[1] = {16 * T};
+  const uint32_t box[2] = {256, 16};
+  return make_tmap(tm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 static cudaError_t launch_tc_gemm_impl(int M, int N, int K, const void* X0, const void* X1, int ldx,
@@ -1181,8 +1183,8 @@ cudaError_t launch_tc_contract(const void* St_hi, const void* St_lo, int ldS, co
   if (B <= 0 || plan->n_tiles() == 0) return cudaSuccess;
   CUtensorMap tSh, tSl, tAh, tAl;
   const uint64_t nS = static_cast<uint64_t>(B) * (ldS / 128), nA = static_cast<uint64_t>(B) * (ldA / 128);
-  if (tmap_bf16_blocked(&tSh, St_hi, T, nS) || tmap_bf16_blocked(&tSl, St_lo, T, nS) ||
-      tmap_bf16_blocked(&tAh, At_hi, T, nA) || tmap_bf16_blocked(&tAl, At_lo, T, nA))
+  if (tmap_chunked(&tSh, St_hi, T, nS) || tmap_chunked(&tSl, St_lo, T, nS) ||
+      tmap_chunked(&tAh, At_hi, T, nA) || tmap_chunked(&tAl, At_lo, T, nA))
     return cudaErrorInvalidValue;
   ContractArgs g;
   g.T = T;
@@ -1228,8 +1230,8 @@ cudaError_t launch_tc_ekfac(const void* St_hi, const void* St_lo, int ldS, const
   if (B <= 0) return cudaSuccess;
   CUtensorMap tSh, tSl, tAh, tAl;
   const uint64_t nS = static_cast<uint64_t>(B) * (ldS / 128), nA = static_cast<uint64_t>(B) * (ldA / 128);
-  if (tmap_bf16_blocked(&tSh, St_hi, T, nS) || tmap_bf16_blocked(&tSl, St_lo, T, nS) ||
-      tmap_bf16_blocked(&tAh, At_hi, T, nA) || tmap_bf16_blocked(&tAl, At_lo, T, nA))
+  if (tmap_chunked(&tSh, St_hi, T, nS) || tmap_chunked(&tSl, St_lo, T, nS) ||
+      tmap_chunked(&tAh, At_hi, T, nA) || tmap_chunked(&tAl, At_lo, T, nA))
     return cudaErrorInvalidValue;
   EkfacArgs g;
   g.T = T;
