@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   const ContractArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   float* stage_buf = reinterpret_cast<float*>(smem + static_cast<size_t>(g.stages) * kCStage);
   uint64_t* full = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(stage_buf) + kCStageBuf);
   uint64_t* empty = full + g.stages;
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(128, 128, 1, 1);
       uint32_t it = 0;
       int rs = 0;         // ring slot of pipeline iteration it (it % stages)
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int item = blockIdx.x; item < g.n_items && ok; item += gridDim.x, ++i) {
         const int buf = i & 1;
         const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
-        if (!mbar_wait(&tempty[buf], aph ^ 1u, g.status)) break;
+        if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, g.status)) break;
         tc_fence_after();
         const uint32_t d = tmem + buf * 128u;
         for (int kb = 0; kb < nkb; ++kb, ++it) {
@@ -332,22 +332,24 @@ __global__ void __launch_bounds__(kThreads, 1)
           } else {
             dsh += kCStage >> 4;
           }
-          if (!mbar_wait(&full[s], ph, g.status)) {
+          if (!mbar_wait_warp(&full[s], ph, g.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
           constexpr uint64_t kOp = kOpBytes >> 4, kRow16 = (2 * kTokGroup) >> 4;  // 16 tokens
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t sh = sh0 + kk * kRow16, sl = sh + kOp, ah = sh + 2 * kOp, al = sh + 3 * kOp;
-            tc_mma_f16(d, sh, ah, idesc, (kb | kk) != 0 ? 1u : 0u);
-            tc_mma_f16(d, sh, al, idesc, 1u);
-            tc_mma_f16(d, sl, ah, idesc, 1u);
+            for (int kk = 0; kk < 4; ++kk) {
+              const uint64_t sh = sh0 + kk * kRow16, sl = sh + kOp, ah = sh + 2 * kOp, al = sh + 3 * kOp;
+              tc_mma_f16(d, sh, ah, idesc, (kb | kk) != 0 ? 1u : 0u);
+              tc_mma_f16(d, sh, al, idesc, 1u);
+              tc_mma_f16(d, sl, ah, idesc, 1u);
+            }
+            tc_commit(&empty[s]);
           }
-          tc_commit(&empty[s]);
         }
-        tc_commit(&tfull[buf]);
+        if (elect_one()) tc_commit(&tfull[buf]);
       }
     }
     __syncwarp();
@@ -429,7 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                const EkfacArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(g.stages) * kCStage);
   uint64_t* empty = full + g.stages;
   uint64_t* tfull = empty + g.stages;
@@ -494,7 +496,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(128, 128, 1, 1);
       uint32_t it = 0;
       int rs = 0;         // ring slot of pipeline iteration it (it % stages)
@@ -507,7 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int b = chunk * g.bpc; b < b1 && ok; ++b, ++i) {
           const int buf = i & 1;
           const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
-          if (!mbar_wait(&tempty[buf], aph ^ 1u, g.status)) {
+          if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, g.status)) {
             ok = false;
             break;
           }
@@ -520,26 +522,28 @@ __global__ void __launch_bounds__(kThreads, 1)
               rs = 0;
               rph ^= 1u;
             }
-            if (!mbar_wait(&full[s], ph, g.status)) {
+            if (!mbar_wait_warp(&full[s], ph, g.status)) {
               ok = false;
               break;
             }
             tc_fence_after();
             const uint32_t sa = smem_u32(smem + static_cast<size_t>(s) * kCStage);
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint32_t o = kk * 2 * kTokGroup;  // 16 tokens
-              const uint64_t sh = sdesc_mn_chunks(sa + 0 * kOpBytes + o, kTokGroup, kChunkBytes);
-              const uint64_t sl = sdesc_mn_chunks(sa + 1 * kOpBytes + o, kTokGroup, kChunkBytes);
-              const uint64_t ah = sdesc_mn_chunks(sa + 2 * kOpBytes + o, kTokGroup, kChunkBytes);
-              const uint64_t al = sdesc_mn_chunks(sa + 3 * kOpBytes + o, kTokGroup, kChunkBytes);
-              tc_mma_f16(d, sh, ah, idesc, (kb | kk) != 0 ? 1u : 0u);
-              tc_mma_f16(d, sh, al, idesc, 1u);
-              tc_mma_f16(d, sl, ah, idesc, 1u);
+              for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t o = kk * 2 * kTokGroup;  // 16 tokens
+                const uint64_t sh = sdesc_mn_chunks(sa + 0 * kOpBytes + o, kTokGroup, kChunkBytes);
+                const uint64_t sl = sdesc_mn_chunks(sa + 1 * kOpBytes + o, kTokGroup, kChunkBytes);
+                const uint64_t ah = sdesc_mn_chunks(sa + 2 * kOpBytes + o, kTokGroup, kChunkBytes);
+                const uint64_t al = sdesc_mn_chunks(sa + 3 * kOpBytes + o, kTokGroup, kChunkBytes);
+                tc_mma_f16(d, sh, ah, idesc, (kb | kk) != 0 ? 1u : 0u);
+                tc_mma_f16(d, sh, al, idesc, 1u);
+                tc_mma_f16(d, sl, ah, idesc, 1u);
+              }
+              tc_commit(&empty[s]);
             }
-            tc_commit(&empty[s]);
           }
-          tc_commit(&tfull[buf]);
+          if (elect_one()) tc_commit(&tfull[buf]);
         }
       }
     }
@@ -718,7 +722,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const RotArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t stage_bytes = kABytes + static_cast<uint32_t>(g.BN) * 128u;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(g.stages) * stage_bytes);
   uint64_t* empty = full + g.stages;
@@ -776,49 +780,47 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // The issuing thread's own work per K block is kept minimal (one lane issues
-      // every MMA, so its instruction latency paces the tensor pipe): ring slot,
-      // phase and operand descriptors advance incrementally. A descriptor's
-      // address field is (byte address >> 4), so +2 steps 32 bytes (K = 16 bf16).
-      const uint32_t idesc = idesc_bf16_f32(128, g.BN, 0, 0);
-      const uint64_t dbase = sdesc_sw128(smem_u32(smem), 16, 1024);
-      const uint64_t dstage = stage_bytes >> 4, dab = kABytes >> 4;
-      uint64_t da = dbase;  // descriptor of operand A in ring slot rs
-      int rs = 0;           // ring slot of the next K block
-      uint32_t rph = 0;     // and its phase parity
-      int i = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++i) {
-        const int buf = i & 1;
-        const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
-        if (!mbar_wait(&tempty[buf], aph ^ 1u, g.status)) break;
+    // Ring slot, phase and operand descriptors advance incrementally. A descriptor's
+    // address field is (byte address >> 4), so +2 steps 32 bytes (K = 16 bf16).
+    const uint32_t idesc = idesc_bf16_f32(128, g.BN, 0, 0);
+    const uint64_t dbase = sdesc_sw128(smem_u32(smem), 16, 1024);
+    const uint64_t dstage = stage_bytes >> 4, dab = kABytes >> 4;
+    uint64_t da = dbase;  // descriptor of operand A in ring slot rs
+    int rs = 0;           // ring slot of the next K block
+    uint32_t rph = 0;     // and its phase parity
+    int i = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++i) {
+      const int buf = i & 1;
+      const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
+      if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, g.status)) break;
+      tc_fence_after();
+      const uint32_t d = tmem + buf * bstride;
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int s = rs;
+        const uint32_t ph = rph;
+        const uint64_t a0 = da, b0 = da + dab;
+        if (++rs == g.stages) {
+          rs = 0;
+          rph ^= 1u;
+          da = dbase;
+        } else {
+          da += dstage;
+        }
+        if (!mbar_wait_warp(&full[s], ph, g.status)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t d = tmem + buf * bstride;
-        for (int kb = 0; kb < nkb; ++kb) {
-          const int s = rs;
-          const uint32_t ph = rph;
-          const uint64_t a0 = da, b0 = da + dab;
-          if (++rs == g.stages) {
-            rs = 0;
-            rph ^= 1u;
-            da = dbase;
-          } else {
-            da += dstage;
-          }
-          if (!mbar_wait(&full[s], ph, g.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
+        if (elect_one()) {
           tc_mma_f16(d, a0, b0, idesc, kb != 0 ? 1u : 0u);
           tc_mma_f16(d, a0 + 2, b0 + 2, idesc, 1u);
           tc_mma_f16(d, a0 + 4, b0 + 4, idesc, 1u);
           tc_mma_f16(d, a0 + 6, b0 + 6, idesc, 1u);
           tc_commit(&empty[s]);
         }
-        tc_commit(&tfull[buf]);
       }
+      if (elect_one()) tc_commit(&tfull[buf]);
     }
     __syncwarp();
   } else {
@@ -866,7 +868,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                  const RotArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int half = g.BN / 2;  // W rows held by this CTA
   const uint32_t stage_bytes = kABytes + static_cast<uint32_t>(half) * 128u;
@@ -930,7 +932,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // as in k_tc_rotate: slot, phase and descriptors advance incrementally
       const uint32_t idesc = idesc_bf16_f32(256, g.BN, 0, 0);
       const uint64_t dbase = sdesc_sw128(smem_u32(smem), 16, 1024);
@@ -943,7 +945,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int t = cl; t < g.n_tiles && ok; t += ncl, ++i) {
         const int buf = i & 1;
         const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
-        if (!mbar_wait(&tempty[buf], aph ^ 1u, g.status)) break;
+        if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, g.status)) break;
         tc_fence_after();
         const uint32_t d = tmem + buf * bstride;
         for (int kb = 0; kb < nkb; ++kb) {
@@ -957,18 +959,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           } else {
             da += dstage;
           }
-          if (!mbar_wait(&full[s], ph, g.status)) {
+          if (!mbar_wait_warp(&full[s], ph, g.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          tc_mma_f16_pair(d, a0, b0, idesc, kb != 0 ? 1u : 0u);
-          tc_mma_f16_pair(d, a0 + 2, b0 + 2, idesc, 1u);
-          tc_mma_f16_pair(d, a0 + 4, b0 + 4, idesc, 1u);
-          tc_mma_f16_pair(d, a0 + 6, b0 + 6, idesc, 1u);
-          tc_commit_pair_mc(&empty[s], 0x3);
+          if (elect_one()) {
+            tc_mma_f16_pair(d, a0, b0, idesc, kb != 0 ? 1u : 0u);
+            tc_mma_f16_pair(d, a0 + 2, b0 + 2, idesc, 1u);
+            tc_mma_f16_pair(d, a0 + 4, b0 + 4, idesc, 1u);
+            tc_mma_f16_pair(d, a0 + 6, b0 + 6, idesc, 1u);
+            tc_commit_pair_mc(&empty[s], 0x3);
+          }
         }
-        tc_commit_pair_mc(&tfull[buf], 0x3);
+        if (elect_one()) tc_commit_pair_mc(&tfull[buf], 0x3);
       }
     }
     __syncwarp();
