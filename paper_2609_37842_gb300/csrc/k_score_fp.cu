@@ -19,7 +19,7 @@
 // parts lie stacked as 3 QB rows of one operand B, so a K = 16 step is three
 // MMAs: x1 by all 3 QB rows, x2 by the first 2 QB, x3 by the first QB, each into
 // the columns one part further on. 48 queries against 16,384 x 49,152 stored
-// coordinates (3.2 GB): 561 us, 0.85 of the measured copy rate (0.95 of it are the
+// coordinates (3.2 GB): 544 us, 0.87 of the measured copy rate (0.95 of it are the
 // K ranges' last wave), against 5,702 us on the CUDA cores.
 //
 // Pipeline per CTA (persistent over (row tile, K range, query tile) items):
@@ -27,9 +27,9 @@
 //    ring of eight or ten, and query tiles of 3 QB rows x 64 coordinates in a ring of three;
 //  * eight converter warps in two groups that take the boxes in turn (one warp per
 //    TMEM lane quarter): shared memory -> three bf16 parts -> TMEM, 48 columns a box;
-//  * one issuing thread: 12 MMAs per pair of boxes (one query tile) and round of
-//    wait, fence and commit (measured at 6 per round, the rounds set the pace: 646 us
-//    for the case above whatever the number of queries);
+//  * one issuing warp (converged, MMAs under elect.sync): 12 MMAs per pair of boxes
+//    (one query tile) and round of wait, fence and commit. With 6 per round the
+//    rounds set the pace, 646 us for the case above whatever the number of queries;
 //  * four drain warps: every 256 coordinates the three accumulators of a row into
 //    registers; at the item's end the sums to the scores or to the K range's slab.
 #include <algorithm>
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* dfull = aempty + kSlots;
   uint64_t* dempty = dfull + 2;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(dempty + 2);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmX);
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMmaW) {
     // ---------------------------------------------------------- issuer
-    if (lane == 0) {
+    {
       const uint32_t id1 = idesc_bf16_f32(128, 3 * QB, 0, 0), id2 = idesc_bf16_f32(128, 2 * QB, 0, 0),
                      id3 = idesc_bf16_f32(128, QB, 0, 0);
       const uint64_t ydesc = sdesc_sw128(smem_u32(ysm), 16, 1024);
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         item_boxes(item, b0, b1);
         for (int b = b0; b < b1 && ok; b += kDrainBoxes, ++run) {
           const int buf = static_cast<int>(run % ND);
-          if (!mbar_wait(&dempty[buf], ((run / ND) & 1u) ^ 1u, g.status)) {
+          if (!mbar_wait_warp(&dempty[buf], ((run / ND) & 1u) ^ 1u, g.status)) {
             ok = false;
             break;
           }
@@ -291,26 +291,28 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int e = min(b1, b + kDrainBoxes);
           for (int bb = b; bb < e; bb += 2, ++pr) {
             const int as = static_cast<int>(pr % kSlots), ys = static_cast<int>(pr % kYRing);
-            if (!mbar_wait(&yfull[ys], (pr / kYRing) & 1u, g.status) ||
-                !mbar_wait(&afull[as], (pr / kSlots) & 1u, g.status)) {
+            if (!mbar_wait_warp(&yfull[ys], (pr / kYRing) & 1u, g.status) ||
+                !mbar_wait_warp(&afull[as], (pr / kSlots) & 1u, g.status)) {
               ok = false;
               break;
             }
             tc_fence_after();
             const uint64_t y0 = ydesc + ((ys * fp_ybox<QB>()) >> 4);
             const uint32_t a0 = tmem + kA0 + 96u * as;
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint64_t y = y0 + 2 * kk;  // K = 16: 32 bytes on
-              const uint32_t a = a0 + 48u * (kk >> 1) + 8u * (kk & 1);
-              mma_f16_ta(d, a, y, id1, (bb != b || kk != 0) ? 1u : 0u);
-              mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
-              mma_f16_ta(d + 2 * QB, a + 32u, y, id3, 1u);
+              for (int kk = 0; kk < 4; ++kk) {
+                const uint64_t y = y0 + 2 * kk;  // K = 16: 32 bytes on
+                const uint32_t a = a0 + 48u * (kk >> 1) + 8u * (kk & 1);
+                mma_f16_ta(d, a, y, id1, (bb != b || kk != 0) ? 1u : 0u);
+                mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
+                mma_f16_ta(d + 2 * QB, a + 32u, y, id3, 1u);
+              }
+              tc_commit(&aempty[as]);
+              tc_commit(&yempty[ys]);
             }
-            tc_commit(&aempty[as]);
-            tc_commit(&yempty[ys]);
           }
-          if (ok) tc_commit(&dfull[buf]);
+          if (ok && elect_one()) tc_commit(&dfull[buf]);
         }
       }
     }

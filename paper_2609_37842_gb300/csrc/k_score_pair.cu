@@ -27,13 +27,12 @@
 //    group gj - NQ is done, its A slots refilled once group gj - NG is done,
 //    both read from the one commit per group, so the queries' L2 latency is off
 //    the A slots' round trip.
-//  * issuing threads: a thread issues an MMA about every 64 cycles whatever N
-//    is, plus ~330 cycles per wait-fence-commit round: at 256 bits per round
-//    the rounds, not the tensor pipe, set the pace (measured: 589 cycles per
-//    four N = 256 MMAs, 8.4 of 9.7 PFLOP/s), at 512 bits the tensor pipe does
-//    (1024 cycles per eight, 9.7 PFLOP/s). An N = 64 MMA takes as long to issue
-//    as an N = 128 one, so 64-query tiles take four stages per group (and one
-//    module of 64 queries has its own two-issuer kernel, k_score_pair_ks.cu).
+//  * issuing warps: an MMA and a wait-fence-commit round have an issue cost of
+//    their own whatever N is, so a group carries two stages, with 64-query tiles
+//    four (and one module of 64 queries has its own two-issuer kernel,
+//    k_score_pair_ks.cu). The warps run their loops converged and issue under
+//    elect.sync, which keeps descriptors and addresses uniform: GPT-2 queries
+//    423 -> 401 us against loops under lane == 0.
 //    128-query tiles of several modules have two accumulators and two issuers,
 //    issuer b running the modules of accumulator b, so one thread's rounds
 //    overlap the other's MMAs. Groups then complete out of order, which the
@@ -158,7 +157,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   uint8_t* smem = align1024(smem_raw);
   uint32_t code_off;
   const TcSmem L = pr_smem_layout<TOPK, BN, G>(&code_off);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   float* sq = reinterpret_cast<float*>(smem + L.sq);
   // group gj: full / empty barrier gj % NQ, query stages of slot gj % NQ, A
@@ -266,7 +265,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
   } else if (warp == kPrMmaWarp || warp == kIss1Warp) {
     constexpr int NI = pr_issuers<BN>();
     const int me = warp == kPrMmaWarp ? 0 : 1;
-    if (lane == 0 && rank == 0 && me < NI) {
+    if (rank == 0 && me < NI) {
       // ---------------------------------------------------------- MMA issuers (leader)
       // Kept to waits, MMAs and commits. With two issuers, issuer b runs the
       // modules of accumulator b and only the owner of a group issues and
@@ -312,7 +311,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             continue;
           }
           if (mine) {
-            if (!mbar_wait_cluster(&dempty[buf], ((gm / ND) & 1u) ^ 1u, g.status)) {
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&dempty[buf], ((gm / ND) & 1u) ^ 1u, g.status))) {
               ok = false;
               break;
             }
@@ -329,21 +328,23 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             // both CTAs' query bytes and expander warps (the MMAs read the
             // queries through the async proxy, tracked by the barrier's
             // transaction count)
-            if (!mbar_wait(&full[s], ph, g.status)) {
+            if (!mbar_wait_warp(&full[s], ph, g.status)) {
               ok = false;
               break;
             }
             if (!mine) continue;
             tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-            for (int st = 0; st < G; ++st)
+              for (int st = 0; st < G; ++st)
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                tc_mma_f4_ta_pair(d, at0 + 32u * st + 8u * kk, b0 + ((st * kStage) >> 4) + 2 * kk, idesc, sfa,
-                                  sfb, (gi | st | kk) != 0 ? 1u : 0u);
-            tc_commit_pair_mc(&empty[s], 0x3);
+                for (int kk = 0; kk < 4; ++kk)
+                  tc_mma_f4_ta_pair(d, at0 + 32u * st + 8u * kk, b0 + ((st * kStage) >> 4) + 2 * kk, idesc, sfa,
+                                    sfb, (gi | st | kk) != 0 ? 1u : 0u);
+              tc_commit_pair_mc(&empty[s], 0x3);
+            }
           }
-          if (mine && ok) tc_commit_pair_mc(&dfull[buf], 0x3);
+          if (mine && ok && elect_one()) tc_commit_pair_mc(&dfull[buf], 0x3);
         }
       }
     }

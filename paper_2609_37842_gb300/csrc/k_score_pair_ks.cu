@@ -2,13 +2,11 @@
 // pairs, with two MMA-issuing threads (Sec. 3.3 Eq. onebit_influence; App. B.3
 // scan): k_score_pair_ks.
 //
-// Why two issuers. A thread issues a tcgen05.mma about every 64 cycles
-// whatever N is, and an N = 64 e2m1 MMA of a pair (M = 256, K = 64) occupies
-// the tensor pipe for only about 32: one issuing thread leaves the pipe half
-// idle at 64 queries, and every wait-fence-commit round of that thread idles it
-// further. Measured back to back on 76 pairs: one thread 4,980 TFLOP/s at
-// N = 64, two threads with their own accumulators 7,907, four 9,719 (the e2m1
-// rate). Here two threads split the K range of every pipeline group: of the
+// Why two issuers. An N = 64 e2m1 MMA of a pair (M = 256, K = 64) occupies the
+// tensor pipe for only about 32 cycles, less than its issue costs a thread, and
+// every wait-fence-commit round of that thread idles the pipe further. The issuing
+// warps run converged and issue under elect.sync (uniform descriptors): 1M rows of
+// 16,384 bits 613 -> 531 us against loops under lane == 0. Here two threads split the K range of every pipeline group: of the
 // group's four 256-bit stages, issuer 0 runs stages 0 and 1 into accumulator
 // d_A (TMEM columns 0-63), issuer 1 stages 2 and 3 into d_B (columns 64-127).
 // The drain adds the two: both hold exact small integers (|d| <= k < 2^24), so
@@ -88,7 +86,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const __grid_constant__ ScoreTcArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   float* sq = reinterpret_cast<float*>(smem + kSqOff);
   // group gj: full / empty barrier gj % NQ, query stages of slot gj % NQ, A
@@ -239,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == kIss0Warp || warp == kIss1Warp) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // ---------------------------------------------------------- issuers (leader)
       // Issuer h runs stages 2h, 2h + 1 of every group into its own accumulator.
       const int half = warp == kIss0Warp ? 0 : 1;
@@ -256,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int tile = tile_begin<false, true>(g), tstep = tile_step<false, true>(), tend = tile_end<false, true>(g);
            tile < tend && ok; tile += tstep, ++tl) {
         // both accumulators drained (the drain releases them together)
-        if (!mbar_wait_cluster(dempty, (tl & 1u) ^ 1u, g.status)) break;
+        if (!__all_sync(0xffffffffu, mbar_wait_cluster(dempty, (tl & 1u) ^ 1u, g.status))) break;
         tc_fence_after();
         for (int gi = 0; gi < nbx; ++gi) {
           const int s = rq;
@@ -276,20 +274,22 @@ __global__ void __launch_bounds__(kThreads, 1)
           sa += kG;
           if (sa >= static_cast<uint32_t>(kSlots)) sa -= kSlots;
           // both CTAs' query bytes and expander warps
-          if (!mbar_wait(&full[s], ph, g.status)) {
+          if (!mbar_wait_warp(&full[s], ph, g.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          issue_half(d, a0, a1, b0, b1, idesc, sfa, sfb, gi == 0);
-          tc_commit_pair_mc(&empty[s], 0x3);
+          if (elect_one()) {
+            issue_half(d, a0, a1, b0, b1, idesc, sfa, sfb, gi == 0);
+            tc_commit_pair_mc(&empty[s], 0x3);
+          }
         }
-        if (ok) tc_commit_pair_mc(dfull, 0x3);
+        if (ok && elect_one()) tc_commit_pair_mc(dfull, 0x3);
       }
       // every MMA of this thread done before TMEM is released (also after a
       // timeout above)
-      tc_commit_pair_mc(&fin[half], 0x1);
-      mbar_wait(&fin[half], 0, g.status);
+      if (elect_one()) tc_commit_pair_mc(&fin[half], 0x1);
+      mbar_wait_warp(&fin[half], 0, g.status);
     }
     __syncwarp();
   } else if (warp == kCodeWarp) {

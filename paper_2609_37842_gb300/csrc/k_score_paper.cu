@@ -10,7 +10,7 @@
 // acc = fl(acc + fl(s_iu d)) in fp32 registers.
 //
 // Bound: the bf16 tensor rate (two products a coordinate). 250 queries against
-// 16,384 rows of 48 x 1024 bits: 570 us (1.45 PFLOP/s issued, 0.74 of the measured
+// 16,384 rows of 48 x 1024 bits: 491 us (1.68 PFLOP/s issued, 0.86 of the measured
 // burst rate; the last wave of items and the drains take 0.11 of it), against 864
 // us for the one-CTA kernel of k_score_tc.cu, which expands into shared memory and
 // issues hi and lo separately, 8 MMAs of N = 128 a round.
@@ -22,9 +22,8 @@
 //    a row from its four code words into 64 TMEM columns, two instructions a
 //    column: column j of a word holds bits j and j + 16 (the queries are laid out in
 //    the same order);
-//  * one issuing thread: 8 MMAs a round (a round of wait, fence and commit costs the
-//    thread ~330 cycles beside ~64 an MMA, so 4 MMAs of 128 cycles would not keep
-//    the tensor pipe busy);
+//  * one issuing warp (converged, MMAs under elect.sync: 570 -> 491 us against a
+//    loop under lane == 0): 8 MMAs a round of wait, fence and commit;
 //  * eight drain warps (two per lane quarter, half the queries each). One
 //    accumulator: the drain of a run (~300 of 8,200 cycles) holds up the next
 //    one's MMAs, and leaves TMEM for four rounds of A.
@@ -110,7 +109,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* dfull = aempty + kSlots;
   uint64_t* dempty = dfull + 1;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(dempty + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmC);
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMmaW) {
     // ---------------------------------------------------------- issuer
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(128, 2 * g.QB, 0, 0);
       const uint64_t ydesc = sdesc_sw128(smem_u32(smem), 16, 1024);
       uint32_t rd = 0, py = 0, run = 0;
@@ -258,34 +257,36 @@ __global__ void __launch_bounds__(kThreads, 1)
         int p0, p1, b, e, u;
         item_pairs(item, p0, p1);
         for (Runs rs(g, p0, p1); ok && rs.next(g, b, e, u); ++run) {
-          if (!mbar_wait(dempty, (run & 1u) ^ 1u, g.status)) {
+          if (!mbar_wait_warp(dempty, (run & 1u) ^ 1u, g.status)) {
             ok = false;
             break;
           }
           tc_fence_after();
           for (int p = b; p < e && ok; p += 2, ++rd) {
             const int as = static_cast<int>(rd % kSlots), n = min(2, e - p);
-            if (!mbar_wait(&afull[as], (rd / kSlots) & 1u, g.status)) {
+            if (!mbar_wait_warp(&afull[as], (rd / kSlots) & 1u, g.status)) {
               ok = false;
               break;
             }
             for (int i = 0; i < n; ++i, ++py) {
               const int ys = static_cast<int>(py % kYRing);
-              if (!mbar_wait(&yfull[ys], (py / kYRing) & 1u, g.status)) {
+              if (!mbar_wait_warp(&yfull[ys], (py / kYRing) & 1u, g.status)) {
                 ok = false;
                 break;
               }
               tc_fence_after();
               const uint64_t y = ydesc + ((ys * kYBox) >> 4);
               const uint32_t a = tmem + kA0 + 64u * as + 32u * i;
+              if (elect_one()) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_f16_ta(tmem, a + 8u * kk, y + 2 * kk, idesc, (p != b || i != 0 || kk != 0) ? 1u : 0u);
-              tc_commit(&yempty[ys]);
+                for (int kk = 0; kk < 4; ++kk)
+                  mma_f16_ta(tmem, a + 8u * kk, y + 2 * kk, idesc, (p != b || i != 0 || kk != 0) ? 1u : 0u);
+                tc_commit(&yempty[ys]);
+              }
             }
-            if (ok) tc_commit(&aempty[as]);
+            if (ok && elect_one()) tc_commit(&aempty[as]);
           }
-          if (ok) tc_commit(dfull);
+          if (ok && elect_one()) tc_commit(dfull);
         }
       }
     }

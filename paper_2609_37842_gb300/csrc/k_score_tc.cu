@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   const TcSmem L = tc_smem_layout<MODE, TOPK, BN, AT>(g.BNq, g.K);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   float* sq = reinterpret_cast<float*>(smem + L.sq);  // [2][BN] query scales of module u (CODES)
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L.bars);
   uint64_t* empty = full + S;
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     dequant_role<MODE, TOPK, BN, ND, kAccS, false>(g, smem, L, tmem, sq, dfull, dempty);
   } else {
     // ---------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
       const uint32_t idesc =
           MODE == EOGP_SCORE_CODES ? idesc_e4m3_f32(128, g.BNq) : idesc_bf16_f32(128, g.BNq, 0, 0);
       // One lane issues every MMA, so its own work per stage is kept minimal:
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
         for (int u = 0; u < g.U && ok; ++u, ++gm) {
           const int buf = static_cast<int>(gm % ND);
           const uint32_t dph = (gm / ND) & 1u;
-          if (!mbar_wait(&dempty[buf], dph ^ 1u, g.status)) {
+          if (!mbar_wait_warp(&dempty[buf], dph ^ 1u, g.status)) {
             ok = false;
             break;
           }
@@ -405,26 +405,28 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
               dst += kStage >> 4;
               acl += 32u;
             }
-            if (!mbar_wait(&full[s], ph, g.status)) {
+            if (!mbar_wait_warp(&full[s], ph, g.status)) {
               ok = false;
               break;
             }
             tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
-              if constexpr (AT) {
-                tc_mma_f8_ta(d, at0 + 8u * kk, a0 + 2 * kk, idesc, acc);
-              } else if (MODE == EOGP_SCORE_CODES) {
-                tc_mma_f8(d, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);
-              } else {
-                tc_mma_f16(d, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);
-                tc_mma_f16(d, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+              for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t acc = (kb | kk) != 0 ? 1u : 0u;
+                if constexpr (AT) {
+                  tc_mma_f8_ta(d, at0 + 8u * kk, a0 + 2 * kk, idesc, acc);
+                } else if (MODE == EOGP_SCORE_CODES) {
+                  tc_mma_f8(d, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);
+                } else {
+                  tc_mma_f16(d, a0 + 2 * kk, b0 + 2 * kk, idesc, acc);
+                  tc_mma_f16(d, a0 + 2 * kk, b1 + 2 * kk, idesc, 1u);
+                }
               }
+              tc_commit(&empty[s]);
             }
-            tc_commit(&empty[s]);
           }
-          tc_commit(&dfull[buf]);
+          if (elect_one()) tc_commit(&dfull[buf]);
         }
       }
     }

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const GemmArgs g) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t b_bytes = static_cast<uint32_t>(g.BN) * 128u;
   const uint32_t stage_bytes = static_cast<uint32_t>(g.nA) * kABytes + static_cast<uint32_t>(g.nW) * b_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(g.stages) * stage_bytes);
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(128, g.BN, 0, 0);
       int rs = 0;
       uint32_t rph = 0;
@@ -125,24 +125,26 @@ __global__ void __launch_bounds__(kThreads, 1)
           rs = 0;
           rph ^= 1u;
         }
-        if (!mbar_wait(&full[s], ph, g.status)) break;
+        if (!mbar_wait_warp(&full[s], ph, g.status)) break;
         tc_fence_after();
         const uint32_t sa = smem_u32(smem + static_cast<size_t>(s) * stage_bytes);
         const uint32_t sb = sa + g.nA * kABytes;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          for (int w = 0; w < g.nW; ++w) {
-            const uint64_t bd = sdesc_sw128(sb + w * b_bytes + kk * 32, 16, 1024);
-            for (int a = 0; a < g.nA; ++a) {
-              if (a == 1 && w == 1) continue;  // lo x lo: below the hi/lo pair's precision
-              const uint64_t ad = sdesc_sw128(sa + a * kABytes + kk * 32, 16, 1024);
-              tc_mma_f16(tmem, ad, bd, idesc, (i | kk | a | w) != 0 ? 1u : 0u);
+          for (int kk = 0; kk < 4; ++kk) {
+            for (int w = 0; w < g.nW; ++w) {
+              const uint64_t bd = sdesc_sw128(sb + w * b_bytes + kk * 32, 16, 1024);
+              for (int a = 0; a < g.nA; ++a) {
+                if (a == 1 && w == 1) continue;  // lo x lo: below the hi/lo pair's precision
+                const uint64_t ad = sdesc_sw128(sa + a * kABytes + kk * 32, 16, 1024);
+                tc_mma_f16(tmem, ad, bd, idesc, (i | kk | a | w) != 0 ? 1u : 0u);
+              }
             }
           }
+          tc_commit(&empty[s]);
         }
-        tc_commit(&empty[s]);
       }
-      tc_commit(done);
+      if (elect_one()) tc_commit(done);
     }
     __syncwarp();
   } else {
