@@ -547,6 +547,21 @@ int check_desc(const eogp_layer_desc* L, int B, int mode) {
   return EOGP_OK;
 }
 
+// The A and S rotations of M token rows, in one launch or two.
+int rotate_module(const RotSide& ra, const RotSide& rs, int M, int T, unsigned* status, cudaStream_t st) {
+  const int sms = sm_count();
+  if (rotate_in_one(ra, rs, M, sms)) {
+    ProfScope ps(EOGP_K_ROTATE, st);
+    CUDA_TRY(launch_tc_rotate_both(ra, rs, M, T, sms, status, st));
+    return EOGP_OK;
+  }
+  for (const RotSide* r : {&ra, &rs}) {
+    ProfScope ps(EOGP_K_ROTATE, st);
+    CUDA_TRY(launch_tc_rotate(*r, M, T, sms, status, st));
+  }
+  return EOGP_OK;
+}
+
 }  // namespace
 
 extern "C" int eogp_compress_workspace_size(const eogp_layer_desc* L, int B, int out_mode, size_t* bytes) {
@@ -606,16 +621,10 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
     void* st_hi = w + lo.st_hi;
     void* st_lo = w + lo.st_lo;
     // Kronecker rotations restricted to the retained columns C / rows R (Sec. 2.2).
-    {
-      ProfScope ps(EOGP_K_ROTATE, st);
-      CUDA_TRY(launch_tc_rotate(M, L->d_in, a, L->d_in, VA, L->d_in, P->nC(), at_hi, at_lo,
-                                lo.ldA, L->T, L->bias_A, nullptr, sm_count(), status, st));
-    }
-    {
-      ProfScope ps(EOGP_K_ROTATE, st);
-      CUDA_TRY(launch_tc_rotate(M, L->d_out, s, L->d_out, VS, L->d_out, P->nR(), st_hi, st_lo,
-                                lo.ldS, L->T, nullptr, L->lengths, sm_count(), status, st));
-    }
+    if (int rc = rotate_module(RotSide{a, L->d_in, VA, P->nC(), at_hi, at_lo, lo.ldA, L->bias_A, nullptr},
+                               RotSide{s, L->d_out, VS, P->nR(), st_hi, st_lo, lo.ldS, nullptr, L->lengths}, M, L->T,
+                               status, st))
+      return rc;
     // Per-example contraction over tokens + scale/gather into z (Eq. first_stage).
     const bool fs = out_mode == EOGP_OUT_FIRST_STAGE;
     {
@@ -632,7 +641,7 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
       const bool cd = out_mode == EOGP_OUT_CODES;
       CUDA_TRY(launch_srht(w + lo.zhi, w + lo.zlo, true, lo.ldzb, B, L->m, L->srht_signs, L->srht_rows,
                            L->k, cd ? nullptr : out, ld_out, cd ? codes : nullptr, ld_codes,
-                           cd ? scales : nullptr, ld_scales, status, st));
+                           cd ? scales : nullptr, ld_scales, status, st, true));
       return EOGP_OK;
     }
     // x = P^T z (Eq. second_stage), split over K; then sum + sign/pack (Eq. onebit).
@@ -646,10 +655,10 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
     ProfScope ps(EOGP_K_PACK, st);
     if (out_mode == EOGP_OUT_COORDS)
       CUDA_TRY(launch_pack(part, lo.splits, slab, lo.ldp, B, L->k, out, ld_out, nullptr, 0, nullptr,
-                           0, status, st));
+                           0, status, st, true));
     else
       CUDA_TRY(launch_pack(part, lo.splits, slab, lo.ldp, B, L->k, nullptr, 0, codes, ld_codes,
-                           scales, ld_scales, status, st));
+                           scales, ld_scales, status, st, true));
     return EOGP_OK;
   }
 
@@ -660,6 +669,11 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
   float* at = reinterpret_cast<float*>(w + lo.at);
   float* stt = reinterpret_cast<float*>(w + lo.st);
   const int nC = P->nC(), nR = P->nR();
+  // Behind a first stage whose blocks all run at once (64 token rows a block, one per
+  // SM; 16 rows a block, four per SM) the launch of the next kernel is hidden: 256
+  // examples of 16 tokens take 25.6 us, 30.5 without. Behind more blocks its own,
+  // waiting, take the room of those still to run: 4096 examples 111 us, 83 without.
+  const bool behind = static_cast<long long>(B) * L->T <= 64ll * sm_count();
   float* z = out_mode == EOGP_OUT_FIRST_STAGE ? out : reinterpret_cast<float*>(w + lo.z);
   const int ldz = out_mode == EOGP_OUT_FIRST_STAGE ? ld_out : L->m;
   if (f32_first_supported(B, L->T, nC, nR)) {
@@ -681,16 +695,16 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
     const bool cd = out_mode == EOGP_OUT_CODES;
     CUDA_TRY(launch_srht(z, nullptr, false, ldz, B, L->m, L->srht_signs, L->srht_rows, L->k,
                          cd ? nullptr : out, ld_out, cd ? codes : nullptr, ld_codes,
-                         cd ? scales : nullptr, ld_scales, status, st));
+                         cd ? scales : nullptr, ld_scales, status, st, behind));
     return EOGP_OK;
   }
   float* x = out_mode == EOGP_OUT_COORDS ? out : reinterpret_cast<float*>(w + lo.x);
   const int ldx = out_mode == EOGP_OUT_COORDS ? ld_out : L->k;
   CUDA_TRY(launch_simt_gemm(B, L->k, L->m, 1.f, z, ldz, 1, static_cast<const float*>(L->Pt), L->m, 1,
-                            x, ldx, st));
+                            x, ldx, st, behind));
   if (out_mode == EOGP_OUT_CODES)
     CUDA_TRY(launch_pack(x, 1, 0, ldx, B, L->k, nullptr, 0, codes, ld_codes, scales, ld_scales,
-                         status, st));
+                         status, st, behind));
   return EOGP_OK;
 }
 
@@ -1017,16 +1031,10 @@ extern "C" int eogp_ekfac_accumulate(const eogp_ekfac_desc* D, const void* a, co
   const int M = B * D->T;
   if (D->dtype == EOGP_BF16) {
     if (!aligned16(a) || !aligned16(s)) return set_error(EOGP_EINVAL, "a / s must be 16-byte aligned");
-    {
-      ProfScope ps(EOGP_K_ROTATE, st);
-      CUDA_TRY(launch_tc_rotate(M, D->d_in, a, D->d_in, D->VA, D->d_in, D->d_in, w + lo.at_hi,
-                                w + lo.at_lo, lo.ldA, D->T, nullptr, nullptr, sm_count(), status, st));
-    }
-    {
-      ProfScope ps(EOGP_K_ROTATE, st);
-      CUDA_TRY(launch_tc_rotate(M, D->d_out, s, D->d_out, D->VS, D->d_out, D->d_out, w + lo.st_hi,
-                                w + lo.st_lo, lo.ldS, D->T, nullptr, nullptr, sm_count(), status, st));
-    }
+    if (int rc = rotate_module(RotSide{a, D->d_in, D->VA, D->d_in, w + lo.at_hi, w + lo.at_lo, lo.ldA, nullptr, nullptr},
+                               RotSide{s, D->d_out, D->VS, D->d_out, w + lo.st_hi, w + lo.st_lo, lo.ldS, nullptr, nullptr},
+                               M, D->T, status, st))
+      return rc;
     ProfScope ps(EOGP_K_CONTRACT, st);
     CUDA_TRY(launch_tc_ekfac(w + lo.st_hi, w + lo.st_lo, lo.ldS, w + lo.at_hi, w + lo.at_lo, lo.ldA, B,
                              D->T, D->d_out, D->d_in, reinterpret_cast<float*>(w + lo.part), lo.n_chunks,
@@ -1173,7 +1181,7 @@ extern "C" int eogp_srht(const float* z, int B, int m, int ldz, const int8_t* si
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   ProfScope ps(EOGP_K_PROJECT, st);
   CUDA_TRY(launch_srht(z, nullptr, false, ldz, B, m, signs, rows, k, x, ldx, codes, ld_codes, scales,
-                       ld_scales, status, st));
+                       ld_scales, status, st, false));
   return EOGP_OK;
 }
 
@@ -1252,7 +1260,7 @@ extern "C" int eogp_pack_sign(const float* x, int B, int k, int ldx, uint32_t* c
   if (!status) return set_error(EOGP_ECUDA, "device status word unavailable");
   ProfScope ps(EOGP_K_PACK, reinterpret_cast<cudaStream_t>(stream));
   CUDA_TRY(launch_pack(x, 1, 0, ldx, B, k, nullptr, 0, codes, ld_codes, scales, ld_scales, status,
-                       reinterpret_cast<cudaStream_t>(stream)));
+                       reinterpret_cast<cudaStream_t>(stream), false));
   return EOGP_OK;
 }
 

@@ -89,6 +89,14 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
+// Programmatic dependent launch: pdl_wait returns once the kernels this one was
+// launched behind (launch_behind) have finished and their writes are visible; what
+// comes before it (barriers, TMEM, descriptors) overlaps their end. pdl_trigger lets
+// a kernel launched behind this one start its own prologue. Without such a
+// neighbour both do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // This thread's warp, as a uniform value.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0); }
 

@@ -31,6 +31,23 @@ int make_tmap(CUtensorMap* tm, CUtensorMapDataType dt, int rank, const void* bas
 
 }  // namespace eogp
 
+// Launch of a kernel that calls pdl_wait before it touches anything the kernels
+// before it on the stream write or read: its prologue overlaps their end.
+template <typename... P, typename... A>
+cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Retained-set plan.
 struct eogp_plan {
   int d_in = 0, d_out = 0, m = 0;
@@ -71,9 +88,10 @@ struct eogp_plan {
 
 // k_pack.cu: x (sum of `splits` partial slabs, slab stride `slab`) -> optional x
 // copy, sign codes and scales. One warp per row.
+// `behind`: launched behind the kernel that writes its input (launch_behind).
 cudaError_t launch_pack(const float* part, int splits, size_t slab, int ldp, int B, int k,
                         float* x_out, int ldx, uint32_t* codes, int ld_codes, float* scales,
-                        int ld_scales, unsigned* status, cudaStream_t st);
+                        int ld_scales, unsigned* status, cudaStream_t st, bool behind);
 
 // k_score.cu
 cudaError_t launch_score_codes(const uint32_t* train, int ldt, const float* ts, int ldts, int N,
@@ -173,12 +191,12 @@ size_t srht_smem_bytes(int m);
 cudaError_t launch_srht(const void* z0, const void* z1, bool hilo, int ldz, int B, int m,
                         const int8_t* signs, const int32_t* rows, int k, float* x, int ldx,
                         uint32_t* codes, int ld_codes, float* scales, int ld_scales, unsigned* status,
-                        cudaStream_t st);
+                        cudaStream_t st, bool behind);
 
 // k_simt.cu: C[i][j] = alpha * sum_k A(i,k) B(j,k), A(i,k) = A[i*sai + k*sak], etc.
 cudaError_t launch_simt_gemm(int M, int N, int K, float alpha, const float* A, long long sai,
                              long long sak, const float* Bm, long long sbj, long long sbk,
-                             float* C, long long ldc, cudaStream_t st);
+                             float* C, long long ldc, cudaStream_t st, bool behind = false);
 // z[b*ldz + r] = scale[r] * sum_t St[(b*T+t)*ldS + posR[r]] * At[(b*T+t)*ldA + posC[r]]
 // The same GEMM (alpha = 1, k contiguous in A and B) for the tiles that hold a
 // noted row (one of n_inote notes, ld_inote apart) or a noted block of jblock
@@ -220,12 +238,26 @@ cudaError_t launch_tc_gemm(int M, int N, int K, const void* X0, const void* X1, 
 cudaError_t launch_tc_gemm_hl(int M, int N, int K, const void* Ah, const void* Al, int lda, const void* Bh,
                               const void* Bl, int ldb, float* out, int ldo, float alpha, unsigned* status,
                               cudaStream_t st);
-// Persistent rotation GEMM: hi/lo = split(X[M x K] W[Wrows x K]^T), columns < ldo
-// (a multiple of 128), rows M = B * T, written in the chunked layout
-// [B][ldo / 8][T][8] that launch_tc_contract and launch_tc_ekfac read.
-cudaError_t launch_tc_rotate(int M, int K, const void* X, int ldx, const void* W, int ldw, int Wrows,
-                             void* hi, void* lo, int ldo, int T, const float* bias,
-                             const int32_t* lengths, int num_sms, unsigned* status, cudaStream_t st);
+// Persistent rotation GEMM: hi/lo = split(X[M x K] W[rows x K]^T) (both dense),
+// columns < ldo (a multiple of 128), rows M = B * T, written in the chunked layout
+// [B][ldo / 8][T][8] that launch_tc_contract and launch_tc_ekfac read. bias [rows]
+// is added to every row, rows of tokens t >= lengths[b] are zero (either may be null).
+struct RotSide {
+  const void* X;
+  int K;
+  const void* W;
+  int rows;
+  void* hi;
+  void* lo;
+  int ldo;
+  const float* bias;
+  const int32_t* lengths;
+};
+cudaError_t launch_tc_rotate(const RotSide& r, int M, int T, int num_sms, unsigned* status, cudaStream_t st);
+// The two sides of a module in one launch, and whether that is the better way.
+bool rotate_in_one(const RotSide& ra, const RotSide& rs, int M, int num_sms);
+cudaError_t launch_tc_rotate_both(const RotSide& ra, const RotSide& rs, int M, int T, int num_sms, unsigned* status,
+                                  cudaStream_t st);
 // Number of K splits launch_tc_gemm actually uses for a requested count.
 int tc_gemm_splits_used(int K, int splits);
 // Per-example tile-sparse contraction over tokens with the scale-and-gather epilogue.

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(256) k_pack_block_row(const float* __restrict_
                                                          float* __restrict__ scales, int ld_scales,
                                                          unsigned* status) {
   __shared__ float wsum[8];
+  eogp::pdl_wait();
   pack_row<8>(part, splits, slab, ldp, k, x_out, ldx, codes, ld_codes, scales, ld_scales, status,
               blockIdx.x, threadIdx.x >> 5, threadIdx.x & 31, wsum);
 }
@@ -131,6 +132,7 @@ __global__ void __launch_bounds__(256) k_pack_warp_row(const float* __restrict__
                                                         uint32_t* __restrict__ codes, int ld_codes,
                                                         float* __restrict__ scales, int ld_scales,
                                                         unsigned* status) {
+  eogp::pdl_wait();
   const int lane = threadIdx.x & 31;
   const int w0 = blockIdx.x * 8 + (threadIdx.x >> 5);
   for (int row = w0; row < B; row += gridDim.x * 8)
@@ -142,17 +144,14 @@ __global__ void __launch_bounds__(256) k_pack_warp_row(const float* __restrict__
 
 cudaError_t launch_pack(const float* part, int splits, size_t slab, int ldp, int B, int k,
                         float* x_out, int ldx, uint32_t* codes, int ld_codes, float* scales,
-                        int ld_scales, unsigned* status, cudaStream_t st) {
+                        int ld_scales, unsigned* status, cudaStream_t st, bool behind) {
   if (B <= 0) return cudaSuccess;
-  if (B < 4096) {
-    k_pack_block_row<<<static_cast<unsigned>(B), 256, 0, st>>>(part, splits, slab, ldp, B, k, x_out,
-                                                               ldx, codes, ld_codes, scales,
-                                                               ld_scales, status);
-  } else {
-    const int blocks = std::min((B + 7) / 8, 152 * 16);
-    k_pack_warp_row<<<static_cast<unsigned>(blocks), 256, 0, st>>>(part, splits, slab, ldp, B, k,
-                                                                   x_out, ldx, codes, ld_codes,
-                                                                   scales, ld_scales, status);
-  }
+  const bool block_row = B < 4096;
+  auto kernel = block_row ? k_pack_block_row : k_pack_warp_row;
+  const unsigned blocks = static_cast<unsigned>(block_row ? B : std::min((B + 7) / 8, 152 * 16));
+  if (behind)
+    return launch_behind(kernel, blocks, 256, 0, st, part, splits, slab, ldp, B, k, x_out, ldx, codes, ld_codes, scales,
+                         ld_scales, status);
+  kernel<<<blocks, 256, 0, st>>>(part, splits, slab, ldp, B, k, x_out, ldx, codes, ld_codes, scales, ld_scales, status);
   return cudaGetLastError();
 }

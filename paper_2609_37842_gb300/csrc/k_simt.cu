@@ -179,6 +179,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
                 int jblock) {
   constexpr int NX = BN / TN, NY = BM / TM;
   __shared__ GemmTiles<BM, BN> sm;
+  eogp::pdl_trigger();
+  eogp::pdl_wait();
   const int i0 = blockIdx.y * BM, j0 = blockIdx.x * BN;
   if (NOTED) {
     int hit = 0;
@@ -236,6 +238,7 @@ template <int BM, int L>
 __global__ void __launch_bounds__(first_threads<BM>()) k_f32_first(const FirstArgs g) {
   constexpr int NT = first_threads<BM>(), TN = 4, NX = 16, NY = NT / NX, TM = BM / NY, P = BM + 4;
   extern __shared__ __align__(16) uint8_t smem_raw[];
+  eogp::pdl_trigger();
   auto& sm = *reinterpret_cast<GemmTiles<BM, 64>*>(smem_raw);
   float* rot = reinterpret_cast<float*>(smem_raw + sizeof(GemmTiles<BM, 64>));
   const int b0 = blockIdx.x * g.G, nb = min(g.G, g.B - b0), rows = nb * g.T;
@@ -343,8 +346,12 @@ int layout_of(const Operand& a, const Operand& b, int K) {
 
 template <int BM, int BN, int TM, int TN, int PD, int L, bool NOTED>
 cudaError_t simt_launch(int M, int N, int K, float alpha, const Operand& A, const Operand& B, float* C, long long ldc,
-                        const int* inote, int n_inote, int ld_inote, const int* jnote, int jblock, cudaStream_t st) {
+                        const int* inote, int n_inote, int ld_inote, const int* jnote, int jblock, cudaStream_t st,
+                        bool behind = false) {
   const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
+  if (behind)
+    return launch_behind(k_simt_gemm<BM, BN, TM, TN, PD, L, NOTED>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, alpha, A,
+                         B, C, ldc, inote, n_inote, ld_inote, jnote, jblock);
   k_simt_gemm<BM, BN, TM, TN, PD, L, NOTED><<<grid, (BM / TM) * (BN / TN), 0, st>>>(M, N, K, alpha, A, B, C, ldc, inote,
                                                                                n_inote, ld_inote, jnote, jblock);
   return cudaGetLastError();
@@ -354,12 +361,12 @@ cudaError_t simt_launch(int M, int N, int K, float alpha, const Operand& A, cons
 
 template <int BM, int BN, int TM, int TN, int PD>
 static cudaError_t simt_layout(int l, int M, int N, int K, float alpha, const Operand& A, const Operand& B, float* C,
-                               long long ldc, cudaStream_t st) {
+                               long long ldc, cudaStream_t st, bool behind) {
   if (l == kAlongK)
-    return simt_launch<BM, BN, TM, TN, PD, kAlongK, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st);
+    return simt_launch<BM, BN, TM, TN, PD, kAlongK, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st, behind);
   if (l == kAlongRows)
-    return simt_launch<BM, BN, TM, TN, PD, kAlongRows, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st);
-  return simt_launch<BM, BN, TM, TN, 1, kAny, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st);
+    return simt_launch<BM, BN, TM, TN, PD, kAlongRows, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st, behind);
+  return simt_launch<BM, BN, TM, TN, 1, kAny, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st, behind);
 }
 
 // The largest tile that still gives the SMs blocks enough; small ones shorten the
@@ -370,16 +377,16 @@ static cudaError_t simt_layout(int l, int M, int N, int K, float alpha, const Op
 // in 32 x 32 tiles.
 cudaError_t launch_simt_gemm(int M, int N, int K, float alpha, const float* A, long long sai,
                              long long sak, const float* Bm, long long sbj, long long sbk,
-                             float* C, long long ldc, cudaStream_t st) {
+                             float* C, long long ldc, cudaStream_t st, bool behind) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   const Operand a{A, sai, sak, M}, b{Bm, sbj, sbk, N};
   const int l = layout_of(a, b, K);
   auto blocks = [&](int bm, int bn) { return static_cast<long long>((M + bm - 1) / bm) * ((N + bn - 1) / bn); };
   // (grid.y holds at most 65,535 tiles of rows: more rows take the largest tile)
   if (M > 65535 * 32 || (N > 64 && M > 64 && blocks(128, 128) >= 304))
-    return simt_layout<128, 128, 8, 8, 2>(l, M, N, K, alpha, a, b, C, ldc, st);
-  if (blocks(64, 64) >= 100) return simt_layout<64, 64, 4, 4, 2>(l, M, N, K, alpha, a, b, C, ldc, st);
-  return simt_layout<32, 32, 4, 2, 4>(l, M, N, K, alpha, a, b, C, ldc, st);
+    return simt_layout<128, 128, 8, 8, 2>(l, M, N, K, alpha, a, b, C, ldc, st, behind);
+  if (blocks(64, 64) >= 100) return simt_layout<64, 64, 4, 4, 2>(l, M, N, K, alpha, a, b, C, ldc, st, behind);
+  return simt_layout<32, 32, 4, 2, 4>(l, M, N, K, alpha, a, b, C, ldc, st, behind);
 }
 
 cudaError_t launch_simt_gemm_noted(int M, int N, int K, const float* A, long long lda, const float* Bm, long long ldb,

@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(kThreads) k_srht(const void* __restrict__ z0, 
   extern __shared__ float v[];
   __shared__ float wsum[kThreads / 32];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  eogp::pdl_wait();
   // J and D: signed row, zero-padded to p.
   for (int c = tid; c < p; c += kThreads) {
     float zc = 0.f;
@@ -101,23 +102,18 @@ size_t srht_smem_bytes(int m) { return static_cast<size_t>(srht_width(m)) * 4; }
 cudaError_t launch_srht(const void* z0, const void* z1, bool hilo, int ldz, int B, int m,
                         const int8_t* signs, const int32_t* rows, int k, float* x, int ldx,
                         uint32_t* codes, int ld_codes, float* scales, int ld_scales, unsigned* status,
-                        cudaStream_t st) {
+                        cudaStream_t st, bool behind) {
   if (B <= 0) return cudaSuccess;
   const int p = srht_width(m);
   const size_t smem = srht_smem_bytes(m);
   const float scale = 1.0f / sqrtf(static_cast<float>(k));
-  if (hilo) {
-    cudaError_t e = cudaFuncSetAttribute(k_srht<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    k_srht<true><<<B, kThreads, smem, st>>>(z0, z1, ldz, m, p, signs, rows, k, scale, x, ldx, codes,
-                                            ld_codes, scales, ld_scales, status);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(k_srht<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    k_srht<false><<<B, kThreads, smem, st>>>(z0, z1, ldz, m, p, signs, rows, k, scale, x, ldx, codes,
-                                             ld_codes, scales, ld_scales, status);
-  }
+  auto kernel = hilo ? k_srht<true> : k_srht<false>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  if (behind)
+    return launch_behind(kernel, B, kThreads, smem, st, z0, z1, ldz, m, p, signs, rows, k, scale, x, ldx, codes, ld_codes,
+                         scales, ld_scales, status);
+  kernel<<<B, kThreads, smem, st>>>(z0, z1, ldz, m, p, signs, rows, k, scale, x, ldx, codes, ld_codes, scales, ld_scales,
+                                    status);
   return cudaGetLastError();
 }

@@ -90,6 +90,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -273,6 +275,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -461,6 +465,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -698,8 +704,10 @@ __device__ __forceinline__ void rot_store(const RotArgs& g, const RotRow& r, int
                                                       v1 - __uint_as_float(h[e] & 0xFFFF0000u));
       l[e] = *reinterpret_cast<const uint32_t*>(&lo);
     }
-    *reinterpret_cast<uint4*>(g.hi + at) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(g.lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
+    if (col + 8 * q < g.ldo) {  // a tile may reach past the padded columns
+      *reinterpret_cast<uint4*>(g.hi + at) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(g.lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
   }
 }
 
@@ -710,35 +718,51 @@ __device__ __forceinline__ void rot_drain(const RotArgs& g, uint32_t tb, int row
   for (; c + 32 <= g.BN; c += 32) {
     float v[32];
     tmem_ld32(tb + c, v);
-    if (r.in && n0 + c < g.ldo) rot_store<32>(g, r, n0 + c, v);
+    if (r.in) rot_store<32>(g, r, n0 + c, v);
   }
   if (c < g.BN) {
     float v[16];
     tmem_ld16(tb + c, v);
-    if (r.in && n0 + c < g.ldo) rot_store<16>(g, r, n0 + c, v);
+    if (r.in) rot_store<16>(g, r, n0 + c, v);
   }
 }
 
+// One rotation, or two in one launch (the A and S sides of a module): the tiles of
+// g[0], then those of g[1], dealt to the CTAs back and forth, so that the shorter
+// ones of g[1] go to the CTAs that g[0] left idle.
+struct RotBoth {
+  RotArgs g[2];
+  int n_tiles, stages;     // of both; ring slots of `slot` bytes
+  uint32_t slot, tcols;    // TMEM columns (two accumulators)
+  __device__ __forceinline__ int tile(int round) const {  // this CTA's tile of a round, n_tiles or more past the end
+    const int n = gridDim.x, b = blockIdx.x;
+    return round * n + ((round & 1) && g[1].n_tiles ? n - 1 - b : b);
+  }
+};
+
 __global__ void __launch_bounds__(kThreads, 1)
-    k_tc_rotate(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
-                const RotArgs g) {
+    k_tc_rotate(const __grid_constant__ CUtensorMap tmX0, const __grid_constant__ CUtensorMap tmW0,
+                const __grid_constant__ CUtensorMap tmX1, const __grid_constant__ CUtensorMap tmW1,
+                const __grid_constant__ RotBoth p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const uint32_t stage_bytes = kABytes + static_cast<uint32_t>(g.BN) * 128u;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(g.stages) * stage_bytes);
-  uint64_t* empty = full + g.stages;
-  uint64_t* tfull = empty + g.stages;  // accumulator ready, per TMEM buffer
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(p.stages) * p.slot);
+  uint64_t* empty = full + p.stages;
+  uint64_t* tfull = empty + p.stages;  // accumulator ready, per TMEM buffer
   uint64_t* tempty = tfull + 2;        // accumulator drained, per TMEM buffer
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
-  const uint32_t tcols = g.BN <= 64 ? 128u : g.BN <= 128 ? 256u : 512u;
-  const uint32_t bstride = tcols / 2;
-  const int nkb = (g.K + 63) / 64;
+  const uint32_t bstride = p.tcols / 2;
+  unsigned* status = p.g[0].status;
 
   if (threadIdx.x == 0) {
-    tma_prefetch_desc(&tmX);
-    tma_prefetch_desc(&tmW);
-    for (int s = 0; s < g.stages; ++s) {
+    tma_prefetch_desc(&tmX0);
+    tma_prefetch_desc(&tmW0);
+    if (p.g[1].n_tiles) {
+      tma_prefetch_desc(&tmX1);
+      tma_prefetch_desc(&tmW1);
+    }
+    for (int s = 0; s < p.stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -748,35 +772,41 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(tmem_slot, tcols);
+  if (warp == 1) tmem_alloc(tmem_slot, p.tcols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
-      uint32_t it = 0;
-      int rs = 0;         // ring slot of pipeline iteration it (it % stages)
-      uint32_t rph = 0;  // and its phase parity ((it / stages) & 1)
+      int rs = 0;         // ring slot of the next K block
+      uint32_t rph = 0;   // and its phase parity
       bool ok = true;
-      for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
-        const int m0 = (t / g.nN) * 128, n0 = (t % g.nN) * g.BN;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+      for (int r = 0, t; ok && (t = p.tile(r)) < p.n_tiles; ++r) {
+        const int side = t >= p.g[0].n_tiles ? 1 : 0;
+        const RotArgs& g = p.g[side];
+        if (side) t -= p.g[0].n_tiles;
+        const CUtensorMap* tx = side ? &tmX1 : &tmX0;
+        const CUtensorMap* tw = side ? &tmW1 : &tmW0;
+        const uint32_t bytes = kABytes + static_cast<uint32_t>(g.BN) * 128u;
+        const int nkb = (g.K + 63) / 64, m0 = (t / g.nN) * 128, n0 = (t % g.nN) * g.BN;
+        for (int kb = 0; kb < nkb; ++kb) {
           const int s = rs;
           const uint32_t ph = rph;
-          if (++rs == g.stages) {
+          if (++rs == p.stages) {
             rs = 0;
             rph ^= 1u;
           }
-          if (!mbar_wait(&empty[s], ph ^ 1u, g.status)) {
+          if (!mbar_wait(&empty[s], ph ^ 1u, status)) {
             ok = false;
             break;
           }
-          uint8_t* st = smem + static_cast<size_t>(s) * stage_bytes;
-          mbar_arrive_expect_tx(&full[s], stage_bytes);
-          tma_load_2d(st, &tmX, kb * 64, m0, &full[s]);
-          tma_load_2d(st + kABytes, &tmW, kb * 64, n0, &full[s]);
+          uint8_t* st = smem + static_cast<size_t>(s) * p.slot;
+          mbar_arrive_expect_tx(&full[s], bytes);
+          tma_load_2d(st, tx, kb * 64, m0, &full[s]);
+          tma_load_2d(st + kABytes, tw, kb * 64, n0, &full[s]);
         }
       }
     }
@@ -784,32 +814,33 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     // Ring slot, phase and operand descriptors advance incrementally. A descriptor's
     // address field is (byte address >> 4), so +2 steps 32 bytes (K = 16 bf16).
-    const uint32_t idesc = idesc_bf16_f32(128, g.BN, 0, 0);
     const uint64_t dbase = sdesc_sw128(smem_u32(smem), 16, 1024);
-    const uint64_t dstage = stage_bytes >> 4, dab = kABytes >> 4;
+    const uint64_t dstage = p.slot >> 4, dab = kABytes >> 4;
     uint64_t da = dbase;  // descriptor of operand A in ring slot rs
     int rs = 0;           // ring slot of the next K block
     uint32_t rph = 0;     // and its phase parity
-    int i = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++i) {
-      const int buf = i & 1;
-      const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
-      if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, g.status)) break;
+    for (int r = 0, t; ok && (t = p.tile(r)) < p.n_tiles; ++r) {
+      const RotArgs& g = p.g[t >= p.g[0].n_tiles ? 1 : 0];
+      const uint32_t idesc = idesc_bf16_f32(128, g.BN, 0, 0);
+      const int nkb = (g.K + 63) / 64;
+      const int buf = r & 1;
+      const uint32_t aph = static_cast<uint32_t>(r >> 1) & 1u;
+      if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, status)) break;
       tc_fence_after();
       const uint32_t d = tmem + buf * bstride;
       for (int kb = 0; kb < nkb; ++kb) {
         const int s = rs;
         const uint32_t ph = rph;
         const uint64_t a0 = da, b0 = da + dab;
-        if (++rs == g.stages) {
+        if (++rs == p.stages) {
           rs = 0;
           rph ^= 1u;
           da = dbase;
         } else {
           da += dstage;
         }
-        if (!mbar_wait_warp(&full[s], ph, g.status)) {
+        if (!mbar_wait_warp(&full[s], ph, status)) {
           ok = false;
           break;
         }
@@ -827,12 +858,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else {
     const int q = warp & 3;
-    int i = 0;
-    for (int t = blockIdx.x; t < g.n_tiles; t += gridDim.x, ++i) {
-      const int buf = i & 1;
-      const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
+    for (int r = 0, t; (t = p.tile(r)) < p.n_tiles; ++r) {
+      const int side = t >= p.g[0].n_tiles ? 1 : 0;
+      const RotArgs& g = p.g[side];
+      if (side) t -= p.g[0].n_tiles;
+      const int buf = r & 1;
+      const uint32_t aph = static_cast<uint32_t>(r >> 1) & 1u;
       uint32_t ok = 1;
-      if (lane == 0) ok = mbar_wait(&tfull[buf], aph, g.status) ? 1u : 0u;
+      if (lane == 0) ok = mbar_wait(&tfull[buf], aph, status) ? 1u : 0u;
       ok = __shfl_sync(0xffffffffu, ok, 0);
       __syncwarp();
       tc_fence_after();
@@ -848,7 +881,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem, tcols);
+  if (warp == 1) tmem_dealloc(tmem, p.tcols);
 }
 
 size_t rotate_smem_bytes(int BN, int stages) {
@@ -903,6 +936,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync_all();  // barriers of both CTAs initialised before any remote arrive
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1033,7 +1067,7 @@ static int tmap_chunked(CUtensorMap* tm, const void* base, uint64_t T, uint64_t 
 static cudaError_t launch_tc_gemm_impl(int M, int N, int K, const void* X0, const void* X1, int ldx,
                                       const void* W, const void* W1, int ldw, int Wrows, int splits, int epi,
                                       void* out0, void* out1, int ldo, size_t slab, float alpha,
-                                      TcGemmCfg cfg, unsigned* status, cudaStream_t st) {
+                                      TcGemmCfg cfg, bool behind, unsigned* status, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   const int nA = X1 ? 2 : 1;
   const int nW = W1 ? 2 : 1;
@@ -1076,6 +1110,7 @@ static cudaError_t launch_tc_gemm_impl(int M, int N, int K, const void* X0, cons
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   dim3 grid((N + cfg.BN - 1) / cfg.BN, (M + 127) / 128, splits);
+  if (behind) return launch_behind(k_tc_gemm, grid, kThreads, smem, st, tX0, tX1, tW, tW1, g);
   k_tc_gemm<<<grid, kThreads, smem, st>>>(tX0, tX1, tW, tW1, g);
   return cudaGetLastError();
 }
@@ -1085,7 +1120,7 @@ cudaError_t launch_tc_gemm(int M, int N, int K, const void* X0, const void* X1, 
                                 void* out0, void* out1, int ldo, size_t slab, TcGemmCfg cfg,
                                 unsigned* status, cudaStream_t st) {
   return launch_tc_gemm_impl(M, N, K, X0, X1, ldx, W, nullptr, ldw, Wrows, splits, epi, out0, out1, ldo,
-                             slab, 1.0f, cfg, status, st);
+                             slab, 1.0f, cfg, true, status, st);
 }
 
 cudaError_t launch_tc_gemm_hl(int M, int N, int K, const void* Ah, const void* Al, int lda, const void* Bh,
@@ -1093,7 +1128,7 @@ cudaError_t launch_tc_gemm_hl(int M, int N, int K, const void* Ah, const void* A
                               cudaStream_t st) {
   // 128-column tiles: a stage holds 2 x 16 KB of A and 2 x 16 KB of B, three stages.
   return launch_tc_gemm_impl(M, N, K, Ah, Al, lda, Bh, Bl, ldb, N, 1, 1, out, nullptr, ldo, 0, alpha,
-                             TcGemmCfg{128, 3}, status, st);
+                             TcGemmCfg{128, 3}, false, status, st);
 }
 
 // CTA pairs measured faster for short reductions (K <= 1536: the hi/lo
@@ -1122,57 +1157,130 @@ int rotate_bn(int n, int gran) {
   return best;
 }
 
-cudaError_t launch_tc_rotate(int M, int K, const void* X, int ldx, const void* W, int ldw, int Wrows,
-                             void* hi, void* lo, int ldo, int T, const float* bias,
-                             const int32_t* lengths, int num_sms, unsigned* status, cudaStream_t st) {
-  if (M <= 0) return cudaSuccess;
-  const bool pairs = rotate_pairs(K, Wrows);
-  const int BN = rotate_bn(Wrows, 16);
-  // As many pipeline stages as fit in 227 KB of shared memory (at most 8).
-  int stages = 2;
-  while (stages < 8 && rotate_smem_bytes(BN, stages + 1) <= 232448) ++stages;
-  CUtensorMap tX, tW;
-  if (tmap_bf16_2d(&tX, X, static_cast<uint64_t>(K), static_cast<uint64_t>(M), ldx, 64, 128) ||
-      tmap_bf16_2d(&tW, W, K, Wrows, ldw, 64, BN))
-    return cudaErrorInvalidValue;
+static RotArgs rot_args(const RotSide& r, int M, int T, int BN, int m_tile, unsigned* status) {
   RotArgs g;
   g.M = M;
-  g.K = K;
+  g.K = r.K;
   g.BN = BN;
-  g.stages = stages;
-  g.nN = (Wrows + BN - 1) / BN;  // columns past the last tile (padding up to ldo) are not written
-  g.n_tiles = ((M + 127) / 128) * g.nN;
-  g.ldo = ldo;
+  g.stages = 0;
+  g.nN = (r.rows + BN - 1) / BN;  // columns past the last tile (padding up to ldo) are not written
+  g.n_tiles = ((M + m_tile - 1) / m_tile) * g.nN;
+  g.ldo = r.ldo;
   g.T = T;
-  g.hi = static_cast<__nv_bfloat16*>(hi);
-  g.lo = static_cast<__nv_bfloat16*>(lo);
-  g.bias = bias;
-  g.nbias = Wrows;
-  g.lengths = lengths;
+  g.hi = static_cast<__nv_bfloat16*>(r.hi);
+  g.lo = static_cast<__nv_bfloat16*>(r.lo);
+  g.bias = r.bias;
+  g.nbias = r.rows;
+  g.lengths = r.lengths;
   g.status = status;
-  if (pairs) {
-    // CTA pairs: tiles of 256 rows, W split in halves of BN / 2 rows.
-    CUtensorMap tWh;
-    if (tmap_bf16_2d(&tWh, W, K, Wrows, ldw, 64, BN / 2)) return cudaErrorInvalidValue;
-    int st2 = 2;
-    while (st2 < 8 && rotate2_smem_bytes(BN, st2 + 1) <= 232448) ++st2;
-    g.stages = st2;
-    g.n_tiles = ((M + 255) / 256) * g.nN;
-    const size_t smem = rotate2_smem_bytes(BN, st2);
-    cudaError_t e = cudaFuncSetAttribute(k_tc_rotate2, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    const int clusters = std::min(g.n_tiles, std::max(1, num_sms / 2));
-    k_tc_rotate2<<<2 * clusters, kThreads, smem, st>>>(tX, tWh, g);
-    return cudaGetLastError();
+  return g;
+}
+
+// One launch of k_tc_rotate over one side, or over both with tiles of BN columns.
+static cudaError_t launch_rot(const RotSide* r, int n, int M, int T, const int* BN, int num_sms, unsigned* status,
+                              cudaStream_t st) {
+  RotBoth p;
+  CUtensorMap tx[2], tw[2];
+  int bn = 0;
+  for (int i = 0; i < n; ++i) {
+    p.g[i] = rot_args(r[i], M, T, BN[i], 128, status);
+    bn = std::max(bn, BN[i]);
+    if (tmap_bf16_2d(&tx[i], r[i].X, static_cast<uint64_t>(r[i].K), static_cast<uint64_t>(M), r[i].K, 64, 128) ||
+        tmap_bf16_2d(&tw[i], r[i].W, r[i].K, r[i].rows, r[i].K, 64, BN[i]))
+      return cudaErrorInvalidValue;
   }
-  const size_t smem = rotate_smem_bytes(BN, stages);
-  cudaError_t e = cudaFuncSetAttribute(k_tc_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (n == 1) {
+    p.g[1] = p.g[0];
+    p.g[1].n_tiles = 0;
+    tx[1] = tx[0];
+    tw[1] = tw[0];
+  }
+  p.n_tiles = p.g[0].n_tiles + p.g[1].n_tiles;
+  p.slot = kABytes + static_cast<uint32_t>(bn) * 128u;
+  p.tcols = bn <= 64 ? 128u : bn <= 128 ? 256u : 512u;
+  // As many pipeline stages as fit in 227 KB of shared memory (at most 8).
+  p.stages = 2;
+  while (p.stages < 8 && rotate_smem_bytes(bn, p.stages + 1) <= 232448) ++p.stages;
+  const size_t smem = rotate_smem_bytes(bn, p.stages);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_tc_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  k_tc_rotate<<<std::min(p.n_tiles, std::max(1, num_sms)), kThreads, smem, st>>>(tx[0], tw[0], tx[1], tw[1], p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tc_rotate(const RotSide& r, int M, int T, int num_sms, unsigned* status, cudaStream_t st) {
+  if (M <= 0) return cudaSuccess;
+  const int BN = rotate_bn(r.rows, 16);
+  if (!rotate_pairs(r.K, r.rows)) return launch_rot(&r, 1, M, T, &BN, num_sms, status, st);
+  // CTA pairs: tiles of 256 rows, W split in halves of BN / 2 rows.
+  CUtensorMap tX, tWh;
+  if (tmap_bf16_2d(&tX, r.X, static_cast<uint64_t>(r.K), static_cast<uint64_t>(M), r.K, 64, 128) ||
+      tmap_bf16_2d(&tWh, r.W, r.K, r.rows, r.K, 64, BN / 2))
+    return cudaErrorInvalidValue;
+  RotArgs g = rot_args(r, M, T, BN, 256, status);
+  g.stages = 2;
+  while (g.stages < 8 && rotate2_smem_bytes(BN, g.stages + 1) <= 232448) ++g.stages;
+  const size_t smem = rotate2_smem_bytes(BN, g.stages);
+  cudaError_t e = cudaFuncSetAttribute(k_tc_rotate2, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const int grid = std::min(g.n_tiles, std::max(1, num_sms));
-  k_tc_rotate<<<grid, kThreads, smem, st>>>(tX, tW, g);
+  const int clusters = std::min(g.n_tiles, std::max(1, num_sms / 2));
+  k_tc_rotate2<<<2 * clusters, kThreads, smem, st>>>(tX, tWh, g);
   return cudaGetLastError();
+}
+
+static long long rot_tiles(const RotSide& r, int M, int BN) {
+  return static_cast<long long>((M + 127) / 128) * ((r.rows + BN - 1) / BN);
+}
+
+// Both sides of a module in one launch: when their tiles are at most two per SM,
+// where a launch of its own leaves most SMs idle for a whole tile.
+bool rotate_in_one(const RotSide& ra, const RotSide& rs, int M, int num_sms) {
+  return rot_tiles(ra, M, rotate_bn(ra.rows, 16)) + rot_tiles(rs, M, rotate_bn(rs.rows, 16)) <= 2ll * num_sms;
+}
+
+// The tile width is the one whose last CTA ends first. A K block of a BN-column tile
+// costs 2 BN cycles of the tensor pipe, at least ~220 in all. Five queries of 512
+// tokens through 768 -> 2304 take 11.6 us in one launch, 13.0 + 10.6 in two.
+cudaError_t launch_tc_rotate_both(const RotSide& ra, const RotSide& rs, int M, int T, int num_sms, unsigned* status,
+                                  cudaStream_t st) {
+  if (M <= 0) return cudaSuccess;
+  const bool swap = rs.K > ra.K;  // the longer reduction first
+  const RotSide r[2] = {swap ? rs : ra, swap ? ra : rs};
+  const int sms = std::max(1, num_sms);
+  int best[2] = {0, 0};
+  long long best_t = -1;
+  const int n = std::max(r[0].rows, r[1].rows);
+  for (int nN = (n + 255) / 256; best_t < 0 || nN <= (n + 63) / 64; ++nN) {  // tiles of the wider side
+    const int bn = ((n + nN - 1) / nN + 15) / 16 * 16;
+    int b[2];
+    long long cost[2], cnt[2];
+    for (int i = 0; i < 2; ++i) {
+      const int parts = (r[i].rows + bn - 1) / bn;
+      b[i] = std::max(16, ((r[i].rows + parts - 1) / parts + 15) / 16 * 16);
+      cnt[i] = rot_tiles(r[i], M, b[i]);
+      cost[i] = static_cast<long long>((r[i].K + 63) / 64) * std::max(2 * b[i], 220);
+    }
+    // the CTA that ends last under the back-and-forth order
+    const long long all = cnt[0] + cnt[1];
+    long long last = 0;
+    for (int c = 0; c < sms; ++c) {
+      long long sum = 0;
+      for (long long rd = 0; rd * sms < all; ++rd) {
+        const long long t = rd * sms + (rd & 1 ? sms - 1 - c : c);
+        if (t < all) sum += cost[t >= cnt[0] ? 1 : 0];
+      }
+      last = std::max(last, sum);
+    }
+    last += 12 * bn;
+    if (best_t < 0 || last < best_t) {
+      best_t = last;
+      best[0] = b[0];
+      best[1] = b[1];
+    }
+  }
+  return launch_rot(r, 2, M, T, best, num_sms, status, st);
 }
 
 int tc_gemm_splits_used(int K, int splits) {
@@ -1213,8 +1321,7 @@ cudaError_t launch_tc_contract(const void* St_hi, const void* St_lo, int ldS, co
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int grid = std::min(g.n_items, std::max(1, num_sms));
-  k_tc_contract<<<grid, kThreads, smem, st>>>(tSh, tSl, tAh, tAl, g);
-  return cudaGetLastError();
+  return launch_behind(k_tc_contract, grid, kThreads, smem, st, tSh, tSl, tAh, tAl, g);
 }
 
 size_t ekfac_smem_bytes(int stages) {
@@ -1259,8 +1366,7 @@ cudaError_t launch_tc_ekfac(const void* St_hi, const void* St_lo, int ldS, const
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int grid = std::min(g.n_items, std::max(1, num_sms));
-  k_tc_ekfac<<<grid, kThreads, smem, st>>>(tSh, tSl, tAh, tAl, g);
-  e = cudaGetLastError();
+  e = launch_behind(k_tc_ekfac, grid, kThreads, smem, st, tSh, tSl, tAh, tAl, g);
   if (e != cudaSuccess) return e;
   k_ekfac_finalize<<<std::max(1, num_sms) * 4, 256, 0, st>>>(part, (B + g.bpc - 1) / g.bpc, d_out, d_in,
                                                             sumsq, ld, accumulate);
