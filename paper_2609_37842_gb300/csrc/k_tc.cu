@@ -612,16 +612,246 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
+// k_tc_ekfac2 -- the same sums on CTA pairs (cta_group::2): 256 x N tiles, N = 64 to
+// 256 in steps of 64. Each CTA of a pair loads its own 128 columns of S~ and its half
+// of the N columns of A~, hi and lo; its accumulator holds its 128 rows. Per MMA flop
+// that is a third to a half of the shared-memory reads of a 128 x 128 tile, which at
+// 128 bytes a cycle take as long as its MMA, and half the L2 reads. TMEM holds two
+// accumulators of N columns, so the squares are summed in registers: eight epilogue
+// warps, N / 2 columns of 32 rows each. Examples, runs and the order of all sums are
+// those of k_tc_ekfac, the results bit for bit the same.
+struct Ekfac2Args {
+  int stages, nkb, N, n_ct, n_tiles, n_items, bpc, B, chS, chA, d_out, d_in;
+  float* part;  // [n_chunks][d_out][d_in]
+  unsigned* status;
+};
+constexpr int kEk2Threads = 320;
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kEk2Threads, 1)
+    k_tc_ekfac2(const __grid_constant__ CUtensorMap tmShi, const __grid_constant__ CUtensorMap tmSlo,
+                const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmAlo,
+                const Ekfac2Args g) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = align1024(smem_raw);
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const uint32_t a_bytes = static_cast<uint32_t>(g.N) * 64u;  // N / 2 columns of 64 tokens
+  const uint32_t stage_bytes = 2 * kOpBytes + 2 * a_bytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + static_cast<size_t>(g.stages) * stage_bytes);
+  uint64_t* empty = full + g.stages;
+  uint64_t* tfull = empty + g.stages;
+  uint64_t* tempty = tfull + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&tmShi);
+    tma_prefetch_desc(&tmSlo);
+    tma_prefetch_desc(&tmAhi);
+    tma_prefetch_desc(&tmAlo);
+    for (int s = 0; s < g.stages; ++s) {
+      mbar_init(&full[s], 2);   // one expect_tx arrive from each CTA (leader's copy is used)
+      mbar_init(&empty[s], 1);  // MMA completion, multicast to both CTAs
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&tfull[b], 1);    // multicast to both CTAs
+      mbar_init(&tempty[b], 16);  // 8 epilogue warps x 2 CTAs (leader's copy is used)
+    }
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc_pair(tmem_slot, 512);
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // barriers of both CTAs initialised before any remote arrive
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int rs = 0;
+      uint32_t rph = 0;
+      bool ok = true;
+      for (int item = cl; item < g.n_items && ok; item += ncl) {
+        const int chunk = item / g.n_tiles, tile = item % g.n_tiles;
+        const int rt = tile / g.n_ct, ct = tile % g.n_ct;
+        const int b1 = min(g.B, (chunk + 1) * g.bpc);
+        for (int b = chunk * g.bpc; b < b1 && ok; ++b) {
+          const int zs = b * g.chS + rt * 32 + static_cast<int>(rank) * 16;
+          const int za = b * g.chA + ct * (g.N / 8) + static_cast<int>(rank) * (g.N / 16);
+          for (int kb = 0; kb < g.nkb; ++kb) {
+            const int s = rs;
+            const uint32_t ph = rph;
+            if (++rs == g.stages) {
+              rs = 0;
+              rph ^= 1u;
+            }
+            if (!mbar_wait(&empty[s], ph ^ 1u, g.status)) {
+              ok = false;
+              break;
+            }
+            const uint32_t st = smem_u32(smem + static_cast<size_t>(s) * stage_bytes);
+            const uint32_t fl = mapa_shared(smem_u32(&full[s]), 0);
+            mbar_arrive_expect_tx_cluster(fl, stage_bytes);
+            const int x = kb * 256;  // 64 tokens of 16 bytes, in words
+            tma_load_2d_pair(st, &tmShi, x, zs, fl);
+            tma_load_2d_pair(st + kOpBytes, &tmSlo, x, zs, fl);
+            tma_load_2d_pair(st + 2 * kOpBytes, &tmAhi, x, za, fl);
+            tma_load_2d_pair(st + 2 * kOpBytes + a_bytes, &tmAlo, x, za, fl);
+          }
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (rank == 0) {
+      const uint32_t idesc = idesc_bf16_f32(256, g.N, 1, 1);
+      const uint64_t dbase = sdesc_mn_chunks(smem_u32(smem), kTokGroup, kChunkBytes);
+      const uint64_t dstage = stage_bytes >> 4, dsl = kOpBytes >> 4, dal = a_bytes >> 4;
+      uint64_t dd = dbase;  // descriptor of S hi in ring slot rs
+      int rs = 0;
+      uint32_t rph = 0;
+      int i = 0;  // examples issued by this pair (selects the TMEM buffer)
+      bool ok = true;
+      for (int item = cl; item < g.n_items && ok; item += ncl) {
+        const int chunk = item / g.n_tiles;
+        const int b1 = min(g.B, (chunk + 1) * g.bpc);
+        for (int b = chunk * g.bpc; b < b1 && ok; ++b, ++i) {
+          const int buf = i & 1;
+          const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
+          if (!mbar_wait_warp(&tempty[buf], aph ^ 1u, g.status)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d = tmem + buf * 256u;
+          for (int kb = 0; kb < g.nkb; ++kb) {
+            const int s = rs;
+            const uint32_t ph = rph;
+            const uint64_t sh0 = dd;
+            if (++rs == g.stages) {
+              rs = 0;
+              rph ^= 1u;
+              dd = dbase;
+            } else {
+              dd += dstage;
+            }
+            if (!mbar_wait_warp(&full[s], ph, g.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            if (elect_one()) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk) {
+                const uint64_t sh = sh0 + kk * (2 * kTokGroup >> 4);  // 16 tokens
+                const uint64_t ah = sh + 2 * dsl;
+                tc_mma_f16_pair(d, sh, ah, idesc, (kb | kk) != 0 ? 1u : 0u);
+                tc_mma_f16_pair(d, sh, ah + dal, idesc, 1u);
+                tc_mma_f16_pair(d, sh + dsl, ah, idesc, 1u);
+              }
+              tc_commit_pair_mc(&empty[s], 0x3);
+            }
+          }
+          if (elect_one()) tc_commit_pair_mc(&tfull[buf], 0x3);
+        }
+      }
+    }
+    __syncwarp();
+  } else {
+    const int q = warp & 3, half = (warp - 2) >> 2, nj = g.N / 64;
+    const uint32_t tb = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(half * (g.N / 2));
+    int i = 0;
+    uint32_t ok = 1;
+    for (int item = cl; item < g.n_items && ok; item += ncl) {
+      const int chunk = item / g.n_tiles, tile = item % g.n_tiles;
+      const int rt = tile / g.n_ct, ct = tile % g.n_ct;
+      const int b0 = chunk * g.bpc, b1 = min(g.B, (chunk + 1) * g.bpc);
+      float acc[4][32];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < 32; ++c) acc[j][c] = 0.f;
+      for (int b = b0; b < b1; ++b, ++i) {
+        const int buf = i & 1;
+        const uint32_t aph = static_cast<uint32_t>(i >> 1) & 1u;
+        if (lane == 0) ok = mbar_wait(&tfull[buf], aph, g.status) ? 1u : 0u;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();
+        tc_fence_after();
+        if (!ok) break;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (j < nj) {
+            float v[32];
+            tmem_ld32(tb + buf * 256u + 32 * j, v);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc[j][c] = __fadd_rn(acc[j][c], __fmul_rn(v[c], v[c]));
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_relaxed_cluster(mapa_shared(smem_u32(&tempty[buf]), 0));
+      }
+      const int row = rt * 256 + static_cast<int>(rank) * 128 + q * 32 + lane;
+      if (ok && row < g.d_out) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int col0 = ct * g.N + half * (g.N / 2) + 32 * j;
+          // d_in is a multiple of 8
+          float* dst = g.part + (static_cast<size_t>(chunk) * g.d_out + row) * g.d_in + col0;
+#pragma unroll
+          for (int c = 0; c < 32; c += 4)
+            if (j < nj && col0 + c < g.d_in)
+              *reinterpret_cast<float4*>(dst + c) = make_float4(acc[j][c], acc[j][c + 1], acc[j][c + 2], acc[j][c + 3]);
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // neither CTA leaves while its peer may still signal it
+  tc_fence_after();
+  if (warp == 1) tmem_dealloc_pair(tmem, 512);
+}
+
+// A finite, normal float as a double, on the integer pipe (the exponent's bias and
+// the significand's place differ): conversions share the few 64-bit lanes of an SM
+// with the additions.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if ((u << 1) - 0x01000000u >= 0xFE000000u) return static_cast<double>(x);  // zero, subnormal, infinite, NaN
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)),
+                          static_cast<int>(u << 29));
+}
+
 // sumsq[j * ld + i] (+)= sum over chunks c of part[c][j][i], chunks in order (fp64).
-__global__ void k_ekfac_finalize(const float* __restrict__ part, int n_chunks, int d_out, int d_in,
-                                 double* __restrict__ sumsq, int ld, int accumulate) {
-  const size_t n = static_cast<size_t>(d_out) * d_in;
-  for (size_t e = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    double t = 0.0;
-    for (int c = 0; c < n_chunks; ++c) t += static_cast<double>(part[static_cast<size_t>(c) * n + e]);
-    const size_t o = (e / d_in) * static_cast<size_t>(ld) + e % d_in;
-    sumsq[o] = accumulate ? sumsq[o] + t : t;
+// A thread sums four neighbouring columns of a row (16-byte loads). Bound by the
+// 64-bit additions: with a conversion and an addition per partial, three partials of
+// 3072 x 768 sums took 29 us whatever the loads; 8 us so.
+__global__ void __launch_bounds__(64)
+    k_ekfac_finalize(const float* __restrict__ part, int n_chunks, int d_out, int d_in, double* __restrict__ sumsq,
+                     int ld, int accumulate) {
+  pdl_wait();
+  const int col = 4 * (blockIdx.x * 64 + threadIdx.x);
+  if (col >= d_in) return;  // d_in is a multiple of 8
+  const size_t slab = static_cast<size_t>(d_out) * d_in;
+  for (int row = blockIdx.y; row < d_out; row += gridDim.y) {
+    const float* p = part + static_cast<size_t>(row) * d_in + col;
+    const float4 f = *reinterpret_cast<const float4*>(p);
+    double t[4] = {widen(f.x), widen(f.y), widen(f.z), widen(f.w)};
+#pragma unroll 4
+    for (int c = 1; c < n_chunks; ++c) {
+      const float4 v = *reinterpret_cast<const float4*>(p + c * slab);
+      t[0] += widen(v.x);
+      t[1] += widen(v.y);
+      t[2] += widen(v.z);
+      t[3] += widen(v.w);
+    }
+    double* o = sumsq + static_cast<size_t>(row) * ld + col;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) o[c] = accumulate ? o[c] + t[c] : t[c];
   }
 }
 
@@ -1056,11 +1286,11 @@ static int tmap_bf16_2d(CUtensorMap* tm, const void* base, uint64_t inner, uint6
 }
 
 // Chunked intermediate [nbatch * 16 chunks][T][8 columns] (bf16), as words: a box is
-// 64 tokens (1 KB) of the 16 chunks of a 128-column block.
-static int tmap_chunked(CUtensorMap* tm, const void* base, uint64_t T, uint64_t nbatch) {
+// 64 tokens (1 KB) of `chunks` chunks, 16 for a 128-column block.
+static int tmap_chunked(CUtensorMap* tm, const void* base, uint64_t T, uint64_t nbatch, uint32_t chunks = 16) {
   const uint64_t dims[2] = {4 * T, 16 * nbatch};
   const uint64_t strides[1] = {16 * T};
-  const uint32_t box[2] = {256, 16};
+  const uint32_t box[2] = {256, chunks};
   return make_tmap(tm, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
@@ -1336,11 +1566,58 @@ int ekfac_chunks(int B, int n_tiles, int num_sms) {
   return (B + bpc - 1) / bpc;
 }
 
-cudaError_t launch_tc_ekfac(const void* St_hi, const void* St_lo, int ldS, const void* At_hi,
-                            const void* At_lo, int ldA, int B, int T, int d_out, int d_in, float* part,
-                            int n_chunks, double* sumsq, int ld, int accumulate, int stages, int num_sms,
-                            unsigned* status, cudaStream_t st) {
-  if (B <= 0) return cudaSuccess;
+// Columns of a pair's tile: the time of the busiest pair is that of its items, in
+// columns per example; shorter than 96 columns a tile waits on its loads of S~.
+static int ekfac2_width(int n_rt, int d_in, int chunks, int pairs, long long* cost) {
+  int best = 0;
+  for (int N = 256; N >= 64; N -= 64) {
+    const long long items = static_cast<long long>(n_rt) * ((d_in + N - 1) / N) * chunks;
+    const long long t = (items + pairs - 1) / pairs * (std::max(N, 96) + 16);
+    if (!best || t < *cost) {
+      best = N;
+      *cost = t;
+    }
+  }
+  return best;
+}
+
+static cudaError_t launch_ekfac2(const void* St_hi, const void* St_lo, int ldS, const void* At_hi, const void* At_lo,
+                                 int ldA, int B, int T, int d_out, int d_in, float* part, int chunks, int N,
+                                 int num_sms, unsigned* status, cudaStream_t st) {
+  CUtensorMap tSh, tSl, tAh, tAl;
+  const uint64_t nS = static_cast<uint64_t>(B) * (ldS / 128), nA = static_cast<uint64_t>(B) * (ldA / 128);
+  if (tmap_chunked(&tSh, St_hi, T, nS) || tmap_chunked(&tSl, St_lo, T, nS) ||
+      tmap_chunked(&tAh, At_hi, T, nA, N / 16) || tmap_chunked(&tAl, At_lo, T, nA, N / 16))
+    return cudaErrorInvalidValue;
+  Ekfac2Args g;
+  g.nkb = (T + 63) / 64;
+  g.N = N;
+  g.n_ct = (d_in + N - 1) / N;
+  g.n_tiles = (d_out + 255) / 256 * g.n_ct;
+  g.n_items = g.n_tiles * chunks;
+  g.bpc = (B + chunks - 1) / chunks;
+  g.B = B;
+  g.chS = ldS / 8;
+  g.chA = ldA / 8;
+  g.d_out = d_out;
+  g.d_in = d_in;
+  g.part = part;
+  g.status = status;
+  const size_t stage = 2 * kOpBytes + 128 * static_cast<size_t>(N);
+  const auto bytes = [&](int stages) { return 1024 + stages * stage + (2 * stages + 4) * 8 + 16; };
+  g.stages = 2;
+  while (bytes(g.stages + 1) <= 232448) ++g.stages;
+  const size_t smem = bytes(g.stages);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_tc_ekfac2, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  return launch_behind(k_tc_ekfac2, 2 * std::min(g.n_items, std::max(1, num_sms / 2)), kEk2Threads, smem, st, tSh, tSl,
+                       tAh, tAl, g);
+}
+
+static cudaError_t launch_ekfac1(const void* St_hi, const void* St_lo, int ldS, const void* At_hi, const void* At_lo,
+                                 int ldA, int B, int T, int d_out, int d_in, float* part, int chunks, int stages,
+                                 int num_sms, unsigned* status, cudaStream_t st) {
   CUtensorMap tSh, tSl, tAh, tAl;
   const uint64_t nS = static_cast<uint64_t>(B) * (ldS / 128), nA = static_cast<uint64_t>(B) * (ldA / 128);
   if (tmap_chunked(&tSh, St_hi, T, nS) || tmap_chunked(&tSl, St_lo, T, nS) ||
@@ -1352,8 +1629,8 @@ cudaError_t launch_tc_ekfac(const void* St_hi, const void* St_lo, int ldS, const
   g.n_rt = (d_out + 127) / 128;
   g.n_ct = (d_in + 127) / 128;
   g.n_tiles = g.n_rt * g.n_ct;
-  g.bpc = (B + n_chunks - 1) / n_chunks;
-  g.n_items = g.n_tiles * ((B + g.bpc - 1) / g.bpc);
+  g.bpc = (B + chunks - 1) / chunks;
+  g.n_items = g.n_tiles * chunks;
   g.B = B;
   g.nblkS = ldS / 128;
   g.nblkA = ldA / 128;
@@ -1366,9 +1643,27 @@ cudaError_t launch_tc_ekfac(const void* St_hi, const void* St_lo, int ldS, const
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const int grid = std::min(g.n_items, std::max(1, num_sms));
-  e = launch_behind(k_tc_ekfac, grid, kThreads, smem, st, tSh, tSl, tAh, tAl, g);
+  return launch_behind(k_tc_ekfac, grid, kThreads, smem, st, tSh, tSl, tAh, tAl, g);
+}
+
+// Pairs, unless their tiles fill the chip worse: an example of a 128 x 128 tile takes
+// as long as one of 184 columns of a pair. 32 examples of 512 tokens, 3072 x 768: 187
+// us in 128 x 128 tiles, 140 in 256 x 192 (two waves of pairs, as are 256 x 256: 186),
+// 144 in 256 x 128 (three).
+cudaError_t launch_tc_ekfac(const void* St_hi, const void* St_lo, int ldS, const void* At_hi, const void* At_lo,
+                            int ldA, int B, int T, int d_out, int d_in, float* part, int n_chunks, double* sumsq,
+                            int ld, int accumulate, int stages, int num_sms, unsigned* status, cudaStream_t st) {
+  if (B <= 0) return cudaSuccess;
+  const int bpc = (B + n_chunks - 1) / n_chunks, chunks = (B + bpc - 1) / bpc, sms = std::max(1, num_sms);
+  const long long items1 = static_cast<long long>((d_out + 127) / 128) * ((d_in + 127) / 128) * chunks;
+  const long long cost1 = (items1 + sms - 1) / sms * 184;
+  long long cost2 = 0;
+  const int N = ekfac2_width((d_out + 255) / 256, d_in, chunks, std::max(1, sms / 2), &cost2);
+  cudaError_t e = cost2 <= cost1 ? launch_ekfac2(St_hi, St_lo, ldS, At_hi, At_lo, ldA, B, T, d_out, d_in, part, chunks,
+                                                 N, sms, status, st)
+                                 : launch_ekfac1(St_hi, St_lo, ldS, At_hi, At_lo, ldA, B, T, d_out, d_in, part, chunks,
+                                                 stages, sms, status, st);
   if (e != cudaSuccess) return e;
-  k_ekfac_finalize<<<std::max(1, num_sms) * 4, 256, 0, st>>>(part, (B + g.bpc - 1) / g.bpc, d_out, d_in,
-                                                            sumsq, ld, accumulate);
-  return cudaGetLastError();
+  const dim3 grid((d_in / 4 + 63) / 64, std::min(d_out, 65535));
+  return launch_behind(k_ekfac_finalize, grid, 64, 0, st, part, chunks, d_out, d_in, sumsq, ld, accumulate);
 }
