@@ -141,17 +141,26 @@ __device__ __forceinline__ int jac_index(int s, int x, int np) {
   return d < np / 2 ? d : L - d;
 }
 
-// (x, y) <- (c x - s y, s x + c y)
-__device__ __forceinline__ void jac_rotate(double c, double s, double& x, double& y) {
-  const double a = x, b = y;
-  x = c * a - s * b;
-  y = s * a + c * b;
+// (x, y) <- (c x - s y, s x + c y). r = (c, s), or LIFT: r = (tan(angle / 2), s) and
+// the rotation as three shears, three operations instead of four.
+template <bool LIFT>
+__device__ __forceinline__ void jac_rotate(double2 r, double& x, double& y) {
+  if (LIFT) {
+    x = __fma_rn(-r.x, y, x);
+    y = __fma_rn(r.y, x, y);
+    x = __fma_rn(-r.x, y, x);
+  } else {
+    const double a = x, b = y;
+    x = r.x * a - r.y * b;
+    y = r.y * a + r.x * b;
+  }
 }
 
 // Entry (x, y) after step s, formed from A before it and the step's rotations:
 // rows x and its partner rotated, then columns y and its partner. A row without a
 // partner (odd n) stays as it is. Loads and arithmetic apart, so that the loads of
 // several entries are in flight together.
+template <bool LIFT>
 struct JacEntry {
   double a, b, c, d;  // rows (x's pair) by columns (y's pair)
   double2 ck, cj;
@@ -178,18 +187,28 @@ struct JacEntry {
     d = __ldcg(Aq + qc);
   }
   __device__ __forceinline__ double value() {
+    if (LIFT) {  // no row is alone
+      const double l = rotated(ck, low_row, a, c), h = rotated(ck, low_row, b, d);
+      if (zero && ck.y != 0.0) return 0.0;  // the annihilated pair
+      return rotated(cj, low_col, l, h);
+    }
     if (row_alone) return low_col ? a : b;
-    jac_rotate(ck.x, ck.y, a, c);
+    jac_rotate<LIFT>(ck, a, c);
     if (col_alone) return low_row ? a : c;
-    jac_rotate(ck.x, ck.y, b, d);
-    jac_rotate(cj.x, cj.y, a, b);
-    jac_rotate(cj.x, cj.y, c, d);
+    jac_rotate<LIFT>(ck, b, d);
+    jac_rotate<LIFT>(cj, a, b);
+    jac_rotate<LIFT>(cj, c, d);
     if (zero && ck.y != 0.0) return 0.0;  // the annihilated pair
     return low_row ? (low_col ? a : b) : (low_col ? c : d);
+  }
+  static __device__ __forceinline__ double rotated(double2 r, bool low, double x, double y) {
+    jac_rotate<true>(r, x, y);
+    return low ? x : y;
   }
 };
 
 // The rotation that annihilates apq.
+template <bool LIFT>
 __device__ double2 jac_params(double app, double aqq, double apq) {
   double c = 1.0, sn = 0.0;
   if (apq != 0.0) {
@@ -200,10 +219,12 @@ __device__ double2 jac_params(double app, double aqq, double apq) {
     } else {
       t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
     }
-    c = 1.0 / sqrt(1.0 + t * t);
+    const double r = sqrt(1.0 + t * t);
+    c = 1.0 / r;
     sn = t * c;
+    if (LIFT) return make_double2(t / (1.0 + r), sn);
   }
-  return make_double2(c, sn);
+  return make_double2(LIFT ? 0.0 : c, sn);
 }
 
 // All blocks of the grid (a cooperative launch) wait until every one has arrived;
@@ -235,13 +256,15 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, u
 // One sweep: np - 1 steps, one grid-wide barrier each. A step reads A from one
 // buffer and writes the other, so everything in it is independent given its
 // rotations: the 2 x 2 blocks of A (pair k's rows by pair j's columns, a thread
-// each: J^T A J takes 16 fp64 operations on the four entries), the rows of V^T, and
-// the rotations of the next step, whose three entries of the new A are formed again
-// from the old one rather than waited for. Bound by the fp64 rate (6 operations per
-// entry and step) and the barrier. Measured at n = 640: 8.5 us a step, against 16.4
-// for two kernels a step (rotations, then whole rows in shared memory).
+// each), the rows of V^T, and the rotations of the next step, whose three entries of
+// the new A are formed again from the old one rather than waited for. Bound by the
+// fp64 rate and the barrier. Even sizes rotate by three shears (LIFT), 12 fp64
+// operations on a block of A instead of 16: 7.3 us a step at n = 640, 8.5 with four
+// operations a rotation, 16.4 with two kernels a step (rotations, then whole rows in
+// shared memory). Odd sizes keep the plain form.
 constexpr int kJacThreads = 512;
 
+template <bool LIFT>
 __global__ void __launch_bounds__(kJacThreads, 1)
     k_jacobi_sweep(double* __restrict__ A0, double* __restrict__ A1, double* __restrict__ Vt, int n, int np,
                    double2* __restrict__ cs0, double2* __restrict__ cs1, unsigned* count, unsigned* status) {
@@ -252,10 +275,10 @@ __global__ void __launch_bounds__(kJacThreads, 1)
   for (int k = blockIdx.x + gridDim.x * threadIdx.x; k < h; k += gridDim.x * kJacThreads) {
     int p, q;
     jac_pair(0, k, np, p, q);
-    double2 r = make_double2(1.0, 0.0);
+    double2 r = make_double2(LIFT ? 0.0 : 1.0, 0.0);
     if (q < n)
-      r = jac_params(__ldcg(A0 + static_cast<size_t>(p) * n + p), __ldcg(A0 + static_cast<size_t>(q) * n + q),
-                     __ldcg(A0 + static_cast<size_t>(p) * n + q));
+      r = jac_params<LIFT>(__ldcg(A0 + static_cast<size_t>(p) * n + p), __ldcg(A0 + static_cast<size_t>(q) * n + q),
+                           __ldcg(A0 + static_cast<size_t>(p) * n + q));
     __stcg(cs0 + k, r);
   }
   if (threadIdx.x == 0) s_task = 0;
@@ -277,14 +300,14 @@ __global__ void __launch_bounds__(kJacThreads, 1)
         for (int k = 32 * (blockIdx.x + pb * warp) + lane; k < h; k += 32 * pb * kWarps) {
           int p, q;
           jac_pair(s + 1, k, np, p, q);
-          double2 r = make_double2(1.0, 0.0);
+          double2 r = make_double2(LIFT ? 0.0 : 1.0, 0.0);
           if (q < n) {
-            JacEntry pp, qq, pq;
+            JacEntry<LIFT> pp, qq, pq;
             pp.load(A, n, np, s, cs, p, p);
             qq.load(A, n, np, s, cs, q, q);
             pq.load(A, n, np, s, cs, p, q);
             const double app = pp.value(), aqq = qq.value();
-            r = jac_params(app, aqq, pq.value());
+            r = jac_params<LIFT>(app, aqq, pq.value());
           }
           __stcg(csn + k, r);
         }
@@ -302,25 +325,25 @@ __global__ void __launch_bounds__(kJacThreads, 1)
         jac_pair(s, k, np, p, q);
         jac_pair(s, j, np, pj, qj);
         const size_t rp = static_cast<size_t>(p) * n, rq = static_cast<size_t>(q) * n;
-        if (q >= n) {  // a row without a partner
+        if (!LIFT && q >= n) {  // a row without a partner
           __stcg(B + rp + pj, __ldcg(A + rp + pj));
           if (qj < n) __stcg(B + rp + qj, __ldcg(A + rp + qj));
           continue;
         }
         const double2 ck = __ldcg(cs + k);
         double a = __ldcg(A + rp + pj), c = __ldcg(A + rq + pj);
-        if (qj < n) {
+        if (LIFT || qj < n) {
           const double2 cj = __ldcg(cs + j);
           double b = __ldcg(A + rp + qj), d = __ldcg(A + rq + qj);
-          jac_rotate(ck.x, ck.y, a, c);
-          jac_rotate(ck.x, ck.y, b, d);
-          jac_rotate(cj.x, cj.y, a, b);
-          jac_rotate(cj.x, cj.y, c, d);
+          jac_rotate<LIFT>(ck, a, c);
+          jac_rotate<LIFT>(ck, b, d);
+          jac_rotate<LIFT>(cj, a, b);
+          jac_rotate<LIFT>(cj, c, d);
           if (k == j && ck.y != 0.0) b = c = 0.0;  // the annihilated pair
           __stcg(B + rp + qj, b);
           __stcg(B + rq + qj, d);
         } else {
-          jac_rotate(ck.x, ck.y, a, c);
+          jac_rotate<LIFT>(ck, a, c);
         }
         __stcg(B + rp + pj, a);
         __stcg(B + rq + pj, c);
@@ -337,7 +360,7 @@ __global__ void __launch_bounds__(kJacThreads, 1)
             double* vp = Vt + static_cast<size_t>(p) * n + x;
             double* vq = Vt + static_cast<size_t>(q) * n + x;
             double a = __ldcg(vp), b = __ldcg(vq);
-            jac_rotate(ck.x, ck.y, a, b);
+            jac_rotate<LIFT>(ck, a, b);
             __stcg(vp, a);
             __stcg(vq, b);
           }
@@ -1030,13 +1053,14 @@ int jacobi_eigen(double* A, double* A2, double* Vt, int nn, double* cs, double* 
   double2* cs0 = reinterpret_cast<double2*>(cs);
   double2* cs1 = cs0 + np / 2;
   unsigned* count = reinterpret_cast<unsigned*>(red + 2);
+  const void* kernel = nn == np ? reinterpret_cast<const void*>(k_jacobi_sweep<true>)
+                                : reinterpret_cast<const void*>(k_jacobi_sweep<false>);
   double prev_off = -1.0;
   for (int sweep = 0; sweep < max_sweeps && nn > 1; ++sweep) {
     PCA_TRY(cudaMemsetAsync(red, 0, 4 * sizeof(double), st));
     int n = nn, npv = np;
     void* args[] = {&cur, &oth, &Vt, &n, &npv, &cs0, &cs1, &count, &status};
-    PCA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_jacobi_sweep), dim3(sms), dim3(kJacThreads), args,
-                                        0, st));
+    PCA_TRY(cudaLaunchCooperativeKernel(kernel, dim3(sms), dim3(kJacThreads), args, 0, st));
     std::swap(cur, oth);  // np - 1 steps, an odd number
     k_offnorm<<<304, 256, 0, st>>>(cur, nn, red);
     PCA_TRY(cudaGetLastError());
