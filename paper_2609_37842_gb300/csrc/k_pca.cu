@@ -258,11 +258,13 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, u
 // rotations: the 2 x 2 blocks of A (pair k's rows by pair j's columns, a thread
 // each), the rows of V^T, and the rotations of the next step, whose three entries of
 // the new A are formed again from the old one rather than waited for. Bound by the
-// fp64 rate and the barrier. Even sizes rotate by three shears (LIFT), 12 fp64
-// operations on a block of A instead of 16: 7.3 us a step at n = 640, 8.5 with four
-// operations a rotation, 16.4 with two kernels a step (rotations, then whole rows in
-// shared memory). Odd sizes keep the plain form.
-constexpr int kJacThreads = 512;
+// fp64 rate and the barrier (1.4 us). Even sizes rotate by three shears (LIFT), 12
+// fp64 operations on a block of A instead of 16. At n = 640: 6.6 us a step; 7.3 with
+// 512 threads and ten blocks for the rotations, 8.5 also with four operations a
+// rotation, 16.4 with two kernels a step (rotations, then whole rows in shared
+// memory). Longer tasks than 32 blocks of A or 64 columns of V^T cost 8 % (the last
+// ones run alone). Odd sizes keep the plain form.
+constexpr int kJacThreads = 768;
 
 template <bool LIFT>
 __global__ void __launch_bounds__(kJacThreads, 1)
@@ -286,7 +288,7 @@ __global__ void __launch_bounds__(kJacThreads, 1)
   const int jc = (h + 31) / 32;           // warp tasks of a pair's rows of A
   const int xc = (n + 63) / 64;           // and of V^T, two columns a lane
   const int nA = h * jc, nAll = nA + h * xc;
-  const int pb = max(1, min((h + 31) / 32, static_cast<int>(gridDim.x) / 8));  // blocks for the rotations
+  const int pb = max(1, min((h + 63) / 64, static_cast<int>(gridDim.x) / 8));  // blocks for the rotations: two warps each
   for (int s = 0; s < np - 1; ++s) {
     const double* A = s & 1 ? A1 : A0;
     double* B = s & 1 ? A0 : A1;
@@ -667,6 +669,7 @@ __device__ __forceinline__ void chol_block(float (&a)[32], int lane, int nb, uns
 }
 
 __global__ void __launch_bounds__(32) k_chol_diag(float* __restrict__ A, int lda, int n, int j0, unsigned* status) {
+  eogp::pdl_trigger();
   const int lane = threadIdx.x, nb = min(32, n - j0);
   float a[32];
 #pragma unroll
@@ -678,13 +681,19 @@ __global__ void __launch_bounds__(32) k_chol_diag(float* __restrict__ A, int lda
     if (lane < nb && j < nb) A[static_cast<long long>(j0 + lane) * lda + j0 + j] = a[j];
 }
 
-// Rows i >= j0 + 32: A[i][j0..j0+32) <- A[i][j0..j0+32) L_d^-T (forward
-// substitution, one thread per row; rows are 16-byte aligned).
+// Rows i >= j0 + 32: A[i][j0..j0+32) <- A[i][j0..j0+32) L_d^-T (one thread per row;
+// rows are 16-byte aligned). A finished column is taken out of all later ones at
+// once, in the same order for every element: one division and one product in the
+// chain per column, where a column at a time its own products are one (8.7 us at
+// n = 640). Panels and updates start behind one another; both changes take 5.6 us
+// off a pair of them.
 __global__ void __launch_bounds__(64) k_chol_panel(float* __restrict__ A, int lda, int n, int j0) {
-  __shared__ float L[32][33];
+  __shared__ __align__(16) float Lt[32][36];  // Lt[c][r] = L_d[r][c]
+  eogp::pdl_trigger();
+  eogp::pdl_wait();
   for (int e = threadIdx.x; e < 1024; e += 64) {
     const int r = e >> 5, c = e & 31;
-    L[r][c] = A[static_cast<long long>(j0 + r) * lda + j0 + c];
+    Lt[c][r] = A[static_cast<long long>(j0 + r) * lda + j0 + c];
   }
   const int i = j0 + 32 + blockIdx.x * 64 + threadIdx.x;
   float4* row = reinterpret_cast<float4*>(A + static_cast<long long>(i) * lda + j0);
@@ -700,10 +709,15 @@ __global__ void __launch_bounds__(64) k_chol_panel(float* __restrict__ A, int ld
   if (i >= n) return;
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
-    float v = x[c];
+    float l[32];
 #pragma unroll
-    for (int t = 0; t < c; ++t) v -= x[t] * L[c][t];
-    x[c] = v / L[c][c];
+    for (int t = c / 4; t < 8; ++t) {
+      const float4 v = *reinterpret_cast<const float4*>(&Lt[c][4 * t]);
+      l[4 * t] = v.x, l[4 * t + 1] = v.y, l[4 * t + 2] = v.z, l[4 * t + 3] = v.w;
+    }
+    x[c] = x[c] / l[c];
+#pragma unroll
+    for (int t = c + 1; t < 32; ++t) x[t] -= x[c] * l[t];
   }
 #pragma unroll
   for (int c = 0; c < 8; ++c) row[c] = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
@@ -715,6 +729,8 @@ __global__ void __launch_bounds__(64) k_chol_panel(float* __restrict__ A, int ld
 __global__ void __launch_bounds__(256) k_chol_update(float* __restrict__ A, int lda, int n, int j0, unsigned* status) {
   __shared__ float Pi[64][33];
   __shared__ float Pj[64][33];
+  eogp::pdl_trigger();
+  eogp::pdl_wait();
   const int j1 = j0 + 32;
   const int b = blockIdx.x;
   int ti = static_cast<int>((sqrtf(8.0f * b + 1.0f) - 1.0f) * 0.5f);
@@ -1150,8 +1166,8 @@ int chol_qr_pass(const SubLayout& L, char* w, const float* Y32, float* X32, floa
   k_chol_diag<<<1, 32, 0, st>>>(G, L.p4, p, 0, status);
   for (int j0 = 0; j0 + 32 < p; j0 += 32) {
     const int below = p - (j0 + 32), nt = (below + 63) / 64;
-    k_chol_panel<<<(below + 63) / 64, 64, 0, st>>>(G, L.p4, p, j0);
-    k_chol_update<<<nt * (nt + 1) / 2, 256, 0, st>>>(G, L.p4, p, j0, status);
+    PCA_TRY(launch_behind(k_chol_panel, (below + 63) / 64, 64, 0, st, G, L.p4, p, j0));
+    PCA_TRY(launch_behind(k_chol_update, nt * (nt + 1) / 2, 256, 0, st, G, L.p4, p, j0, status));
   }
   PCA_TRY(cudaGetLastError());
   PCA_TRY(cudaMemsetAsync(Li, 0, static_cast<size_t>(p) * L.p4 * 4, st));
