@@ -794,7 +794,7 @@ def timed_call(fn, stream, reps=3):
 
 
 def bench_query_scoring(w, N, Q, dev, stream, probes, bf16_burst, peaks_src, seed, paper=True):
-    """CODES scores (dense and with the top 20 fused) of Q one-bit queries against N
+    """CODES scores (dense and with the top 20) of Q one-bit queries against N
     stored codes of the workload's modules; PAPER mode (unquantised queries) too."""
     import torch
     from paper_2609_37842_gb300 import eogp as E
@@ -843,7 +843,7 @@ def bench_query_scoring(w, N, Q, dev, stream, probes, bf16_burst, peaks_src, see
 
 def bench_scan(dev, stream, probes, bf16_burst, peaks_src, hbm, rows=0, qs_arg=""):
     """The scoring-bound sweep: 4,194,304 stored 16,384-bit codes, Q in {1, 64, 1024,
-    8192} (chunks of 1024 queries), top 20 fused for Q >= 1024."""
+    8192} (chunks of 1024 queries), top 20 for Q >= 1024."""
     import torch
     from paper_2609_37842_gb300 import eogp as E
     from paper_2609_37842_gb300 import synth
@@ -870,7 +870,7 @@ def bench_scan(dev, stream, probes, bf16_burst, peaks_src, hbm, rows=0, qs_arg="
         byts = len(chunks) * (N * Wsc * 4 + N * 4) + Q * N * 4
         ent = {"ms": qms, "scores_per_s": N * Q / (qms / 1000.0), "GBps": byts / (qms / 1000.0) / 1e9,
                "frac_of_hbm": byts / (qms / 1000.0) / 1e9 / hbm}
-        if Q >= 64:   # tensor-core kernel: +-1 multiply-adds against the rate of the MMA it issues
+        if Q >= 17:   # tensor-core kernel: +-1 multiply-adds against the rate of the MMA it issues
             tfl = 2.0 * N * ksc * Q / (qms / 1000.0) / 1e12
             pk, pk_src, pk_mode = score_peak([ksc], probes, bf16_burst, peaks_src)
             kern = ("k_score_pair_ks" if Q <= 64 else "k_score_pair") if "mxf4" in pk_mode else "k_score_tc"
@@ -881,7 +881,7 @@ def bench_scan(dev, stream, probes, bf16_burst, peaks_src, hbm, rows=0, qs_arg="
             ent.update({"kernel": "k_score_codes_smallq (popcount)", "word_ops_per_s": wops})
             if probes:
                 ent["popc_frac"] = wops / probes["popc_words_per_s"]
-        if Q >= 1024:  # per-query top 20 in the scoring epilogue: no Q x N output
+        if Q >= 1024:  # per-query top 20: no Q x N output to the caller
             K = 20
             wt = E.workspace(E.score_topk_workspace_size(N, [ksc], E.SCORE_CODES, Q, K), dev)
             kms = timed_call(lambda: E.score_topk(tr, tsc, [ksc], E.SCORE_CODES, qc, K, query_scales=qs, ws=wt),
