@@ -106,11 +106,12 @@ int eogp_profile_read(int kind, int* launches, double* total_ms, int reset);
  *     kernel. 0 (default): e2m1 (kind::mxf4, unit scales) when every module is
  *     a multiple of 256 bits and the stored rows are 16-byte aligned, else
  *     e4m3; 1: always e4m3 (kind::f8f6f4). Scores are bit-identical.
- *   EOGP_OPT_TOPK_PATH: ranking path of eogp_score_topk. 0 (default) and 2: dense
- *     scores, up to 1 GiB of them at a time, then a ranking kernel; 1: ranking
- *     fused into the tensor-core scoring kernel where it applies (slower, but a
- *     workspace of tens of MB). With 0, requests the fused kernel could take are
- *     refused beyond 49,152 rows that are not aligned for it.
+ *   EOGP_OPT_TOPK_PATH: ranking path of eogp_score_topk. 2: dense scores, up to 1
+ *     GiB of them at a time, then a ranking kernel; 1: ranking fused into the
+ *     tensor-core scoring kernel where it applies (mostly slower, but a workspace
+ *     of tens of MB); 0 (default): the faster one, dense but for 1024 or more
+ *     queries over millions of rows of one wide module. With 0, requests the fused
+ *     kernel could take are refused beyond 49,152 rows that are not aligned for it.
  * eogp_set_option returns EOGP_EINVAL for an unknown option or value. */
 #define EOGP_OPT_SCORE_OPERAND 0
 #define EOGP_OPT_TOPK_PATH     1
@@ -530,9 +531,9 @@ int eogp_score_topk_workspace_size(int N, const int* k_per_module, int U, int mo
 
 /* Per query, the `topk` best stored rows under the eogp_score definition of
  * `mode`. The scores of as many stored rows as fit 1 GiB of workspace are formed
- * and ranked at a time; with EOGP_OPT_TOPK_PATH = 1, where the tensor-core
- * kernels apply and topk <= 32, the ranking runs in their epilogue instead, with
- * no scores written and a workspace of tens of MB. Arguments as eogp_score, plus:
+ * and ranked at a time; with EOGP_OPT_TOPK_PATH = 1 (or 0 and millions of rows),
+ * where the tensor-core kernels apply and topk <= 32, the ranking runs in their
+ * epilogue instead, with no scores written and a workspace of tens of MB. Arguments as eogp_score, plus:
  *   top_scores [Q x ld_top_scores] fp32 device and top_index [Q x ld_top_index]
  *   int32 device (stored row numbers), ld >= topk: row q lists its best rows by
  *   score descending, equal scores by lower row number; NaN scores never rank;

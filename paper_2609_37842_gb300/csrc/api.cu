@@ -1397,9 +1397,12 @@ struct TopkPlan {
 // tensor-core kernel's epilogue, no scores in memory; there it holds up the MMAs
 // while the lists fill. Measured, top 20, fused / dense in us: 64 queries over
 // 300K rows of 16,384 bits 657 / 258, 1024 queries 3,756 / 1,853, 1024 over
-// 2M rows 12,236 / 11,984; 64 over 20,000 rows of 48 x 1024 bits 378 / 148. So the
-// dense path is the default; EOGP_OPT_TOPK_PATH = 1 selects the fused one where it
+// 2M rows 12,236 / 11,984, 3M 17,065 / 17,773, 4.2M 22,903 / 24,460 (the scores' way
+// through memory); 256 over 4.2M 7,352 / 6,127; 1024 over 4M rows of 4,096 bits 14,606
+// / 13,148; 64 over 20,000 rows of 48 x 1024 bits 378 / 148. So the default is dense
+// but for kTopkFused*; EOGP_OPT_TOPK_PATH = 1 selects the fused path wherever it
 // applies.
+constexpr int kTopkFusedMinN = 2500000, kTopkFusedMinQ = 1024, kTopkFusedMinBits = 16384;  // of one module
 constexpr size_t kTopkDenseMax = size_t(1) << 30;
 // Stored rows up to which any row alignment is ranked; more of them in a request
 // the fused path supports need the alignment of the tensor cores on every path.
@@ -1420,7 +1423,8 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
   // alignment allows.
   const bool can = tc_ok && score_tc_topk_fits(mode, ks, U, Q, K) && force != 0 &&
                    (mode != EOGP_SCORE_CODES || Q >= 64);
-  p.fused = can && force == 1;
+  const bool wide = U == 1 && ks[0] >= kTopkFusedMinBits && Q >= kTopkFusedMinQ && N >= kTopkFusedMinN;
+  p.fused = can && (force == 1 || (wide && mode == EOGP_SCORE_CODES));
   p.tc_rows = can && (force == 1 || N > kTopkAnyRowsMaxN);
   p.q_bytes = tc_ok ? score_tc_ws_bytes(mode, ks, U, Q) : 0;
   if (p.fused) {
