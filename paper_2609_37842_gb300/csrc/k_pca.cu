@@ -157,9 +157,10 @@ __device__ __forceinline__ void jac_rotate(double2 r, double& x, double& y) {
 }
 
 // Entry (x, y) after step s, formed from A before it and the step's rotations:
-// rows x and its partner rotated, then columns y and its partner. A row without a
-// partner (odd n) stays as it is. Loads and arithmetic apart, so that the loads of
-// several entries are in flight together.
+// rows x and its partner rotated, then columns y and its partner. The index without a
+// partner (odd n) has no rotation of its own; its row takes the column rotations and
+// its column the row rotations, like any other. Loads and arithmetic apart, so that
+// the loads of several entries are in flight together.
 template <bool LIFT>
 struct JacEntry {
   double a, b, c, d;  // rows (x's pair) by columns (y's pair)
@@ -192,7 +193,10 @@ struct JacEntry {
       if (zero && ck.y != 0.0) return 0.0;  // the annihilated pair
       return rotated(cj, low_col, l, h);
     }
-    if (row_alone) return low_col ? a : b;
+    if (row_alone) {
+      if (!col_alone) jac_rotate<LIFT>(cj, a, b);
+      return low_col ? a : b;
+    }
     jac_rotate<LIFT>(ck, a, c);
     if (col_alone) return low_row ? a : c;
     jac_rotate<LIFT>(ck, b, d);
@@ -327,9 +331,14 @@ __global__ void __launch_bounds__(kJacThreads, 1)
         jac_pair(s, k, np, p, q);
         jac_pair(s, j, np, pj, qj);
         const size_t rp = static_cast<size_t>(p) * n, rq = static_cast<size_t>(q) * n;
-        if (!LIFT && q >= n) {  // a row without a partner
-          __stcg(B + rp + pj, __ldcg(A + rp + pj));
-          if (qj < n) __stcg(B + rp + qj, __ldcg(A + rp + qj));
+        if (!LIFT && q >= n) {  // a row without a partner: its columns' rotations only
+          double a = __ldcg(A + rp + pj);
+          if (qj < n) {
+            double b = __ldcg(A + rp + qj);
+            jac_rotate<LIFT>(__ldcg(cs + j), a, b);
+            __stcg(B + rp + qj, b);
+          }
+          __stcg(B + rp + pj, a);
           continue;
         }
         const double2 ck = __ldcg(cs + k);
