@@ -407,7 +407,9 @@ int eogp_fit_pca_workspace_size(int n, int m, int k, size_t* bytes);
  * eigensolver on the device, in fp64. This call BLOCKS the host until the fit
  * is done (it reads a convergence measure once per sweep).
  * Errors: EOGP_EINVAL (k < 1 or k > min(n, m), ldz < m, ld_pt < m),
- * EOGP_EWORKSPACE, EOGP_EUNSUPPORTED (min(n, m) > 12288), EOGP_ECUDA. */
+ * EOGP_EWORKSPACE, EOGP_EUNSUPPORTED (min(n, m) > 12288), EOGP_EDEVICE (Z, or its
+ * second moment in the arithmetic of the fit, holds an infinity or a NaN; Pt and eig
+ * are then not written), EOGP_ECUDA. */
 int eogp_fit_pca(const float* Z, int n, int m, int ldz, int k, void* Pt, int ld_pt, int pt_dtype,
                  float* eig, void* ws, size_t ws_bytes, eogp_stream_t stream);
 
@@ -420,7 +422,8 @@ int eogp_fit_pca(const float* Z, int n, int m, int ldz, int k, void* Pt, int ld_
  *   eogp_fit_pca_from_moment: Pt, eig as eogp_fit_pca for the matrix C / n_total
  *     (n_total = rows summed into C); workspace from
  *     eogp_fit_pca_from_moment_workspace_size; m <= 12288; blocks the host.
- * Errors: EOGP_EINVAL, EOGP_EUNSUPPORTED, EOGP_EWORKSPACE, EOGP_ECUDA. */
+ * Errors: EOGP_EINVAL, EOGP_EUNSUPPORTED, EOGP_EWORKSPACE, EOGP_EDEVICE (as above),
+ * EOGP_ECUDA. */
 int eogp_second_moment(const float* Z, int n, int m, int ldz, double* C, int ldc, int accumulate,
                        eogp_stream_t stream);
 int eogp_fit_pca_from_moment_workspace_size(int m, int k, size_t* bytes);

@@ -411,7 +411,8 @@ __global__ void __launch_bounds__(256) k_offnorm(const double* __restrict__ A, i
   }
 }
 
-// mu[i] = A[i][i]; sel[rank(i)] = i for the k largest (descending, ties to lower index).
+// mu[i] = A[i][i]; sel[rank(i)] = i for the k largest (descending, ties to lower index,
+// NaN below every number: the ranks are a permutation whatever A holds).
 __global__ void k_rank(const double* __restrict__ A, int n, int k, double* __restrict__ mu,
                        int* __restrict__ sel) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -421,7 +422,9 @@ __global__ void k_rank(const double* __restrict__ A, int n, int k, double* __res
   int rank = 0;
   for (int j = 0; j < n; ++j) {
     const double vj = A[static_cast<size_t>(j) * n + j];
-    rank += (vj > vi) || (vj == vi && j < i);
+    const bool above = vj > vi || (vi != vi && vj == vj);
+    const bool tie = vj == vi || (vi != vi && vj != vj);
+    rank += above || (tie && j < i);
   }
   if (rank < k) sel[rank] = i;
 }
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(256) k_emit(const TS* __restrict__ src, int ld
   const int r = blockIdx.x;
   const TS* v = src + static_cast<size_t>(sel ? sel[r] : r) * ld_src;
   double ss = 0.0, mx = -1.0;
-  int ix = 0x7fffffff;
+  int ix = 0;  // also the place read for a row without a number
   for (int c = threadIdx.x; c < m; c += blockDim.x) {
     const double x = static_cast<double>(v[c]);
     ss = fma(x, x, ss);
@@ -1081,17 +1084,21 @@ int jacobi_eigen(double* A, double* A2, double* Vt, int nn, double* cs, double* 
   const void* kernel = nn == np ? reinterpret_cast<const void*>(k_jacobi_sweep<true>)
                                 : reinterpret_cast<const void*>(k_jacobi_sweep<false>);
   double prev_off = -1.0;
-  for (int sweep = 0; sweep < max_sweeps && nn > 1; ++sweep) {
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     PCA_TRY(cudaMemsetAsync(red, 0, 4 * sizeof(double), st));
-    int n = nn, npv = np;
-    void* args[] = {&cur, &oth, &Vt, &n, &npv, &cs0, &cs1, &count, &status};
-    PCA_TRY(cudaLaunchCooperativeKernel(kernel, dim3(sms), dim3(kJacThreads), args, 0, st));
-    std::swap(cur, oth);  // np - 1 steps, an odd number
+    if (nn > 1) {
+      int n = nn, npv = np;
+      void* args[] = {&cur, &oth, &Vt, &n, &npv, &cs0, &cs1, &count, &status};
+      PCA_TRY(cudaLaunchCooperativeKernel(kernel, dim3(sms), dim3(kJacThreads), args, 0, st));
+      std::swap(cur, oth);  // np - 1 steps, an odd number
+    }
     k_offnorm<<<304, 256, 0, st>>>(cur, nn, red);
     PCA_TRY(cudaGetLastError());
     double h[2];
     PCA_TRY(cudaMemcpyAsync(h, red, sizeof(h), cudaMemcpyDeviceToHost, st));
     PCA_TRY(cudaStreamSynchronize(st));
+    if (!std::isfinite(h[1]))
+      return eogp::set_error(EOGP_EDEVICE, "fit_pca: values that are not finite (in the input or its second moment)");
     const double off = std::sqrt(h[0]), tot = std::sqrt(h[1]);
     if (!(off > 1e-11 * tot)) break;
     if (prev_off >= 0.0 && sweep >= 4 && off > 0.5 * prev_off) break;  // rounding floor
