@@ -355,12 +355,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // Query q's three bf16 parts, in rows part * QB + q % QB of query tile q / QB
-// (rows of Dp values, zero past D; the rows of a tile past Q are zero), and
-// whether the part block (x, q) splits holds a value that is not finite. Clears the row tiles' notes.
+// (rows of Dp values, zero past D; the rows of a tile past Q are zero), and whether
+// the part of it that block (q, y) splits holds a value that is not finite. Clears the
+// row tiles' notes. Queries are on grid.x: whole tiles of 65,535 are 65,536 of them.
 __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict__ y, int ldq, int Q, int D, int Dp,
                                                         int QB, uint16_t* __restrict__ parts, int* __restrict__ qbad,
                                                         int* __restrict__ rbad, int nrt) {
-  const int q = blockIdx.y, c0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x), nthr = gridDim.x * blockDim.x;
+  const int q = blockIdx.x, c0 = 2 * (blockIdx.y * blockDim.x + threadIdx.x), nthr = gridDim.y * blockDim.x;
   uint16_t* o = parts + (static_cast<size_t>(q / QB) * 3 * QB + q % QB) * Dp;
   const size_t step = static_cast<size_t>(QB) * Dp;
   int bad = 0;
@@ -377,8 +378,8 @@ __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict_
     *reinterpret_cast<uint32_t*>(o + 2 * step + c) = pack_hi(h3[0], h3[1]);
   }
   bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) qbad[static_cast<size_t>(blockIdx.x) * gridDim.y + q] = bad;
-  for (int i = (q * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x; i < nrt; i += gridDim.y * nthr) rbad[i] = 0;
+  if (threadIdx.x == 0) qbad[static_cast<size_t>(blockIdx.y) * gridDim.x + q] = bad;
+  for (int i = (q * gridDim.y + blockIdx.y) * blockDim.x + threadIdx.x; i < nrt; i += gridDim.x * nthr) rbad[i] = 0;
 }
 
 // scores[q][i] = the slabs' values in order; four scores a thread (ldp is a
@@ -484,7 +485,7 @@ cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const flo
   int* rbad = reinterpret_cast<int*>(w + p.rbad);
   float* part = reinterpret_cast<float*>(w + p.part);
   const int sb = std::min(kSplitBlocks, (p.Dp / 2 + 255) / 256);
-  k_split3_queries<<<dim3(sb, p.nqt * p.QB), 256, 0, st>>>(query, ldq, Q, D, p.Dp, p.QB, parts, qbad, rbad, p.nrt);
+  k_split3_queries<<<dim3(p.nqt * p.QB, sb), 256, 0, st>>>(query, ldq, Q, D, p.Dp, p.QB, parts, qbad, rbad, p.nrt);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   CUtensorMap tx, ty;
