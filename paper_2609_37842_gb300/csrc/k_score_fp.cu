@@ -2,35 +2,43 @@
 //
 // Precision. Both sides stay 32-bit values: each fp32 number is the exact sum of
 // three bf16 numbers (its 24-bit significand cut into 8 + 8 + 8 bits by
-// truncation, x = x1 + x2 + x3), and the six products down to 2^-16 of the
-// leading one are formed, every one of them exact in fp32:
-//   d0 += x1 y1,   d1 += x1 y2 + x2 y1,   d2 += x1 y3 + x2 y2 + x3 y1
-// (what is left out, x2 y3 and below, is 2^-24 of the product). The three
-// magnitudes have accumulators of their own, and every 256 coordinates they are
-// added in fp32 registers with round to nearest, so the tensor core's own
-// accumulation never runs over more than 16 steps. Error against 64-bit sums
-// (relative 2-norm, normal values): 2.7e-7 at 512 coordinates, 2.9e-7 at 49,152;
-// k_simt_gemm, one fp32 chain per score, has 4.0e-7 and 4.0e-6.
-// Infinities and NaN have no such split: a row tile or query that holds one is
-// noted, and k_simt_gemm computes its scores again afterwards.
+// truncation, x = x1 + x2 + x3), and eight of the nine products are formed, every
+// one of them exact in fp32:
+//   d0 += x1 y1,   d1 += x1 y2 + x2 y1,   d2 += x1 y3 + x2 y2 + x3 y1,   d3 += x2 y3 + x3 y2
+// (with 64 queries a tile the last two go to d2). |x2| < 2^-7 |x| and |x3| < 2^-15 |x|:
+// what is left out, x3 y3, is below 2^-30 of the product. Without x2 y3 and x3 y2, up
+// to 2^-21 together and of the product's sign, a score of one coordinate was off by as
+// much as 4.2e-7. The magnitudes have accumulators of their own, and every 256
+// coordinates they are added in fp32 registers with round to nearest, so the tensor
+// core's own accumulation never runs over more than 16 steps. Largest error against
+// 64-bit sums, of the sum of magnitudes, in brackets that of k_simt_gemm (one fp32
+// chain per score): one coordinate among 512 5.9e-8 (5.9e-8), two 1.5e-7 (1.1e-7), eight
+// 1.5e-7 (2.0e-7), all 512 1.0e-7 (2.5e-7), 49,152 1.2e-8 (3.0e-7). Sums near the end of
+// fp32's range are within a few units of 2^-149 a product.
+// Infinities, NaN and tiny values with bits below 2^-133, where bf16 ends, have no such
+// split: it leaves bits in the lower half of x3. A row tile or query that holds one
+// is noted, and k_simt_gemm computes its scores again afterwards.
 //
-// Bound: HBM (the stored coordinates, once per 64 queries). One CTA takes 128
-// stored rows (MMA M, operand A in TMEM) against QB <= 64 queries; the query
-// parts lie stacked as 3 QB rows of one operand B, so a K = 16 step is three
-// MMAs: x1 by all 3 QB rows, x2 by the first 2 QB, x3 by the first QB, each into
-// the columns one part further on. 48 queries against 16,384 x 49,152 stored
-// coordinates (3.2 GB): 544 us, 0.87 of the measured copy rate (0.95 of it are the
-// K ranges' last wave), against 5,702 us on the CUDA cores.
+// Bound: HBM (the stored coordinates, once per 64 queries), and from 48 queries on the
+// power limit. One CTA takes 128 stored rows (MMA M, operand A in TMEM) against QB <=
+// 64 queries; the query parts lie stacked as 3 QB rows of one operand B, so a K = 16
+// step is three MMAs: x1 and x2 by all 3 QB rows, x3 by the first 2 QB, each into the
+// columns one part further on. (A tile of 64 queries has no TMEM for d3 without a longer
+// drain: five MMAs, 660 us against 710 for 64 queries.) 16,384 x 49,152 stored
+// coordinates (3.2 GB), passes behind one another: 16 queries 539 us, 48 574 to 599 as
+// the clock falls (alone 555 us at 1.79 GHz; the six larger products 565, alone 542 at
+// 1.84), 0.83 of the measured copy rate, against 5,702 us on the CUDA cores.
 //
 // Pipeline per CTA (persistent over (row tile, K range, query tile) items):
 //  * TMA producer: fp32 boxes of 128 rows x 32 coordinates (128-byte swizzle) in a
 //    ring of eight or ten, and query tiles of 3 QB rows x 64 coordinates in a ring of three;
 //  * eight converter warps in two groups that take the boxes in turn (one warp per
 //    TMEM lane quarter): shared memory -> three bf16 parts -> TMEM, 48 columns a box;
-//  * one issuing warp (converged, MMAs under elect.sync): 12 MMAs per pair of boxes
-//    (one query tile) and round of wait, fence and commit. With 6 per round the
-//    rounds set the pace, 646 us for the case above whatever the number of queries;
-//  * four drain warps: every 256 coordinates the three accumulators of a row into
+//  * one issuing warp (converged, MMAs under elect.sync): 12 MMAs (20 with 64
+//    queries) per pair of boxes (one query tile) and round of wait, fence and commit.
+//    With 6 per round, one box, the rounds set the pace, 646 us for the case above
+//    whatever the number of queries;
+//  * four drain warps: every 256 coordinates the accumulators of a row into
 //    registers; at the item's end the sums to the scores or to the K range's slab.
 #include <algorithm>
 
@@ -51,13 +59,21 @@ constexpr int kDrainBoxes = 8;                  // boxes (of 32 coordinates) per
 constexpr int kSplitBlocks = 16;                // blocks per query of the query split, at most
 constexpr int kMinD = 512;                      // fewer coordinates stay on k_simt_gemm
 
-// TMEM: two accumulator sets of 3 QB columns (one with 64 queries: its drain then
-// holds up the next run's MMAs), and A slots of 96 columns, each two boxes.
+// TMEM: two accumulator sets of 4 QB columns, one with 48 queries, one of 3 QB with 64
+// (its drain then holds up the next run's MMAs), and A slots of 96 columns, each two
+// boxes.
+template <int QB>
+constexpr int fp_parts() {
+  return QB == 64 ? 3 : 4;
+}
 template <int QB>
 constexpr int fp_accs() {
-  return QB == 64 ? 1 : 2;
+  return QB >= 48 ? 1 : 2;
 }
-constexpr int kSlots = 2;
+template <int QB>
+constexpr int fp_slots() {
+  return QB == 48 ? 3 : 2;
+}
 template <int QB>
 constexpr int fp_xring() {
   return QB == 64 ? 8 : 10;
@@ -69,7 +85,7 @@ constexpr uint32_t fp_ybox() {
 template <int QB>
 constexpr size_t fp_smem() {
   return 1024 + fp_xring<QB>() * kXBox + kYRing * static_cast<size_t>(fp_ybox<QB>()) +
-         (2 * fp_xring<QB>() + 2 * kYRing + 2 * kSlots + 4) * 8 + 16;
+         (2 * fp_xring<QB>() + 2 * kYRing + 2 * fp_slots<QB>() + 4) * 8 + 16;
 }
 
 struct FpArgs {
@@ -77,7 +93,7 @@ struct FpArgs {
   float* out;    // scores, or with S > 1 the slabs [S][Q][ldo]
   size_t slab;
   int ldo;
-  int* rbad;     // [nrt]: the row tile holds a value that is not finite
+  int* rbad;     // [nrt]: the row tile holds a value without a split
   unsigned* status;
 };
 
@@ -94,7 +110,8 @@ __device__ __forceinline__ void mma_f16_ta(uint32_t d, uint32_t a, uint64_t b, u
       : "memory");
 }
 
-// Exact three-way split of a finite x: upper halves of x, x - x1 and x - x1 - x2.
+// Three-way split: upper halves of x, x - x1 and x - x1 - x2. Exact if and only if the
+// lower half of h3 is zero (an infinity or a NaN makes h3 the canonical NaN 0x7FFFFFFF).
 __device__ __forceinline__ void split3(float x, uint32_t& h1, uint32_t& h2, uint32_t& h3) {
   h1 = __float_as_uint(x) & 0xFFFF0000u;
   const float r = __fsub_rn(x, __uint_as_float(h1));
@@ -107,8 +124,8 @@ __device__ __forceinline__ uint32_t pack_hi(uint32_t lo, uint32_t hi) { return _
 template <int QB>
 __global__ void __launch_bounds__(kThreads, 1)
     k_score_fp(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, const FpArgs g) {
-  constexpr int ND = fp_accs<QB>(), kXRing = fp_xring<QB>();
-  constexpr uint32_t kAcc = 3u * QB;             // columns of an accumulator set
+  constexpr int ND = fp_accs<QB>(), kXRing = fp_xring<QB>(), kSlots = fp_slots<QB>();
+  constexpr uint32_t kAcc = fp_parts<QB>() * QB;             // columns of an accumulator set
   constexpr uint32_t kA0 = ND * kAcc;            // first A column
   static_assert(kXRing % 2 == 0, "each converter group owns every second box");
   static_assert(kA0 + 96u * kSlots <= 512u, "TMEM budget");
@@ -183,16 +200,21 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t d = tmem + lane_base + buf * kAcc;
 #pragma unroll
         for (int c = 0; c < QB; c += 16) {
-          uint32_t v0[16], v1[16], v2[16];
+          uint32_t v0[16], v1[16], v2[16], v3[16];
           tmem_ld16_issue(d + c, v0);
           tmem_ld16_issue(d + QB + c, v1);
           tmem_ld16_issue(d + 2 * QB + c, v2);
+          if constexpr (fp_parts<QB>() == 4) tmem_ld16_issue(d + 3 * QB + c, v3);
           tmem_wait_ld(v0);
           tmem_wait_ld(v1);
           tmem_wait_ld(v2);
+          if constexpr (fp_parts<QB>() == 4) tmem_wait_ld(v3);
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            sum[c + j] += __uint_as_float(v0[j]) + (__uint_as_float(v1[j]) + __uint_as_float(v2[j]));
+          for (int j = 0; j < 16; ++j) {
+            float low = __uint_as_float(v2[j]);
+            if constexpr (fp_parts<QB>() == 4) low += __uint_as_float(v3[j]);
+            sum[c + j] += __uint_as_float(v0[j]) + (__uint_as_float(v1[j]) + low);
+          }
         }
         tc_fence_before();
         __syncwarp();
@@ -221,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int item = blockIdx.x; item < g.n_items && ok; item += gridDim.x) {
       int b0, b1;
       item_boxes(item, b0, b1);
-      float bad = 0.f;  // NaN once a value is not finite
+      uint32_t bad = 0;  // lower half: bits that a value's three parts leave out
       for (int b = b0; b < b1; ++b, ++it) {
         if ((it & 1u) != static_cast<uint32_t>(grp)) continue;
         const uint32_t pr = it >> 1;  // pair of boxes = A slot use
@@ -242,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             split3(v[e], h1[e], h2[e], h3[e]);
-            bad = fmaf(v[e], 0.f, bad);
+            bad |= h3[e];
           }
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
@@ -267,13 +289,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&afull[as]);
       }
-      if (__any_sync(0xffffffffu, bad != bad) && lane == 0) g.rbad[item / (g.nqt * g.S)] = 1;
+      if (__any_sync(0xffffffffu, (bad & 0xFFFFu) != 0) && lane == 0) g.rbad[item / (g.nqt * g.S)] = 1;
     }
   } else if (warp == kMmaW) {
     // ---------------------------------------------------------- issuer
     {
-      const uint32_t id1 = idesc_bf16_f32(128, 3 * QB, 0, 0), id2 = idesc_bf16_f32(128, 2 * QB, 0, 0),
-                     id3 = idesc_bf16_f32(128, QB, 0, 0);
+      const uint32_t id3 = idesc_bf16_f32(128, 3 * QB, 0, 0), id2 = idesc_bf16_f32(128, 2 * QB, 0, 0),
+                     id1 = idesc_bf16_f32(128, QB, 0, 0);
+      constexpr uint64_t kPart = (QB * 128) >> 4;  // a query part on, whole swizzle atoms
       const uint64_t ydesc = sdesc_sw128(smem_u32(ysm), 16, 1024);
       uint32_t pr = 0, run = 0;  // pairs of boxes (and query tiles), accumulation runs of earlier items
       bool ok = true;
@@ -304,9 +327,23 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int kk = 0; kk < 4; ++kk) {
                 const uint64_t y = y0 + 2 * kk;  // K = 16: 32 bytes on
                 const uint32_t a = a0 + 48u * (kk >> 1) + 8u * (kk & 1);
-                mma_f16_ta(d, a, y, id1, (bb != b || kk != 0) ? 1u : 0u);
-                mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
-                mma_f16_ta(d + 2 * QB, a + 32u, y, id3, 1u);
+                const bool start = kk == 0 && bb == b;  // of a run
+                if constexpr (fp_parts<QB>() == 3) {
+                  mma_f16_ta(d, a, y, id3, start ? 0u : 1u);
+                  mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
+                  mma_f16_ta(d + 2 * QB, a + 32u, y, id1, 1u);
+                  mma_f16_ta(d + 2 * QB, a + 16u, y + 2 * kPart, id1, 1u);
+                  mma_f16_ta(d + 2 * QB, a + 32u, y + kPart, id1, 1u);
+                } else {
+                  mma_f16_ta(d, a, y, id3, start ? 0u : 1u);
+                  if (start) {  // d1 and d2 hold x1's products already, d3 starts here
+                    mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
+                    mma_f16_ta(d + 3 * QB, a + 16u, y + 2 * kPart, id1, 0u);
+                  } else {
+                    mma_f16_ta(d + QB, a + 16u, y, id3, 1u);
+                  }
+                  mma_f16_ta(d + 2 * QB, a + 32u, y, id2, 1u);
+                }
               }
               tc_commit(&aempty[as]);
               tc_commit(&yempty[ys]);
@@ -356,7 +393,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // Query q's three bf16 parts, in rows part * QB + q % QB of query tile q / QB
 // (rows of Dp values, zero past D; the rows of a tile past Q are zero), and whether
-// the part of it that block (q, y) splits holds a value that is not finite. Clears the
+// the part of it that block (q, y) splits holds a value without a split. Clears the
 // row tiles' notes. Queries are on grid.x: whole tiles of 65,535 are 65,536 of them.
 __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict__ y, int ldq, int Q, int D, int Dp,
                                                         int QB, uint16_t* __restrict__ parts, int* __restrict__ qbad,
@@ -371,7 +408,7 @@ __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict_
     for (int e = 0; e < 2; ++e) {
       const float v = (q < Q && c + e < D) ? y[static_cast<size_t>(q) * ldq + c + e] : 0.f;
       split3(v, h1[e], h2[e], h3[e]);
-      bad |= (__float_as_uint(v) & 0x7F800000u) == 0x7F800000u;
+      bad |= static_cast<int>(h3[e] & 0xFFFFu);
     }
     *reinterpret_cast<uint32_t*>(o + c) = pack_hi(h1[0], h1[1]);
     *reinterpret_cast<uint32_t*>(o + step + c) = pack_hi(h2[0], h2[1]);
@@ -521,7 +558,7 @@ cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const flo
     e = launch_sum_slabs(part, p.S, g.slab, p.ldp, N, Q, out, ldo, st);
     if (e != cudaSuccess) return e;
   }
-  // scores of rows and queries with an infinity or a NaN, in fp32
+  // scores of rows and queries with a value without a split, one fp32 chain each
   return launch_simt_gemm_noted(Q, N, D, query, ldq, train, ldt, out, ldo, qbad, sb, p.nqt * p.QB, rbad,
                                 128, st);
 }
