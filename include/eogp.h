@@ -477,9 +477,10 @@ int eogp_score_workspace_size(int N, const int* k_per_module, int U, int mode, i
  *          coordinates [Q x ld_query] (module u at column sum_{v<u} k_v),
  *          query_scales ignored; scores[q][i] = sum_u s_iu <y_qu, b_iu>.
  *          With every k_u a multiple of 64 and the workspace
- *          eogp_score_workspace_size reports (4 Q sum_u k_u bytes), this runs on
- *          the tensor cores with y split into bf16 hi + lo (about 2^-17 relative)
- *          and fp32 sums: |error| <= 1e-5 sum_u s_iu ||y_qu||_1 for k_u <= 16384.
+ *          eogp_score_workspace_size reports (or 4 Q sum_u k_u bytes, rounded up to
+ *          256, which divides no sum), this runs on the tensor cores with y split
+ *          into bf16 hi + lo (about 2^-17 relative) and fp32 sums:
+ *          |error| <= 1e-5 sum_u s_iu ||y_qu||_1 for k_u <= 16384.
  *   FP:    train = fp32 coordinates [N x ld_train], query = fp32 [Q x ld_query];
  *          scores[q][i] = <y_q, x_i>; scales ignored. With 512 coordinates or
  *          more, ld_train % 4 == 0, a 16-byte aligned base and the workspace
@@ -499,6 +500,10 @@ int eogp_score_workspace_size(int N, const int* k_per_module, int U, int mode, i
  * the tensor cores multiplies exact +-1 operands: e2m1 through the block-scaled
  * fp4 MMA with unit scales when every k_u is a multiple of 256, else e4m3; the
  * scores are the same bit for bit either way.
+ * PAPER and FP on the tensor cores: how the sum over coordinates is divided and added
+ * follows from N, Q, the modules and the workspace alone. So equal rows have equal
+ * scores within a call, and a call repeats bit for bit, but a shard's scores may
+ * differ in their last bits from those of a call over the whole store.
  * Errors: EOGP_EINVAL, EOGP_EWORKSPACE, EOGP_ECUDA. */
 int eogp_score(const void* train, int ld_train, const float* train_scales, int ld_tscale, int N,
                const int* k_per_module, int U, int mode, const void* query, int ld_query,
@@ -543,8 +548,10 @@ int eogp_score_topk_workspace_size(int N, const int* k_per_module, int U, int mo
  *   top_scores [Q x ld_top_scores] fp32 device and top_index [Q x ld_top_index]
  *   int32 device (stored row numbers), ld >= topk: row q lists its best rows by
  *   score descending, equal scores by lower row number; NaN scores never rank;
- *   places beyond N hold (-inf, -1). CODES scores are bitwise those of
- *   eogp_score, so the lists are exact.
+ *   places beyond N hold (-inf, -1). The scores are bitwise those of one eogp_score
+ *   call over the N rows with the workspace it asks for (PAPER with
+ *   EOGP_OPT_TOPK_PATH = 1: up to their last bits), however many rows are formed at
+ *   a time.
  * ws: 256-byte aligned, at least eogp_score_topk_workspace_size bytes.
  * Errors: EOGP_EINVAL (topk outside [1, EOGP_TOPK_MAX], bad sizes),
  *   EOGP_EWORKSPACE, EOGP_EUNSUPPORTED (tensor-core shape with code rows not

@@ -1291,18 +1291,19 @@ extern "C" int eogp_score_workspace_size(int N, const int* k_per_module, int U, 
       U <= 1024 && score_tc_supported(mode, k_per_module, U, Q))
     *bytes = score_tc_ws_bytes(mode, k_per_module, U, Q);
   if (mode == EOGP_SCORE_PAPER && *bytes && N > 0)
-    *bytes = std::max(*bytes, score_paper_ws_bytes(N, k_per_module, U, Q, sm_count()));
+    *bytes = std::max(*bytes, score_paper_ws_bytes(N, k_per_module, U, Q, {N, Q}, sm_count()));
   long long W, D;
   if (mode == EOGP_SCORE_FP && score_args_ok(N, k_per_module, U, &W, &D) && score_fp_supported(N, D, Q))
-    *bytes = score_fp_ws_bytes(N, D, Q, sm_count());
+    *bytes = score_fp_ws_bytes(N, D, Q, {N, Q}, sm_count());
   return EOGP_OK;
 }
 
-// Dense scoring into `scores`; the tensor-core kernels when the shape, the
-// pointers and the workspace allow, otherwise the CUDA-core kernels.
+// Dense scoring into `scores` of N rows and Q queries, a part or all of `all`; the
+// tensor-core kernels when the shape, the pointers and the workspace allow, otherwise
+// the CUDA-core kernels.
 static int score_dense(const void* train, int ld_train, const float* train_scales, int ld_tscale,
                        int N, const int* k_per_module, int U, int mode, const void* query,
-                       int ld_query, const float* query_scales, int ld_qscale, int Q,
+                       int ld_query, const float* query_scales, int ld_qscale, int Q, ScoreRequest all,
                        float* scores, int ld_scores, void* ws, size_t ws_bytes, long long W,
                        long long D, cudaStream_t st) {
   if (mode == EOGP_SCORE_CODES || mode == EOGP_SCORE_PAPER) {
@@ -1323,8 +1324,8 @@ static int score_dense(const void* train, int ld_train, const float* train_scale
       if (!status) return set_error(EOGP_ECUDA, "device status word unavailable");
       if (mode == EOGP_SCORE_PAPER && score_paper_supported(N, k_per_module, U, Q, train, ld_train))
         CUDA_TRY(launch_score_paper_tc(static_cast<const uint32_t*>(train), ld_train, train_scales, ld_tscale, N,
-                                       k_per_module, U, static_cast<const float*>(query), ld_query, Q, scores,
-                                       ld_scores, ws, ws_bytes, sm_count(), status, st));
+                                       k_per_module, U, static_cast<const float*>(query), ld_query, Q, all,
+                                       scores, ld_scores, ws, ws_bytes, sm_count(), status, st));
       else
         CUDA_TRY(launch_score_tc(mode, static_cast<const uint32_t*>(train), ld_train, train_scales,
                                  ld_tscale, N, k_per_module, U, query, ld_query, query_scales,
@@ -1341,13 +1342,13 @@ static int score_dense(const void* train, int ld_train, const float* train_scale
   } else if (mode == EOGP_SCORE_FP) {
     if (ld_train < D || ld_query < D) return set_error(EOGP_EINVAL, "leading dimension too small");
     // Tensor cores under the same conditions as above.
-    if (score_fp_supported(N, D, Q) && ws && ws_bytes >= score_fp_ws_bytes(N, D, Q, sm_count()) &&
+    if (score_fp_supported(N, D, Q) && ws && ws_bytes >= score_fp_ws_bytes(N, D, Q, all, sm_count()) &&
         (ld_train % 4) == 0 && aligned16(train) && (reinterpret_cast<uintptr_t>(ws) & 255) == 0) {
       unsigned* status = status_word();
       if (!status) return set_error(EOGP_ECUDA, "device status word unavailable");
       CUDA_TRY(launch_score_fp(static_cast<const float*>(train), ld_train, N, static_cast<int>(D),
-                               static_cast<const float*>(query), ld_query, Q, scores, ld_scores, ws, sm_count(),
-                               status, st));
+                               static_cast<const float*>(query), ld_query, Q, all, scores, ld_scores, ws,
+                               sm_count(), status, st));
       return EOGP_OK;
     }
     CUDA_TRY(launch_simt_gemm(Q, N, static_cast<int>(D), 1.f, static_cast<const float*>(query), ld_query,
@@ -1376,7 +1377,7 @@ extern "C" int eogp_score(const void* train, int ld_train, const float* train_sc
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   ProfScope ps(EOGP_K_SCORE, st);
   return score_dense(train, ld_train, train_scales, ld_tscale, N, k_per_module, U, mode, query,
-                     ld_query, query_scales, ld_qscale, Q, scores, ld_scores, ws, ws_bytes, W, D, st);
+                     ld_query, query_scales, ld_qscale, Q, {N, Q}, scores, ld_scores, ws, ws_bytes, W, D, st);
 }
 
 // ---------------------------------------------------------------- top-K
@@ -1439,15 +1440,10 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
     p.dense_bytes = al256(static_cast<size_t>(Q) * ((static_cast<size_t>(std::min(p.rows, N)) + 3) & ~size_t(3)) * 4);
     long long W, D;
     const int nr = std::min(p.rows, N);
-    // a last chunk of fewer rows may take more K ranges: room for either
-    if (mode == EOGP_SCORE_FP && score_args_ok(N, ks, U, &W, &D) && score_fp_supported(nr, D, Q)) {
-      p.q_bytes = score_fp_ws_bytes(nr, D, Q, sm_count());
-      if (N > nr && N % nr) p.q_bytes = std::max(p.q_bytes, score_fp_ws_bytes(N % nr, D, Q, sm_count()));
-    }
-    if (mode == EOGP_SCORE_PAPER && tc_ok && nr > 0) {
-      p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(nr, ks, U, Q, sm_count()));
-      if (N % nr) p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(N % nr, ks, U, Q, sm_count()));
-    }
+    if (mode == EOGP_SCORE_FP && score_args_ok(N, ks, U, &W, &D) && score_fp_supported(nr, D, Q))
+      p.q_bytes = score_fp_ws_bytes(nr, D, Q, {N, Q}, sm_count());
+    if (mode == EOGP_SCORE_PAPER && tc_ok && nr > 0)
+      p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(nr, ks, U, Q, {N, Q}, sm_count()));
     const long long slots = (static_cast<long long>(N) + p.slice - 1) / p.slice;
     p.n1 = slots > 1 ? slots * K : 0;
     p.n2 = p.n1 > kTopkListSlice ? (p.n1 + kTopkListSlice - 1) / kTopkListSlice * K : 0;
@@ -1539,7 +1535,7 @@ extern "C" int eogp_score_topk(const void* train, int ld_train, const float* tra
     if (nr > 0) {
       const int rc = score_dense(static_cast<const uint8_t*>(train) + static_cast<size_t>(r) * ld_train * esz, ld_train,
                                  train_scales ? train_scales + static_cast<size_t>(r) * ld_tscale : nullptr, ld_tscale,
-                                 nr, k_per_module, U, mode, query, ld_query, query_scales, ld_qscale, Q, dense, ldd,
+                                 nr, k_per_module, U, mode, query, ld_query, query_scales, ld_qscale, Q, {N, Q}, dense, ldd,
                                  qws, p.q_bytes, W, D, st);
       if (rc != EOGP_OK) return rc;
     }

@@ -130,12 +130,19 @@ cudaError_t launch_score_tc(int mode, const uint32_t* train, int ldt, const floa
                             int ldqs, int Q, float* out, int ldo, const TcTopK* topk, void* ws,
                             int num_sms, unsigned* status, cudaStream_t st);
 
+// Rows and queries of the whole request that a launch of the kernels below serves a
+// part of. It alone, not the part, says into how many ranges a sum over coordinates is
+// divided, so that equal stored rows have equal scores in every part.
+struct ScoreRequest {
+  int N, Q;
+};
+
 // k_score_fp.cu: unquantised scores on the tensor cores (rows of `train` 16-byte
 // aligned), with a workspace of score_fp_ws_bytes.
 bool score_fp_supported(int N, long long D, int Q);
-size_t score_fp_ws_bytes(int N, long long D, int Q, int num_sms);
+size_t score_fp_ws_bytes(int N, long long D, int Q, ScoreRequest all, int num_sms);
 cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const float* query, int ldq, int Q,
-                            float* out, int ldo, void* ws, int num_sms, unsigned* status, cudaStream_t st);
+                            ScoreRequest all, float* out, int ldo, void* ws, int num_sms, unsigned* status, cudaStream_t st);
 
 // out[q][i] = the S slabs' values [S][Q x ldp], added in order.
 cudaError_t launch_sum_slabs(const float* part, int S, size_t slab, int ldp, int N, int Q, float* out, int ldo,
@@ -145,9 +152,9 @@ cudaError_t launch_sum_slabs(const float* part, int S, size_t slab, int ldp, int
 // 16-byte aligned, modules multiples of 64 bits). With the 4 Q sum k bytes the
 // queries take alone as workspace, one K range per row tile.
 bool score_paper_supported(int N, const int* ks, int U, int Q, const void* train, int ldt);
-size_t score_paper_ws_bytes(int N, const int* ks, int U, int Q, int num_sms);
+size_t score_paper_ws_bytes(int N, const int* ks, int U, int Q, ScoreRequest all, int num_sms);
 cudaError_t launch_score_paper_tc(const uint32_t* train, int ldt, const float* ts, int ldts, int N, const int* ks,
-                                  int U, const float* y, int ldy, int Q, float* out, int ldo, void* ws,
+                                  int U, const float* y, int ldy, int Q, ScoreRequest all, float* out, int ldo, void* ws,
                                   size_t ws_bytes, int num_sms, unsigned* status, cudaStream_t st);
 
 // k_topk.cu: the K best (K <= EOGP_TOPK_MAX) of every slice of a row of scores

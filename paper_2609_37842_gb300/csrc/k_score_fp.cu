@@ -452,17 +452,22 @@ struct FpPlan {
   size_t parts, qbad, rbad, part, total;
 };
 
-// K ranges: the number that leaves the last wave of items fullest, counting 256
+int fp_tile_queries(int Q) {
+  const int n = (Q + 63) / 64;
+  return ((Q + n - 1) / n + 15) / 16 * 16;
+}
+
+// K ranges: the number that leaves the request's last wave of items fullest, counting 256
 // coordinates of a range's time for its start, drain and sum.
-FpPlan fp_plan(int N, int D, int Q, int num_sms) {
+FpPlan fp_plan(int N, int D, int Q, ScoreRequest all, int num_sms) {
   FpPlan p;
-  p.nqt = (Q + 63) / 64;
-  p.QB = ((Q + p.nqt - 1) / p.nqt + 15) / 16 * 16;
+  p.QB = fp_tile_queries(Q);
   p.nqt = (Q + p.QB - 1) / p.QB;
   p.nrt = (N + 127) / 128;
   p.Dp = (D + 63) / 64 * 64;
   p.nbox = p.Dp / 32;  // even: boxes past D are zero
-  const long long tiles = static_cast<long long>(p.nqt) * p.nrt;
+  const int qb = fp_tile_queries(all.Q);
+  const long long tiles = static_cast<long long>((all.Q + qb - 1) / qb) * ((all.N + 127) / 128);
   const int nyt = p.Dp / 64;
   long long best = -1;
   p.S = 1;
@@ -509,13 +514,14 @@ bool score_fp_supported(int N, long long D, int Q) {
          static_cast<long long>((N + 127) / 128) * ((Q + 63) / 64) * 32 < (1ll << 30);
 }
 
-size_t score_fp_ws_bytes(int N, long long D, int Q, int num_sms) {
-  return fp_plan(N, static_cast<int>(D), Q, num_sms).total;
+size_t score_fp_ws_bytes(int N, long long D, int Q, ScoreRequest all, int num_sms) {
+  return fp_plan(N, static_cast<int>(D), Q, all, num_sms).total;
 }
 
 cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const float* query, int ldq, int Q,
-                            float* out, int ldo, void* ws, int num_sms, unsigned* status, cudaStream_t st) {
-  const FpPlan p = fp_plan(N, D, Q, num_sms);
+                            ScoreRequest all, float* out, int ldo, void* ws, int num_sms, unsigned* status,
+                            cudaStream_t st) {
+  const FpPlan p = fp_plan(N, D, Q, all, num_sms);
   char* w = static_cast<char*>(ws);
   uint16_t* parts = reinterpret_cast<uint16_t*>(w + p.parts);
   int* qbad = reinterpret_cast<int*>(w + p.qbad);

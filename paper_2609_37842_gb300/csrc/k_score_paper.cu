@@ -359,17 +359,22 @@ struct PaperPlan {
   size_t query, total;  // workspace of the queries alone, and with the slabs
 };
 
-// K ranges (whole code boxes): the number that leaves the last wave of items
+int paper_tile_queries(int Q) {
+  const int n = (Q + kQB - 1) / kQB;
+  return ((Q + n - 1) / n + 15) / 16 * 16;
+}
+
+// K ranges (whole code boxes): the number that leaves the request's last wave of items
 // fullest, counting four pairs of a range's time for its start, drain and sum.
-PaperPlan paper_plan(int N, long long D, int Q, int num_sms) {
+PaperPlan paper_plan(int N, long long D, int Q, ScoreRequest all, int num_sms) {
   PaperPlan p;
-  p.nqt = (Q + kQB - 1) / kQB;
-  p.QB = ((Q + p.nqt - 1) / p.nqt + 15) / 16 * 16;
+  p.QB = paper_tile_queries(Q);
   p.nqt = (Q + p.QB - 1) / p.QB;
   p.nrt = (N + 127) / 128;
   p.npair = static_cast<int>(D / 64);
   const int nbox = (p.npair + 15) / 16;
-  const long long tiles = static_cast<long long>(p.nqt) * p.nrt;
+  const int qb = paper_tile_queries(all.Q);
+  const long long tiles = static_cast<long long>((all.Q + qb - 1) / qb) * ((all.N + 127) / 128);
   long long best = -1;
   p.S = 1;
   p.pps = 16 * nbox;
@@ -400,14 +405,14 @@ bool score_paper_supported(int N, const int* ks, int U, int Q, const void* train
   return true;
 }
 
-size_t score_paper_ws_bytes(int N, const int* ks, int U, int Q, int num_sms) {
+size_t score_paper_ws_bytes(int N, const int* ks, int U, int Q, ScoreRequest all, int num_sms) {
   long long D = 0;
   for (int u = 0; u < U; ++u) D += ks[u];
-  return paper_plan(N, D, Q, num_sms).total;
+  return paper_plan(N, D, Q, all, num_sms).total;
 }
 
 cudaError_t launch_score_paper_tc(const uint32_t* train, int ldt, const float* ts, int ldts, int N, const int* ks,
-                                  int U, const float* y, int ldy, int Q, float* out, int ldo, void* ws,
+                                  int U, const float* y, int ldy, int Q, ScoreRequest all, float* out, int ldo, void* ws,
                                   size_t ws_bytes, int num_sms, unsigned* status, cudaStream_t st) {
   PaperArgs g;  // ~4 KB parameter block, copied at launch
   int D = 0;
@@ -415,7 +420,7 @@ cudaError_t launch_score_paper_tc(const uint32_t* train, int ldt, const float* t
     D += ks[u];
     g.pend[u] = D / 64;
   }
-  PaperPlan p = paper_plan(N, D, Q, num_sms);
+  PaperPlan p = paper_plan(N, D, Q, all, num_sms);
   if (ws_bytes < p.total) {  // room for the queries alone: one K range
     p.S = 1;
     p.pps = (p.npair + 15) / 16 * 16;
