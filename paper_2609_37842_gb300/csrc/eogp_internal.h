@@ -205,12 +205,11 @@ cudaError_t launch_simt_gemm(int M, int N, int K, float alpha, const float* A, l
                              long long sak, const float* Bm, long long sbj, long long sbk,
                              float* C, long long ldc, cudaStream_t st, bool behind = false);
 // z[b*ldz + r] = scale[r] * sum_t St[(b*T+t)*ldS + posR[r]] * At[(b*T+t)*ldA + posC[r]]
-// The same GEMM (alpha = 1, k contiguous in A and B) for the tiles that hold a
-// noted row (one of n_inote notes, ld_inote apart) or a noted block of jblock
-// columns only.
+// The same GEMM (alpha = 1, k contiguous in A and B) for the entries of noted rows (one
+// of n_inote notes, ld_inote apart) and noted columns only.
 cudaError_t launch_simt_gemm_noted(int M, int N, int K, const float* A, long long lda, const float* Bm, long long ldb,
                                    float* C, long long ldc, const int* inote, int n_inote, int ld_inote,
-                                   const int* jnote, int jblock, cudaStream_t st);
+                                   const int* jnote, cudaStream_t st);
 // First stage of the fp32 path in one kernel (rotations, bias and lengths,
 // contraction and gather), for modules whose rotated rows of a few examples fit
 // shared memory.

@@ -16,8 +16,8 @@
 // 1.5e-7 (2.0e-7), all 512 1.0e-7 (2.5e-7), 49,152 1.2e-8 (3.0e-7). Sums near the end of
 // fp32's range are within a few units of 2^-149 a product.
 // Infinities, NaN and tiny values with bits below 2^-133, where bf16 ends, have no such
-// split: it leaves bits in the lower half of x3. A row tile or query that holds one
-// is noted, and k_simt_gemm computes its scores again afterwards.
+// split: it leaves bits in the lower half of x3. A row or query that holds one is
+// noted, and k_simt_gemm computes its scores, and no others, again afterwards.
 //
 // Bound: HBM (the stored coordinates, once per 64 queries), and from 48 queries on the
 // power limit. One CTA takes 128 stored rows (MMA M, operand A in TMEM) against QB <=
@@ -93,7 +93,7 @@ struct FpArgs {
   float* out;    // scores, or with S > 1 the slabs [S][Q][ldo]
   size_t slab;
   int ldo;
-  int* rbad;     // [nrt]: the row tile holds a value without a split
+  int* rbad;     // [N]: the row holds a value without a split
   unsigned* status;
 };
 
@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&afull[as]);
       }
-      if (__any_sync(0xffffffffu, (bad & 0xFFFFu) != 0) && lane == 0) g.rbad[item / (g.nqt * g.S)] = 1;
+      // (rows past N are zeros)
+      if (bad & 0xFFFFu) g.rbad[item / (g.nqt * g.S) * 128 + r] = 1;
     }
   } else if (warp == kMmaW) {
     // ---------------------------------------------------------- issuer
@@ -394,10 +395,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Query q's three bf16 parts, in rows part * QB + q % QB of query tile q / QB
 // (rows of Dp values, zero past D; the rows of a tile past Q are zero), and whether
 // the part of it that block (q, y) splits holds a value without a split. Clears the
-// row tiles' notes. Queries are on grid.x: whole tiles of 65,535 are 65,536 of them.
+// rows' notes. Queries are on grid.x: whole tiles of 65,535 are 65,536 of them.
 __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict__ y, int ldq, int Q, int D, int Dp,
                                                         int QB, uint16_t* __restrict__ parts, int* __restrict__ qbad,
-                                                        int* __restrict__ rbad, int nrt) {
+                                                        int* __restrict__ rbad, int N) {
   const int q = blockIdx.x, c0 = 2 * (blockIdx.y * blockDim.x + threadIdx.x), nthr = gridDim.y * blockDim.x;
   uint16_t* o = parts + (static_cast<size_t>(q / QB) * 3 * QB + q % QB) * Dp;
   const size_t step = static_cast<size_t>(QB) * Dp;
@@ -416,7 +417,7 @@ __global__ void __launch_bounds__(256) k_split3_queries(const float* __restrict_
   }
   bad = __syncthreads_or(bad);
   if (threadIdx.x == 0) qbad[static_cast<size_t>(blockIdx.y) * gridDim.x + q] = bad;
-  for (int i = (q * gridDim.y + blockIdx.y) * blockDim.x + threadIdx.x; i < nrt; i += gridDim.x * nthr) rbad[i] = 0;
+  for (int i = (q * gridDim.y + blockIdx.y) * blockDim.x + threadIdx.x; i < N; i += gridDim.x * nthr) rbad[i] = 0;
 }
 
 // scores[q][i] = the slabs' values in order; four scores a thread (ldp is a
@@ -486,7 +487,7 @@ FpPlan fp_plan(int N, int D, int Q, ScoreRequest all, int num_sms) {
   p.parts = 0;
   p.qbad = al(static_cast<size_t>(p.nqt) * 3 * p.QB * p.Dp * 2);
   p.rbad = p.qbad + al(static_cast<size_t>(kSplitBlocks) * p.nqt * p.QB * 4);
-  p.part = p.rbad + al(static_cast<size_t>(p.nrt) * 4);
+  p.part = p.rbad + al(static_cast<size_t>(N) * 4);
   p.total = p.part + (p.S > 1 ? al(static_cast<size_t>(p.S) * Q * p.ldp * 4) : 0);
   return p;
 }
@@ -528,7 +529,7 @@ cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const flo
   int* rbad = reinterpret_cast<int*>(w + p.rbad);
   float* part = reinterpret_cast<float*>(w + p.part);
   const int sb = std::min(kSplitBlocks, (p.Dp / 2 + 255) / 256);
-  k_split3_queries<<<dim3(p.nqt * p.QB, sb), 256, 0, st>>>(query, ldq, Q, D, p.Dp, p.QB, parts, qbad, rbad, p.nrt);
+  k_split3_queries<<<dim3(p.nqt * p.QB, sb), 256, 0, st>>>(query, ldq, Q, D, p.Dp, p.QB, parts, qbad, rbad, N);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   CUtensorMap tx, ty;
@@ -565,6 +566,5 @@ cudaError_t launch_score_fp(const float* train, int ldt, int N, int D, const flo
     if (e != cudaSuccess) return e;
   }
   // scores of rows and queries with a value without a split, one fp32 chain each
-  return launch_simt_gemm_noted(Q, N, D, query, ldq, train, ldt, out, ldo, qbad, sb, p.nqt * p.QB, rbad,
-                                128, st);
+  return launch_simt_gemm_noted(Q, N, D, query, ldq, train, ldt, out, ldo, qbad, sb, p.nqt * p.QB, rbad, st);
 }

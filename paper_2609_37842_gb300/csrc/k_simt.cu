@@ -170,23 +170,31 @@ __device__ __forceinline__ void tile_gemm(GemmTiles<BM, BN>& sm, const Operand& 
   }
 }
 
-// NOTED: only tiles holding a noted row (one of its n_inote notes inote[b ld_inote + i])
-// or a noted block of columns (jnote[j / jblock]) are computed; the others keep what C holds.
+// NOTED: only the entries of noted rows (one of the n_inote notes inote[b ld_inote + i])
+// and noted columns (jnote[j]) are written, and only tiles with one are computed.
 template <int BM, int BN, int TM, int TN, int PD, int L, bool NOTED>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
     k_simt_gemm(int M, int N, int K, float alpha, const Operand A, const Operand B, float* __restrict__ C,
-                long long ldc, const int* __restrict__ inote, int n_inote, int ld_inote, const int* __restrict__ jnote,
-                int jblock) {
+                long long ldc, const int* __restrict__ inote, int n_inote, int ld_inote, const int* __restrict__ jnote) {
   constexpr int NX = BN / TN, NY = BM / TM;
   __shared__ GemmTiles<BM, BN> sm;
+  __shared__ uint8_t noted[NOTED ? BM + BN : 1];  // the tile's rows, then its columns
   eogp::pdl_trigger();
   eogp::pdl_wait();
   const int i0 = blockIdx.y * BM, j0 = blockIdx.x * BN;
   if (NOTED) {
     int hit = 0;
-    for (int i = threadIdx.x; i < BM && i0 + i < M; i += NX * NY)
-      for (int b = 0; b < n_inote; ++b) hit |= inote[static_cast<size_t>(b) * ld_inote + i0 + i];
-    for (int j = threadIdx.x; j < BN && j0 + j < N; j += NX * NY) hit |= jnote[(j0 + j) / jblock];
+    for (int i = threadIdx.x; i < BM && i0 + i < M; i += NX * NY) {
+      int h = 0;
+      for (int b = 0; b < n_inote; ++b) h |= inote[static_cast<size_t>(b) * ld_inote + i0 + i];
+      noted[i] = h != 0;
+      hit |= h;
+    }
+    for (int j = threadIdx.x; j < BN && j0 + j < N; j += NX * NY) {
+      const int h = jnote[j0 + j];
+      noted[BM + j] = h != 0;
+      hit |= h;
+    }
     if (!__syncthreads_or(hit)) return;
   }
   float acc[TM][TN];
@@ -199,7 +207,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 #pragma unroll
     for (int y = 0; y < TN; ++y) {
       const int j = j0 + frag_pos<TN, NX>(tx, y);
-      if (j < N) C[i * ldc + j] = alpha * acc[x][y];
+      if (j < N && (!NOTED || noted[i - i0] || noted[BM + j - j0])) C[i * ldc + j] = alpha * acc[x][y];
     }
   }
 }
@@ -346,14 +354,14 @@ int layout_of(const Operand& a, const Operand& b, int K) {
 
 template <int BM, int BN, int TM, int TN, int PD, int L, bool NOTED>
 cudaError_t simt_launch(int M, int N, int K, float alpha, const Operand& A, const Operand& B, float* C, long long ldc,
-                        const int* inote, int n_inote, int ld_inote, const int* jnote, int jblock, cudaStream_t st,
+                        const int* inote, int n_inote, int ld_inote, const int* jnote, cudaStream_t st,
                         bool behind = false) {
   const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
   if (behind)
     return launch_behind(k_simt_gemm<BM, BN, TM, TN, PD, L, NOTED>, grid, (BM / TM) * (BN / TN), 0, st, M, N, K, alpha, A,
-                         B, C, ldc, inote, n_inote, ld_inote, jnote, jblock);
+                         B, C, ldc, inote, n_inote, ld_inote, jnote);
   k_simt_gemm<BM, BN, TM, TN, PD, L, NOTED><<<grid, (BM / TM) * (BN / TN), 0, st>>>(M, N, K, alpha, A, B, C, ldc, inote,
-                                                                               n_inote, ld_inote, jnote, jblock);
+                                                                               n_inote, ld_inote, jnote);
   return cudaGetLastError();
 }
 
@@ -363,10 +371,10 @@ template <int BM, int BN, int TM, int TN, int PD>
 static cudaError_t simt_layout(int l, int M, int N, int K, float alpha, const Operand& A, const Operand& B, float* C,
                                long long ldc, cudaStream_t st, bool behind) {
   if (l == kAlongK)
-    return simt_launch<BM, BN, TM, TN, PD, kAlongK, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st, behind);
+    return simt_launch<BM, BN, TM, TN, PD, kAlongK, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, st, behind);
   if (l == kAlongRows)
-    return simt_launch<BM, BN, TM, TN, PD, kAlongRows, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st, behind);
-  return simt_launch<BM, BN, TM, TN, 1, kAny, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, 1, st, behind);
+    return simt_launch<BM, BN, TM, TN, PD, kAlongRows, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, st, behind);
+  return simt_launch<BM, BN, TM, TN, 1, kAny, false>(M, N, K, alpha, A, B, C, ldc, nullptr, 0, 0, nullptr, st, behind);
 }
 
 // The largest tile that still gives the SMs blocks enough; small ones shorten the
@@ -391,10 +399,10 @@ cudaError_t launch_simt_gemm(int M, int N, int K, float alpha, const float* A, l
 
 cudaError_t launch_simt_gemm_noted(int M, int N, int K, const float* A, long long lda, const float* Bm, long long ldb,
                                    float* C, long long ldc, const int* inote, int n_inote, int ld_inote,
-                                   const int* jnote, int jblock, cudaStream_t st) {
+                                   const int* jnote, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   return simt_launch<64, 64, 8, 4, 1, kAny, true>(M, N, K, 1.f, Operand{A, lda, 1, M}, Operand{Bm, ldb, 1, N}, C, ldc,
-                                                  inote, n_inote, ld_inote, jnote, jblock, st);
+                                                  inote, n_inote, ld_inote, jnote, st);
 }
 
 // Rows per block of k_f32_first (64, or 16 where that gives too few blocks), 0 when
