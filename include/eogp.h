@@ -541,8 +541,9 @@ int eogp_score_topk_workspace_size(int N, const int* k_per_module, int U, int mo
                                    int topk, size_t* bytes);
 
 /* Per query, the `topk` best stored rows under the eogp_score definition of
- * `mode`. The scores of as many stored rows as fit 1 GiB of workspace are formed
- * and ranked at a time; with EOGP_OPT_TOPK_PATH = 1 (or 0 and millions of rows),
+ * `mode`. At most 1 GiB of scores are formed and ranked at a time (some of the stored
+ * rows, and of more than 16,384 queries some of those); the workspace holds them, the
+ * lists of the rows ranked so far and eogp_score's own. With EOGP_OPT_TOPK_PATH = 1 (or 0 and millions of rows),
  * where the tensor-core kernels apply and topk <= 32, the ranking runs in their
  * epilogue instead, with no scores written and a workspace of tens of MB. Arguments as eogp_score, plus:
  *   top_scores [Q x ld_top_scores] fp32 device and top_index [Q x ld_top_index]

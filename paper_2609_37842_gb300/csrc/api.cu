@@ -1388,13 +1388,15 @@ struct TopkPlan {
   bool tc_rows;  // refused unless the code rows are aligned for the tensor cores
   int slots;     // fused: per-CTA lists
   int slice, rows;       // dense: stored rows ranked per block, and scored at a time (a multiple of slice)
+  int queries;           // dense: queries scored and ranked at a time
   long long n1, n2;      // dense: list entries per query of the first level, and of the second (0: none)
   size_t q_bytes, dense_bytes, list_bytes, buf_bytes, scr_bytes, total;
 };
 
 // Paths. Dense: scores (tensor cores where they apply) of as many stored rows as
 // 1 GiB of workspace holds, ranked slice by slice by k_topk_select, and so on
-// over the rows; then the slices' lists are ranked. Fused: the ranking in the
+// over the rows; then the slices' lists are ranked. Queries of which 1 GiB does not
+// hold a slice (more than 16,384) are ranked some after others. Fused: the ranking in the
 // tensor-core kernel's epilogue, no scores in memory; there it holds up the MMAs
 // while the lists fill. Measured, top 20, fused / dense in us: 64 queries over
 // 300K rows of 16,384 bits 657 / 258, 1024 queries 3,756 / 1,853, 1024 over
@@ -1435,20 +1437,26 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
     p.scr_bytes = al256(score_tc_scratch_bytes(mode, ks, U, Q, K, p.slots));
   } else {
     p.slice = topk_slice(N, Q);
-    const long long fit = static_cast<long long>(kTopkDenseMax / (4 * static_cast<size_t>(std::max(Q, 1))));
-    p.rows = N <= fit ? std::max(N, 1) : static_cast<int>(std::max<long long>(1, fit / p.slice) * p.slice);
-    p.dense_bytes = al256(static_cast<size_t>(Q) * ((static_cast<size_t>(std::min(p.rows, N)) + 3) & ~size_t(3)) * 4);
+    const size_t row_bytes = 4 * static_cast<size_t>(std::max(4, std::min((N + 3) & ~3, p.slice)));
+    const int most = static_cast<int>(std::min<size_t>(kTopkDenseMax / row_bytes, 1 << 30)) & ~63;
+    const int parts = (Q - 1) / most + 1;
+    p.queries = parts > 1 ? ((Q - 1) / parts / 64 + 1) * 64 : Q;  // even parts of whole query tiles
+    const long long fit = static_cast<long long>(kTopkDenseMax / (4 * static_cast<size_t>(p.queries)));
+    p.rows = N <= fit ? std::max(N, 1) : static_cast<int>(fit / p.slice * p.slice);
+    p.dense_bytes =
+        al256(static_cast<size_t>(p.queries) * ((static_cast<size_t>(std::min(p.rows, N)) + 3) & ~size_t(3)) * 4);
+    if (tc_ok) p.q_bytes = score_tc_ws_bytes(mode, ks, U, p.queries);
     long long W, D;
     const int nr = std::min(p.rows, N);
     if (mode == EOGP_SCORE_FP && score_args_ok(N, ks, U, &W, &D) && score_fp_supported(nr, D, Q))
-      p.q_bytes = score_fp_ws_bytes(nr, D, Q, {N, Q}, sm_count());
+      p.q_bytes = score_fp_ws_bytes(nr, D, p.queries, {N, Q}, sm_count());
     if (mode == EOGP_SCORE_PAPER && tc_ok && nr > 0)
-      p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(nr, ks, U, Q, {N, Q}, sm_count()));
+      p.q_bytes = std::max(p.q_bytes, score_paper_ws_bytes(nr, ks, U, p.queries, {N, Q}, sm_count()));
     const long long slots = (static_cast<long long>(N) + p.slice - 1) / p.slice;
     p.n1 = slots > 1 ? slots * K : 0;
     p.n2 = p.n1 > kTopkListSlice ? (p.n1 + kTopkListSlice - 1) / kTopkListSlice * K : 0;
-    p.list_bytes = al256(static_cast<size_t>(Q) * ((p.n1 + 3) & ~3ll) * 4) +
-                   al256(static_cast<size_t>(Q) * ((p.n2 + 3) & ~3ll) * 4);
+    p.list_bytes = al256(static_cast<size_t>(p.queries) * ((p.n1 + 3) & ~3ll) * 4) +
+                   al256(static_cast<size_t>(p.queries) * ((p.n2 + 3) & ~3ll) * 4);
   }
   p.total = al256(p.q_bytes) + p.dense_bytes + 2 * p.list_bytes + 2 * p.buf_bytes +
             (p.fused ? al256(static_cast<size_t>(Q) * 4) : 0) + p.scr_bytes;
@@ -1521,43 +1529,50 @@ extern "C" int eogp_score_topk(const void* train, int ld_train, const float* tra
                              0, &tk, qws, sm_count(), status, st));
     return EOGP_OK;
   }
-  // Dense: chunks of p.rows stored rows scored and ranked slice by slice.
+  // Dense: p.queries queries and p.rows stored rows at a time, scored and ranked slice by slice.
   const int ldd = (std::min(p.rows, N) + 3) & ~3;
   const size_t ld1 = static_cast<size_t>((p.n1 + 3) & ~3ll), ld2 = static_cast<size_t>((p.n2 + 3) & ~3ll);
-  const size_t l1 = al256(static_cast<size_t>(Q) * ld1 * 4);  // bytes of a first-level list array
-  float* s1 = lst;
-  int* i1 = lsi;
-  float* s2 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(lst) + l1);
-  int* i2 = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(lsi) + l1);
+  const size_t l1 = al256(static_cast<size_t>(p.queries) * ld1 * 4);  // bytes of a first-level list array
   const size_t esz = 4;  // code words and fp32 coordinates alike
-  for (long long r0 = 0; r0 < std::max(N, 1); r0 += p.rows) {
-    const int r = static_cast<int>(r0), nr = std::min(p.rows, N - r);
-    if (nr > 0) {
-      const int rc = score_dense(static_cast<const uint8_t*>(train) + static_cast<size_t>(r) * ld_train * esz, ld_train,
-                                 train_scales ? train_scales + static_cast<size_t>(r) * ld_tscale : nullptr, ld_tscale,
-                                 nr, k_per_module, U, mode, query, ld_query, query_scales, ld_qscale, Q, {N, Q}, dense, ldd,
-                                 qws, p.q_bytes, W, D, st);
-      if (rc != EOGP_OK) return rc;
+  for (long long q0 = 0; q0 < Q; q0 += p.queries) {
+    const int nq = static_cast<int>(std::min<long long>(p.queries, Q - q0));
+    const uint8_t* yq = static_cast<const uint8_t*>(query) + static_cast<size_t>(q0) * ld_query * esz;
+    const float* yqs = query_scales ? query_scales + static_cast<size_t>(q0) * ld_qscale : nullptr;
+    float* ts = top_scores + static_cast<size_t>(q0) * ld_top_scores;
+    int* ti = top_index + static_cast<size_t>(q0) * ld_top_index;
+    float* s1 = lst;
+    int* i1 = lsi;
+    float* s2 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(lst) + l1);
+    int* i2 = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(lsi) + l1);
+    for (long long r0 = 0; r0 < std::max(N, 1); r0 += p.rows) {
+      const int r = static_cast<int>(r0), nr = std::min(p.rows, N - r);
+      if (nr > 0) {
+        const int rc = score_dense(static_cast<const uint8_t*>(train) + static_cast<size_t>(r) * ld_train * esz,
+                                   ld_train, train_scales ? train_scales + static_cast<size_t>(r) * ld_tscale : nullptr,
+                                   ld_tscale, nr, k_per_module, U, mode, yq, ld_query, yqs, ld_qscale, nq, {N, Q},
+                                   dense, ldd, qws, p.q_bytes, W, D, st);
+        if (rc != EOGP_OK) return rc;
+      }
+      const size_t at = static_cast<size_t>(r / p.slice) * topk;  // the chunk's first list entry
+      if (p.n1 == 0)
+        CUDA_TRY(launch_topk_select(dense, nullptr, ldd, nq, nr, r, topk, p.slice, false, ts, ld_top_scores, ti,
+                                    ld_top_index, st));
+      else
+        CUDA_TRY(launch_topk_select(dense, nullptr, ldd, nq, nr, r, topk, p.slice, true, s1 + at, ld1, i1 + at, ld1, st));
     }
-    const size_t at = static_cast<size_t>(r / p.slice) * topk;  // the chunk's first list entry
-    if (p.n1 == 0)
-      CUDA_TRY(launch_topk_select(dense, nullptr, ldd, Q, nr, r, topk, p.slice, false, top_scores, ld_top_scores,
-                                  top_index, ld_top_index, st));
-    else
-      CUDA_TRY(launch_topk_select(dense, nullptr, ldd, Q, nr, r, topk, p.slice, true, s1 + at, ld1, i1 + at, ld1, st));
+    // The lists, as rows of scores, until one slice holds what is left of a query.
+    long long n = p.n1;
+    size_t ld = ld1, ldo = ld2;
+    while (n > kTopkListSlice) {
+      CUDA_TRY(launch_topk_select(s1, i1, ld, nq, static_cast<int>(n), 0, topk, kTopkListSlice, true, s2, ldo, i2, ldo, st));
+      n = (n + kTopkListSlice - 1) / kTopkListSlice * topk;
+      std::swap(s1, s2);
+      std::swap(i1, i2);
+      std::swap(ld, ldo);
+    }
+    if (n > 0)
+      CUDA_TRY(launch_topk_select(s1, i1, ld, nq, static_cast<int>(n), 0, topk, kTopkListSlice, false, ts, ld_top_scores,
+                                  ti, ld_top_index, st));
   }
-  // The lists, as rows of scores, until one slice holds what is left of a query.
-  long long n = p.n1;
-  size_t ld = ld1, ldo = ld2;
-  while (n > kTopkListSlice) {
-    CUDA_TRY(launch_topk_select(s1, i1, ld, Q, static_cast<int>(n), 0, topk, kTopkListSlice, true, s2, ldo, i2, ldo, st));
-    n = (n + kTopkListSlice - 1) / kTopkListSlice * topk;
-    std::swap(s1, s2);
-    std::swap(i1, i2);
-    std::swap(ld, ldo);
-  }
-  if (n > 0)
-    CUDA_TRY(launch_topk_select(s1, i1, ld, Q, static_cast<int>(n), 0, topk, kTopkListSlice, false, top_scores,
-                                ld_top_scores, top_index, ld_top_index, st));
   return EOGP_OK;
 }
