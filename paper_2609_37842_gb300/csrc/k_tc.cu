@@ -27,6 +27,7 @@
 
 #include "eogp_dev.cuh"
 #include "eogp_internal.h"
+#include "rotate_order.h"
 
 using namespace eogp;
 
@@ -1470,47 +1471,16 @@ bool rotate_in_one(const RotSide& ra, const RotSide& rs, int M, int num_sms) {
   return rot_tiles(ra, M, rotate_bn(ra.rows, 16)) + rot_tiles(rs, M, rotate_bn(rs.rows, 16)) <= 2ll * num_sms;
 }
 
-// The tile width is the one whose last CTA ends first. A K block of a BN-column tile
-// costs 2 BN cycles of the tensor pipe, at least ~220 in all. Five queries of 512
-// tokens through 768 -> 2304 take 11.6 us in one launch, 13.0 + 10.6 in two.
+// Five queries of 512 tokens through 768 -> 2304 take 11.6 us in one launch, 13.0 +
+// 10.6 in two.
 cudaError_t launch_tc_rotate_both(const RotSide& ra, const RotSide& rs, int M, int T, int num_sms, unsigned* status,
                                   cudaStream_t st) {
   if (M <= 0) return cudaSuccess;
   const bool swap = rs.K > ra.K;  // the longer reduction first
   const RotSide r[2] = {swap ? rs : ra, swap ? ra : rs};
-  const int sms = std::max(1, num_sms);
-  int best[2] = {0, 0};
-  long long best_t = -1;
-  const int n = std::max(r[0].rows, r[1].rows);
-  for (int nN = (n + 255) / 256; best_t < 0 || nN <= (n + 63) / 64; ++nN) {  // tiles of the wider side
-    const int bn = ((n + nN - 1) / nN + 15) / 16 * 16;
-    int b[2];
-    long long cost[2], cnt[2];
-    for (int i = 0; i < 2; ++i) {
-      const int parts = (r[i].rows + bn - 1) / bn;
-      b[i] = std::max(16, ((r[i].rows + parts - 1) / parts + 15) / 16 * 16);
-      cnt[i] = rot_tiles(r[i], M, b[i]);
-      cost[i] = static_cast<long long>((r[i].K + 63) / 64) * std::max(2 * b[i], 220);
-    }
-    // the CTA that ends last under the back-and-forth order
-    const long long all = cnt[0] + cnt[1];
-    long long last = 0;
-    for (int c = 0; c < sms; ++c) {
-      long long sum = 0;
-      for (long long rd = 0; rd * sms < all; ++rd) {
-        const long long t = rd * sms + (rd & 1 ? sms - 1 - c : c);
-        if (t < all) sum += cost[t >= cnt[0] ? 1 : 0];
-      }
-      last = std::max(last, sum);
-    }
-    last += 12 * bn;
-    if (best_t < 0 || last < best_t) {
-      best_t = last;
-      best[0] = b[0];
-      best[1] = b[1];
-    }
-  }
-  return launch_rot(r, 2, M, T, best, num_sms, status, st);
+  int bn[2];
+  rotate_both_widths({r[0].rows, r[1].rows}, {r[0].K, r[1].K}, M, std::max(1, num_sms), bn);
+  return launch_rot(r, 2, M, T, bn, num_sms, status, st);
 }
 
 int tc_gemm_splits_used(int K, int splits) {
