@@ -676,10 +676,10 @@ extern "C" int eogp_compress_layer(const eogp_layer_desc* L, const void* a, cons
   const bool behind = static_cast<long long>(B) * L->T <= 64ll * sm_count();
   float* z = out_mode == EOGP_OUT_FIRST_STAGE ? out : reinterpret_cast<float*>(w + lo.z);
   const int ldz = out_mode == EOGP_OUT_FIRST_STAGE ? ld_out : L->m;
-  if (f32_first_supported(B, L->T, nC, nR)) {
+  if (f32_first_supported(B, L->T, nC, nR, sm_count())) {
     CUDA_TRY(launch_f32_first(af, sf, static_cast<const float*>(VA), static_cast<const float*>(VS), L->d_in, L->d_out,
                               L->bias_A, L->lengths, B, L->T, L->m, nC, nR, P->d_posR, P->d_posC, P->d_scale, z, ldz,
-                              st));
+                              sm_count(), st));
   } else {
     CUDA_TRY(launch_simt_gemm(M, nC, L->d_in, 1.f, af, L->d_in, 1, static_cast<const float*>(VA),
                               L->d_in, 1, at, nC, st));
@@ -1436,7 +1436,7 @@ static TopkPlan topk_plan(int N, const int* ks, int U, int mode, int Q, int K) {
     p.buf_bytes = al256(score_tc_list_buf_bytes(mode, ks, U, Q, K, p.slots));
     p.scr_bytes = al256(score_tc_scratch_bytes(mode, ks, U, Q, K, p.slots));
   } else {
-    p.slice = topk_slice(N, Q);
+    p.slice = topk_slice(N, Q, sm_count());
     const size_t row_bytes = 4 * static_cast<size_t>(std::max(4, std::min((N + 3) & ~3, p.slice)));
     const int most = static_cast<int>(std::min<size_t>(kTopkDenseMax / row_bytes, 1 << 30)) & ~63;
     const int parts = (Q - 1) / most + 1;

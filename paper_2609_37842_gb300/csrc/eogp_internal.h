@@ -161,7 +161,7 @@ cudaError_t launch_score_paper_tc(const uint32_t* train, int ldt, const float* t
 // [Q x ld] (ld a multiple of 4, 16-byte aligned): slice s of row q to K places at
 // K s + ld_o q. `map`: the values' stored rows (lists of an earlier level), else
 // place + row0; `mid`: the lists go on to a further level.
-int topk_slice(int N, int Q);
+int topk_slice(int N, int Q, int num_sms);
 cudaError_t launch_topk_select(const float* scores, const int* map, size_t ld, int Q, int N, int row0, int K, int slice,
                                bool mid, float* out_s, size_t ld_os, int* out_i, size_t ld_oi, cudaStream_t st);
 // Merge of per-slot lists [S][Q][K] (index -1 = empty) into [Q, K].
@@ -213,11 +213,11 @@ cudaError_t launch_simt_gemm_noted(int M, int N, int K, const float* A, long lon
 // First stage of the fp32 path in one kernel (rotations, bias and lengths,
 // contraction and gather), for modules whose rotated rows of a few examples fit
 // shared memory.
-bool f32_first_supported(int B, int T, int nC, int nR);
+bool f32_first_supported(int B, int T, int nC, int nR, int num_sms);
 cudaError_t launch_f32_first(const float* a, const float* s, const float* VA, const float* VS, int d_in, int d_out,
                              const float* bias, const int32_t* lengths, int B, int T, int m, int nC, int nR,
                              const int32_t* posR, const int32_t* posC, const float* scale, float* z, int ldz,
-                             cudaStream_t st);
+                             int num_sms, cudaStream_t st);
 cudaError_t launch_contract_f32(const float* At, int ldA, const float* St, int ldS, int B, int T,
                                 int m, const int32_t* posR, const int32_t* posC,
                                 const float* scale, float* z, int ldz, cudaStream_t st);

@@ -412,8 +412,8 @@ static size_t f32_first_smem(int bm, int nC, int nR) {
   return (bm == 64 ? sizeof(GemmTiles<64, 64>) : sizeof(GemmTiles<16, 64>)) +
          static_cast<size_t>(nC + nR) * (bm + 4) * 4;
 }
-static int f32_first_rows(int B, int T, int nC, int nR) {
-  if (T <= 16 && static_cast<long long>(B) * T <= 2 * 152 * 32 && f32_first_smem(16, nC, nR) <= 200 * 1024) return 16;
+static int f32_first_rows(int B, int T, int nC, int nR, int num_sms) {
+  if (T <= 16 && static_cast<long long>(B) * T <= 64ll * num_sms && f32_first_smem(16, nC, nR) <= 200 * 1024) return 16;
   return T <= 64 && f32_first_smem(64, nC, nR) <= 200 * 1024 ? 64 : 0;
 }
 
@@ -426,13 +426,13 @@ static cudaError_t first_launch(const FirstArgs& g, size_t smem, cudaStream_t st
   return cudaGetLastError();
 }
 
-bool f32_first_supported(int B, int T, int nC, int nR) { return f32_first_rows(B, T, nC, nR) > 0; }
+bool f32_first_supported(int B, int T, int nC, int nR, int num_sms) { return f32_first_rows(B, T, nC, nR, num_sms) > 0; }
 
 cudaError_t launch_f32_first(const float* a, const float* s, const float* VA, const float* VS, int d_in, int d_out,
                              const float* bias, const int32_t* lengths, int B, int T, int m, int nC, int nR,
                              const int32_t* posR, const int32_t* posC, const float* scale, float* z, int ldz,
-                             cudaStream_t st) {
-  const int bm = f32_first_rows(B, T, nC, nR);
+                             int num_sms, cudaStream_t st) {
+  const int bm = f32_first_rows(B, T, nC, nR, num_sms);
   if (!bm) return cudaErrorInvalidValue;
   FirstArgs g;
   g.B = B;

@@ -261,10 +261,10 @@ __global__ void __launch_bounds__(256) k_topk_merge(const float* __restrict__ ls
 // One block ranks up to 16,384 stored rows of a query by itself; more rows take
 // the fewest slices of that size, or for few queries enough of at least 4096 rows
 // to give every SM two blocks.
-int topk_slice(int N, int Q) {
+int topk_slice(int N, int Q, int num_sms) {
   if (N <= kSelSlice) return kSelSlice;
   const int least = (N + kSelSlice - 1) / kSelSlice;
-  const int S = std::max(least, std::min((N + 4095) / 4096, (2 * 152 + Q - 1) / std::max(Q, 1)));
+  const int S = std::max(least, std::min((N + 4095) / 4096, (2 * num_sms + Q - 1) / std::max(Q, 1)));
   return ((N + S - 1) / S + 3) & ~3;
 }
 
