@@ -312,6 +312,17 @@ __device__ __forceinline__ void tc_mma_f4_ta_pair(uint32_t d_tmem, uint32_t a_tm
       : "memory");
 }
 
+// kind::f16 with operand A in TMEM.
+__device__ __forceinline__ void tc_mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 // Same MMA with operand A in tensor memory: a_tmem addresses the first of the
 // K / 4 32-bit columns holding A (TMEM lane = row of A, four e4m3 elements per
 // column, element 4c + e in byte e of column c).

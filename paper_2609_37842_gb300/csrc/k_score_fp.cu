@@ -97,19 +97,6 @@ struct FpArgs {
   unsigned* status;
 };
 
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, unsigned* status) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status));
-}
-
-__device__ __forceinline__ void mma_f16_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d),
-      "r"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
 // Three-way split: upper halves of x, x - x1 and x - x1 - x2. Exact if and only if the
 // lower half of h3 is zero (an infinity or a NaN makes h3 the canonical NaN 0x7FFFFFFF).
 __device__ __forceinline__ void split3(float x, uint32_t& h1, uint32_t& h2, uint32_t& h3) {
@@ -192,7 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; c < QB; ++c) sum[c] = 0.f;
       for (int b = b0; b < b1; b += kDrainBoxes, ++run) {
         const int buf = static_cast<int>(run % ND);
-        if (!warp_wait(&dfull[buf], (run / ND) & 1u, g.status)) {
+        if (!mbar_wait_warp(&dfull[buf], (run / ND) & 1u, g.status)) {
           ok = false;
           break;
         }
@@ -248,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if ((it & 1u) != static_cast<uint32_t>(grp)) continue;
         const uint32_t pr = it >> 1;  // pair of boxes = A slot use
         const int xs = static_cast<int>(it % kXRing), as = static_cast<int>(pr % kSlots);
-        if (!warp_wait(&xfull[xs], (it / kXRing) & 1u, g.status)) {
+        if (!mbar_wait_warp(&xfull[xs], (it / kXRing) & 1u, g.status)) {
           ok = false;
           break;
         }
@@ -275,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&xempty[xs]);  // the box is in registers
-        if (!warp_wait(&aempty[as], ((pr / kSlots) & 1u) ^ 1u, g.status)) {
+        if (!mbar_wait_warp(&aempty[as], ((pr / kSlots) & 1u) ^ 1u, g.status)) {
           ok = false;
           break;
         }
@@ -330,20 +317,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t a = a0 + 48u * (kk >> 1) + 8u * (kk & 1);
                 const bool start = kk == 0 && bb == b;  // of a run
                 if constexpr (fp_parts<QB>() == 3) {
-                  mma_f16_ta(d, a, y, id3, start ? 0u : 1u);
-                  mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
-                  mma_f16_ta(d + 2 * QB, a + 32u, y, id1, 1u);
-                  mma_f16_ta(d + 2 * QB, a + 16u, y + 2 * kPart, id1, 1u);
-                  mma_f16_ta(d + 2 * QB, a + 32u, y + kPart, id1, 1u);
+                  tc_mma_f16_ta(d, a, y, id3, start ? 0u : 1u);
+                  tc_mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
+                  tc_mma_f16_ta(d + 2 * QB, a + 32u, y, id1, 1u);
+                  tc_mma_f16_ta(d + 2 * QB, a + 16u, y + 2 * kPart, id1, 1u);
+                  tc_mma_f16_ta(d + 2 * QB, a + 32u, y + kPart, id1, 1u);
                 } else {
-                  mma_f16_ta(d, a, y, id3, start ? 0u : 1u);
+                  tc_mma_f16_ta(d, a, y, id3, start ? 0u : 1u);
                   if (start) {  // d1 and d2 hold x1's products already, d3 starts here
-                    mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
-                    mma_f16_ta(d + 3 * QB, a + 16u, y + 2 * kPart, id1, 0u);
+                    tc_mma_f16_ta(d + QB, a + 16u, y, id2, 1u);
+                    tc_mma_f16_ta(d + 3 * QB, a + 16u, y + 2 * kPart, id1, 0u);
                   } else {
-                    mma_f16_ta(d + QB, a + 16u, y, id3, 1u);
+                    tc_mma_f16_ta(d + QB, a + 16u, y, id3, 1u);
                   }
-                  mma_f16_ta(d + 2 * QB, a + 32u, y, id2, 1u);
+                  tc_mma_f16_ta(d + 2 * QB, a + 32u, y, id2, 1u);
                 }
               }
               tc_commit(&aempty[as]);

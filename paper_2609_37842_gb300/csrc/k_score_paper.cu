@@ -63,19 +63,6 @@ struct PaperArgs {
   int pend[kMaxMods];  // first pair after module u
 };
 
-__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, unsigned* status) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status));
-}
-
-__device__ __forceinline__ void mma_f16_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d),
-      "r"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
 // The accumulation runs of pairs [p0, p1): cut at module ends and every kRunPairs.
 struct Runs {
   int p, end, u;  // next pair, item's end, module of p
@@ -159,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; c < kQB / 2; ++c) acc[c] = 0.f;
       for (Runs r(g, p0, p1); r.next(g, b, e, u); ++run) {
         const float si = row < g.N ? g.ts[static_cast<size_t>(row) * g.ldts + u] : 0.f;
-        if (!warp_wait(dfull, run & 1u, g.status)) {
+        if (!mbar_wait_warp(dfull, run & 1u, g.status)) {
           ok = false;
           break;
         }
@@ -203,7 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (Runs rs(g, p0, p1); ok && rs.next(g, b, e, u);) {
         for (int p = b; p < e; p += 2, ++rd) {
           const int as = static_cast<int>(rd % kSlots);
-          if (!warp_wait(&aempty[as], ((rd / kSlots) & 1u) ^ 1u, g.status)) {
+          if (!mbar_wait_warp(&aempty[as], ((rd / kSlots) & 1u) ^ 1u, g.status)) {
             ok = false;
             break;
           }
@@ -217,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&cempty[(bx + held) % kCRing]);
               }
-              if (!warp_wait(&cfull[cs], ((bx + pb) / kCRing) & 1u, g.status)) {
+              if (!mbar_wait_warp(&cfull[cs], ((bx + pb) / kCRing) & 1u, g.status)) {
                 ok = false;
                 break;
               }
@@ -280,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               if (elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
-                  mma_f16_ta(tmem, a + 8u * kk, y + 2 * kk, idesc, (p != b || i != 0 || kk != 0) ? 1u : 0u);
+                  tc_mma_f16_ta(tmem, a + 8u * kk, y + 2 * kk, idesc, (p != b || i != 0 || kk != 0) ? 1u : 0u);
                 tc_commit(&yempty[ys]);
               }
             }
