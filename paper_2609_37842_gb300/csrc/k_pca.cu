@@ -411,20 +411,28 @@ __global__ void __launch_bounds__(256) k_offnorm(const double* __restrict__ A, i
   }
 }
 
-// mu[i] = A[i][i]; sel[rank(i)] = i for the k largest (descending, ties to lower index,
-// NaN below every number: the ranks are a permutation whatever A holds).
+// Order of a double as an integer: larger value, larger key; -0 and +0 equal, NaN below
+// every number.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v), mag = b & 0x7FFFFFFFFFFFFFFFll;
+  if (mag > 0x7FF0000000000000ll) return -0x7FFFFFFFFFFFFFFFll - 1;
+  return mag == 0 ? 0 : b < 0 ? b ^ 0x7FFFFFFFFFFFFFFFll : b;
+}
+
+// mu[i] = A[i][i]; sel[rank(i)] = i for the k largest (descending, ties to lower index:
+// the ranks are a permutation whatever A holds). Integer keys: comparisons of doubles
+// share the few 64-bit lanes of an SM.
 __global__ void k_rank(const double* __restrict__ A, int n, int k, double* __restrict__ mu,
                        int* __restrict__ sel) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double vi = A[static_cast<size_t>(i) * n + i];
   mu[i] = vi;
+  const long long ki = order_key(vi);
   int rank = 0;
   for (int j = 0; j < n; ++j) {
-    const double vj = A[static_cast<size_t>(j) * n + j];
-    const bool above = vj > vi || (vi != vi && vj == vj);
-    const bool tie = vj == vi || (vi != vi && vj != vj);
-    rank += above || (tie && j < i);
+    const long long kj = order_key(A[static_cast<size_t>(j) * n + j]);
+    rank += kj > ki || (kj == ki && j < i);
   }
   if (rank < k) sel[rank] = i;
 }
