@@ -1404,7 +1404,12 @@ struct TopkPlan {
 // through memory); 256 over 4.2M 7,352 / 6,127; 1024 over 4M rows of 4,096 bits 14,606
 // / 13,148; 64 over 20,000 rows of 48 x 1024 bits 378 / 148. So the default is dense
 // but for kTopkFused*; EOGP_OPT_TOPK_PATH = 1 selects the fused path wherever it
-// applies.
+// applies. Beyond that line, in ms: 16,384 bits, 900 queries over 3M rows 17.07 /
+// 17.20, over 4.2M 22.95 / 24.00, 512 over 4.2M 12.53 / 12.44, 2,048 over 4.2M 43.8 /
+// 49.8 (inside it); 12,288 bits, 1024 over 4.2M 19.8 / 21.3; 8,192 bits, 1024 over 3M
+// 13.5 / 12.6, over 4.2M 17.4 / 17.5, over 8M 29.7 / 33.3. The dense path's own
+// outlay is the scores' way through memory, so fused wins where rows and queries are
+// many; the line keeps to the side where the gain is a few percent either way.
 constexpr int kTopkFusedMinN = 2500000, kTopkFusedMinQ = 1024, kTopkFusedMinBits = 16384;  // of one module
 constexpr size_t kTopkDenseMax = size_t(1) << 30;
 // Stored rows up to which any row alignment is ranked; more of them in a request

@@ -5,8 +5,10 @@
 // large translations: on the GB300 systems this library was measured on,
 // cudaHostAlloc'd buffers fed cudaMemcpyAsync at anywhere from ~80 to ~210 GB/s
 // from one allocation to the next, anonymous memory advised for huge pages and
-// then registered with cudaHostRegister ran at ~211 GB/s every time, and the
-// same memory on 64 KB base pages (no huge-page advice) at ~51 GB/s.
+// then registered with cudaHostRegister ran at ~211 GB/s, and the same memory on
+// 64 KB base pages (no huge-page advice) at ~51 GB/s. The advice is a request: a
+// host with no huge page to give backs the region with base pages, and nothing here
+// finds that out (one run's copies ran at 58 GB/s).
 //
 // Three size classes:
 //  * at least half a huge page: a region of its own, aligned to and advised for

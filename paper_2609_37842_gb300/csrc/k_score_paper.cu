@@ -7,7 +7,7 @@
 // <= 256 rows of one operand B, so a K = 16 step is one MMA of M = 128 stored rows
 // (operand A, in TMEM) and N = 2 QB; the drain adds the two sums of a query.
 // Accumulation runs cover at most 1024 coordinates of one module; after each,
-// acc = fl(acc + fl(s_iu d)) in fp32 registers.
+// acc = fl(acc + s_iu d) (one fused multiply-add) in fp32 registers.
 //
 // Bound: the bf16 tensor rate (two products a coordinate). 250 queries against
 // 16,384 rows of 48 x 1024 bits: 491 us (1.68 PFLOP/s issued, 0.86 of the measured
