@@ -31,6 +31,15 @@ int make_tmap(CUtensorMap* tm, CUtensorMapDataType dt, int rank, const void* bas
 
 }  // namespace eogp
 
+// Allows a kernel all dynamic shared memory a block can have beside its `fixed` bytes
+// of static arrays. The limit belongs to the process: set to each launch's own need, a
+// thread with a smaller module could lower it between another's call here and its
+// launch, which was then refused (3 in 1,000 calls of two threads).
+template <typename... P>
+cudaError_t allow_smem(void (*kernel)(P...), size_t fixed = 0) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(232448 - fixed));
+}
+
 // Launch of a kernel that calls pdl_wait before it touches anything the kernels
 // before it on the stream write or read: its prologue overlaps their end.
 template <typename... P, typename... A>

@@ -1199,7 +1199,7 @@ int chol_qr_pass(const SubLayout& L, char* w, const float* Y32, float* X32, floa
   k_trinv_diag<<<nblk, 32, 0, st>>>(G, L.p4, Li, L.p4, p);
   const int cw = static_cast<size_t>(p) * 8 * sizeof(float) <= 200 * 1024 ? 8 : 4;
   const size_t cols = static_cast<size_t>(p) * cw * sizeof(float);
-  PCA_TRY(cudaFuncSetAttribute(k_trinv_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(cols)));
+  PCA_TRY(allow_smem(k_trinv_cols, 10 * 1024));
   k_trinv_cols<<<dim3(nblk, 32 / cw), 256, cols, st>>>(G, L.p4, Li, L.p4, p, cw);
   PCA_TRY(cudaGetLastError());
   k_split_rows<<<grid_for(static_cast<long long>(p) * L.p8), 256, 0, st>>>(Li, L.p4, p, p, nullptr, Sh, Sl, L.p8);

@@ -558,8 +558,7 @@ template <int MODE, bool TOPK, int BN, bool AT>
 cudaError_t launch_tc_kernel(const CUtensorMap& t0, const CUtensorMap& t1, const ScoreTcArgs& g,
                              int grid, cudaStream_t st) {
   const size_t smem = tc_smem_need<MODE, TOPK, BN, AT>(g.BNq, g.K);
-  cudaError_t e = cudaFuncSetAttribute(k_score_tc<MODE, TOPK, BN, AT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(k_score_tc<MODE, TOPK, BN, AT>);
   if (e != cudaSuccess) return e;
   k_score_tc<MODE, TOPK, BN, AT><<<grid, kThreadsTc, smem, st>>>(t0, t1, g);
   return cudaGetLastError();

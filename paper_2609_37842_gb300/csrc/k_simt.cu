@@ -419,8 +419,7 @@ static int f32_first_rows(int B, int T, int nC, int nR, int num_sms) {
 
 template <int BM, int L>
 static cudaError_t first_launch(const FirstArgs& g, size_t smem, cudaStream_t st) {
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_f32_first<BM, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(k_f32_first<BM, L>);
   if (e != cudaSuccess) return e;
   k_f32_first<BM, L><<<static_cast<unsigned>((g.B + g.G - 1) / g.G), first_threads<BM>(), smem, st>>>(g);
   return cudaGetLastError();

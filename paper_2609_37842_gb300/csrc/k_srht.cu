@@ -108,7 +108,7 @@ cudaError_t launch_srht(const void* z0, const void* z1, bool hilo, int ldz, int 
   const size_t smem = srht_smem_bytes(m);
   const float scale = 1.0f / sqrtf(static_cast<float>(k));
   auto kernel = hilo ? k_srht<true> : k_srht<false>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(kernel, 1024);
   if (e != cudaSuccess) return e;
   if (behind)
     return launch_behind(kernel, B, kThreads, smem, st, z0, z1, ldz, m, p, signs, rows, k, scale, x, ldx, codes, ld_codes,

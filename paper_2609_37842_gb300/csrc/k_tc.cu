@@ -1337,8 +1337,7 @@ static cudaError_t launch_tc_gemm_impl(int M, int N, int K, const void* X0, cons
   g.slab = slab;
   g.status = status;
   const size_t smem = gemm_smem_bytes(cfg.BN, cfg.stages, nA, nW);
-  cudaError_t e = cudaFuncSetAttribute(k_tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(k_tc_gemm);
   if (e != cudaSuccess) return e;
   dim3 grid((N + cfg.BN - 1) / cfg.BN, (M + 127) / 128, splits);
   if (behind) return launch_behind(k_tc_gemm, grid, kThreads, smem, st, tX0, tX1, tW, tW1, g);
@@ -1433,8 +1432,7 @@ static cudaError_t launch_rot(const RotSide* r, int n, int M, int T, const int* 
   p.stages = 2;
   while (p.stages < 8 && rotate_smem_bytes(bn, p.stages + 1) <= 232448) ++p.stages;
   const size_t smem = rotate_smem_bytes(bn, p.stages);
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_tc_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(k_tc_rotate);
   if (e != cudaSuccess) return e;
   k_tc_rotate<<<std::min(p.n_tiles, std::max(1, num_sms)), kThreads, smem, st>>>(tx[0], tw[0], tx[1], tw[1], p);
   return cudaGetLastError();
@@ -1453,8 +1451,7 @@ cudaError_t launch_tc_rotate(const RotSide& r, int M, int T, int num_sms, unsign
   g.stages = 2;
   while (g.stages < 8 && rotate2_smem_bytes(BN, g.stages + 1) <= 232448) ++g.stages;
   const size_t smem = rotate2_smem_bytes(BN, g.stages);
-  cudaError_t e = cudaFuncSetAttribute(k_tc_rotate2, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(k_tc_rotate2);
   if (e != cudaSuccess) return e;
   const int clusters = std::min(g.n_tiles, std::max(1, num_sms / 2));
   k_tc_rotate2<<<2 * clusters, kThreads, smem, st>>>(tX, tWh, g);
@@ -1517,8 +1514,7 @@ cudaError_t launch_tc_contract(const void* St_hi, const void* St_lo, int ldS, co
   g.ldzb = ldzb;
   g.status = status;
   const size_t smem = contract_smem_bytes(stages);
-  cudaError_t e = cudaFuncSetAttribute(k_tc_contract, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(k_tc_contract);
   if (e != cudaSuccess) return e;
   const int grid = std::min(g.n_items, std::max(1, num_sms));
   return launch_behind(k_tc_contract, grid, kThreads, smem, st, tSh, tSl, tAh, tAl, g);
@@ -1578,8 +1574,7 @@ static cudaError_t launch_ekfac2(const void* St_hi, const void* St_lo, int ldS, 
   g.stages = 2;
   while (bytes(g.stages + 1) <= 232448) ++g.stages;
   const size_t smem = bytes(g.stages);
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_tc_ekfac2, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(k_tc_ekfac2);
   if (e != cudaSuccess) return e;
   return launch_behind(k_tc_ekfac2, 2 * std::min(g.n_items, std::max(1, num_sms / 2)), kEk2Threads, smem, st, tSh, tSl,
                        tAh, tAl, g);
@@ -1609,8 +1604,7 @@ static cudaError_t launch_ekfac1(const void* St_hi, const void* St_lo, int ldS, 
   g.part = part;
   g.status = status;
   const size_t smem = ekfac_smem_bytes(stages);
-  cudaError_t e = cudaFuncSetAttribute(k_tc_ekfac, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(k_tc_ekfac);
   if (e != cudaSuccess) return e;
   const int grid = std::min(g.n_items, std::max(1, num_sms));
   return launch_behind(k_tc_ekfac, grid, kThreads, smem, st, tSh, tSl, tAh, tAl, g);
